@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 #include "lbm_nn.h"
@@ -239,15 +240,50 @@ __global__ void __launch_bounds__(128) k_wgrad(const bf16* __restrict__ x, const
             }
 }
 
-// Partial bias gradients of row blocks: part[blockIdx.x][c] = sum of dy over the block's rows.
-__global__ void k_bias_grad(const bf16* __restrict__ dy, long long M, int C, float* __restrict__ part,
-                            long long rows_per_block) {
+// Partial bias gradients of row blocks: part[blockIdx.x][c] = sum of dy over the
+// block's rows.  Bound by reading dy once: a thread keeps V consecutive channels
+// (one 16- or 8-byte load per row) and takes every R-th row of the block, R =
+// kBiasThreads / (C / V) rows in flight, so that a warp reads consecutive
+// memory; the R partial sums of a channel are then added in row order.  (One
+// thread per channel walking 4096 rows kept 16 threads of a block busy on a
+// 16-channel layer: the 15 layers of a training step on 8 x 64^3 voxels took
+// 5.4 ms with their chunk sums, 0.2 ms this way.)
+// Channel groups beyond kBiasThreads go to further blocks along y.
+constexpr int kBiasThreads = 256;
+
+template <int V>
+__global__ void __launch_bounds__(kBiasThreads) k_bias_grad(const bf16* __restrict__ dy, long long M, int C,
+                                                            float* __restrict__ part, long long rows_per_block) {
+    __shared__ float sm[kBiasThreads][V];
+    const int G = C / V;  // channel groups
+    const int g0 = blockIdx.y * kBiasThreads, gn = G - g0 < kBiasThreads ? G - g0 : kBiasThreads;
+    const int R = kBiasThreads / gn;
+    const int r = threadIdx.x / gn, g = threadIdx.x - r * gn;
     const long long r0 = (long long)blockIdx.x * rows_per_block;
     const long long r1 = r0 + rows_per_block < M ? r0 + rows_per_block : M;
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        float s = 0.f;
-        for (long long r = r0; r < r1; r++) s += __bfloat162float(dy[r * C + c]);
-        part[(long long)blockIdx.x * C + c] = s;
+    float s[V];
+#pragma unroll
+    for (int k = 0; k < V; k++) s[k] = 0.f;
+    if (r < R) {
+        const bf16* src = dy + (size_t)(g0 + g) * V;
+#pragma unroll 8
+        for (long long row = r0 + r; row < r1; row += R) {
+            const bf16* p = src + row * C;
+            bf16 h[V];
+            if constexpr (V == 8) *reinterpret_cast<uint4*>(h) = __ldg(reinterpret_cast<const uint4*>(p));
+            else if constexpr (V == 4) *reinterpret_cast<uint2*>(h) = __ldg(reinterpret_cast<const uint2*>(p));
+            else h[0] = p[0];
+#pragma unroll
+            for (int k = 0; k < V; k++) s[k] += __bfloat162float(h[k]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < V; k++) sm[threadIdx.x][k] = s[k];
+    __syncthreads();
+    for (int c = threadIdx.x; c < gn * V; c += kBiasThreads) {
+        float t = 0.f;
+        for (int q = 0; q < R; q++) t += sm[q * gn + c / V][c % V];
+        part[(long long)blockIdx.x * C + (size_t)g0 * V + c] = t;
     }
 }
 
@@ -556,10 +592,22 @@ extern "C" int lbm_nn_conv3d_wgrad(const void* x, const void* dy, int n, int d, 
         if (!rc) rc = sum_chunks(part, grid.y, (long long)K * cout, dw, S(stream));
     }
     if (rc || !dbias) return rc;
-    const long long rpb = 4096, nb = (M + rpb - 1) / rpb;
+    // two blocks per SM, and at least 64 rows each
+    long long rpb = (M + 303) / 304;
+    if (rpb < 64) rpb = 64;
+    const long long nb = (M + rpb - 1) / rpb;
     float* part = chunk_scratch((size_t)nb * cout);  // the weight gradient's sums are already in dw
     if (!part) return fail(LBM_ERR_OOM, "bias-gradient partial sums");
-    k_bias_grad<<<(unsigned)nb, 128, 0, S(stream)>>>(static_cast<const bf16*>(dy), M, cout, part, rpb);
+    auto bias = [&](auto V, auto kern) {
+        const int G = cout / decltype(V)::value;
+        kern<<<dim3((unsigned)nb, (unsigned)((G + kBiasThreads - 1) / kBiasThreads)), kBiasThreads, 0, S(stream)>>>(
+            static_cast<const bf16*>(dy), M, cout, part, rpb);
+    };
+    // the widest load that every row's channels allow (row starts are C values apart)
+    const uintptr_t at = reinterpret_cast<uintptr_t>(dy);
+    if (cout % 8 == 0 && at % 16 == 0) bias(std::integral_constant<int, 8>{}, k_bias_grad<8>);
+    else if (cout % 4 == 0 && at % 8 == 0) bias(std::integral_constant<int, 4>{}, k_bias_grad<4>);
+    else bias(std::integral_constant<int, 1>{}, k_bias_grad<1>);
     rc = check(cudaGetLastError(), "k_bias_grad launch");
     return rc ? rc : sum_chunks(part, nb, cout, dbias, S(stream));
 }

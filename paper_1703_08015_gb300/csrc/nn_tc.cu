@@ -866,18 +866,42 @@ float* chunk_scratch(size_t floats) {
     return g_part_buf;
 }
 
-// dst[e] += sum over c = 0 .. chunks-1 of part[c][e], in that order.
-__global__ void k_sum_chunks(const float* __restrict__ part, long long chunks, long long E, float* __restrict__ dst) {
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (long long)gridDim.x * blockDim.x) {
+// dst[e] += sum over the chunks c of part[c][e], in a fixed order: NC threads
+// share an element (thread j takes chunks j, j + NC, ..), their sums are added
+// in thread order.  A thread's chain of loads over
+// its chunks is what it costs, so few elements (biases: up to 304 chunks of a
+// handful of channels) take more threads each.
+template <int NC>
+__global__ void __launch_bounds__(256) k_sum_chunks(const float* __restrict__ part, long long chunks, long long E,
+                                                    float* __restrict__ dst) {
+    constexpr int NE = 256 / NC;  // elements per block
+    __shared__ float sm[NC][NE];
+    const int i = threadIdx.x % NE, j = threadIdx.x / NE;
+    for (long long e0 = (long long)blockIdx.x * NE; e0 < E; e0 += (long long)gridDim.x * NE) {
+        const long long e = e0 + i;
         float s = 0.f;
-        for (long long c = 0; c < chunks; c++) s += part[c * E + e];
-        dst[e] += s;
+        if (e < E) {
+#pragma unroll 4
+            for (long long c = j; c < chunks; c += NC) s += part[c * E + e];
+        }
+        sm[j][i] = s;
+        __syncthreads();
+        if (j == 0 && e < E) {
+            float t = 0.f;
+#pragma unroll
+            for (int k = 0; k < NC; k++) t += sm[k][i];
+            dst[e] += t;
+        }
+        __syncthreads();
     }
 }
 
 int sum_chunks(const float* part, long long chunks, long long E, float* dst, cudaStream_t s) {
-    const long long blocks = (E + 255) / 256;
-    k_sum_chunks<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(part, chunks, E, dst);
+    const bool few = E < 4096;
+    const long long ne = few ? 8 : 32, blocks = (E + ne - 1) / ne;
+    const unsigned grid = (unsigned)(blocks < 8192 ? blocks : 8192);
+    if (few) k_sum_chunks<32><<<grid, 256, 0, s>>>(part, chunks, E, dst);
+    else k_sum_chunks<8><<<grid, 256, 0, s>>>(part, chunks, E, dst);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_sum_chunks launch");
 }
