@@ -77,10 +77,11 @@ int lbm_nn_weight_flip(const void* wgt, int cin, int cout, void* wt, void* strea
  * as in lbm_nn_conv3d) and, when dbias is not NULL, dbias[co] += sum_p
  * dy[p][co] (FP32 accumulators).  The voxels are split into chunks whose
  * partial sums are stored, then added to dw / dbias in chunk order: the
- * result is the same bits on every call (no atomics).  For 8 <= cin <= 256
- * the sums run on the tcgen05 tensor cores as one GEMM per tap over operands
- * packed channel-major; the packed operands and the partial sums live in
- * library-owned device buffers (grown on demand, kept for the process; calls
+ * result is the same bits on every call (no atomics).  The sums run on the
+ * tcgen05 tensor cores for every shape, reading both operands from
+ * channels-last tiles in shared memory (zero-padded to 8 input and 16 output
+ * channels); the partial sums live in a library-owned device buffer (grown on
+ * demand, kept for the process; calls
  * must not overlap on different streams).  Errors: LBM_ERR_ARG, LBM_ERR_OOM
  * (no room for the partial sums), LBM_ERR_CUDA. */
 int lbm_nn_conv3d_wgrad(const void* x, const void* dy, int n, int d, int h, int w, int cin, int cout,

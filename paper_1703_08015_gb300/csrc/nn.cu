@@ -148,98 +148,6 @@ __global__ void __launch_bounds__(128) k_conv(const bf16* __restrict__ x, int N,
             }
 }
 
-// dW[(tap,ci)][co] = sum_p x[p + off(tap)][ci] dy[p][co]: GEMM with 64 rows of
-// (tap, ci) per block, NF*8 output channels from blockIdx.z * NF*8, split over
-// voxel chunks (blockIdx.y); each block stores its chunk's partial sums to
-// part[blockIdx.y], added to dw in chunk order afterwards.  The gather form,
-// for the shapes the tcgen05 weight gradient does not take (fewer than 8
-// input channels, more than 256).
-template <int NF>
-__global__ void __launch_bounds__(128) k_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dy, int N,
-                                               int D, int H, int W, int Cin, int Cout, int wrap,
-                                               float* __restrict__ dw, long long vox_per_block) {
-    constexpr int BN = NF * 8;
-    __shared__ __align__(16) bf16 As[BM][LD];  // [k row][voxel]
-    __shared__ __align__(16) bf16 Bs[BN][LD];  // [co][voxel]
-    __shared__ int vpos[BK][4];                 // n, z, y, x of the stage's voxels (n < 0: none)
-    const long long M = (long long)N * D * H * W;
-    const int K = 27 * Cin;
-    const int k0 = blockIdx.x * BM;
-    const int n0 = blockIdx.z * BN;
-    const long long v_begin = (long long)blockIdx.y * vox_per_block;
-    const long long v_end = v_begin + vox_per_block < M ? v_begin + vox_per_block : M;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    float acc[NF][4];
-#pragma unroll
-    for (int f = 0; f < NF; f++) acc[f][0] = acc[f][1] = acc[f][2] = acc[f][3] = 0.f;
-    // this thread gathers row kr of every A stage, voxels vq, vq + 2, ...
-    const int kr = tid & 63, vq = tid >> 6;
-    const int kg = k0 + kr;
-    const bool krow = kg < K;
-    const int tap = krow ? kg / Cin : 0, ci = krow ? kg - tap * Cin : 0;
-    const int dz = tap / 9 - 1, dyy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-    const bool wx = wrap & 1, wy = wrap & 2, wz = wrap & 4;
-    const bf16 zero = __float2bfloat16(0.f);
-    for (long long v0 = v_begin; v0 < v_end; v0 += BK) {
-        if (tid < BK) {
-            const long long v = v0 + tid;
-            if (v < v_end) {
-                long long t = v;
-                vpos[tid][3] = (int)(t % W);
-                t /= W;
-                vpos[tid][2] = (int)(t % H);
-                t /= H;
-                vpos[tid][1] = (int)(t % D);
-                vpos[tid][0] = (int)(t / D);
-            } else {
-                vpos[tid][0] = -1;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < BK / 2; j++) {
-            const int vv = vq + 2 * j;
-            bf16 val = zero;
-            const int n = vpos[vv][0];
-            if (krow && n >= 0) {
-                const int zz = nb_coord(vpos[vv][1], dz, D, wz), yy = nb_coord(vpos[vv][2], dyy, H, wy),
-                          xx = nb_coord(vpos[vv][3], dx, W, wx);
-                if ((zz | yy | xx) >= 0) val = x[((((long long)n * D + zz) * H + yy) * W + xx) * Cin + ci];
-            }
-            As[kr][vv] = val;
-        }
-        for (int e = tid; e < BN * BK; e += 128) {
-            const int vv = e / BN, nn = e - vv * BN;
-            const long long v = v0 + vv;
-            Bs[nn][vv] = (v < v_end && n0 + nn < Cout) ? dy[v * Cout + n0 + nn] : zero;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int ks = 0; ks < BK; ks += 16) {
-            const int r = warp * 16 + (lane >> 2), c = ks + (lane & 3) * 2;
-            const unsigned a[4] = {lds32(&As[r][c]), lds32(&As[r + 8][c]), lds32(&As[r][c + 8]),
-                                   lds32(&As[r + 8][c + 8])};
-#pragma unroll
-            for (int f = 0; f < NF; f++) {
-                const int nn = f * 8 + (lane >> 2);
-                const unsigned b[2] = {lds32(&Bs[nn][c]), lds32(&Bs[nn][c + 8])};
-                mma_bf16(acc[f], a, b);
-            }
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int f = 0; f < NF; f++)
-#pragma unroll
-        for (int h2 = 0; h2 < 2; h2++)
-#pragma unroll
-            for (int j = 0; j < 2; j++) {
-                const int row = k0 + warp * 16 + (lane >> 2) + h2 * 8;
-                const int co = n0 + f * 8 + (lane & 3) * 2 + j;
-                if (row < K && co < Cout) dw[(long long)blockIdx.y * K * Cout + (long long)row * Cout + co] = acc[f][h2 * 2 + j];
-            }
-}
-
 // Partial bias gradients of row blocks: part[blockIdx.x][c] = sum of dy over the
 // block's rows.  Bound by reading dy once: a thread keeps V consecutive channels
 // (one 16- or 8-byte load per row) and takes every R-th row of the block, R =
@@ -488,8 +396,8 @@ static int check(cudaError_t e, const char* what) { return e == cudaSuccess ? LB
 using namespace lbm;
 using namespace lbm::nn;
 
-// Output-channel tiling shared by the forward and weight-gradient GEMMs: the
-// channels are split into equal tiles of at most 128, each a multiple of 8.
+// Output-channel tiling of the forward GEMM: the channels are split into equal
+// tiles of at most 128, each a multiple of 8.
 static int pick_nf(int cout, int* n_tiles) {
     const int tiles = (cout + 127) / 128;
     const int per = (cout + tiles - 1) / tiles;
@@ -562,35 +470,10 @@ extern "C" int lbm_nn_conv3d_wgrad(const void* x, const void* dy, int n, int d, 
                                    int wrap, float* dw, float* dbias, void* stream) {
     if (!x || !dy || !dw || n < 1 || d < 1 || h < 1 || w < 1 || cin < 1 || cout < 1 || (wrap & ~7))
         return fail(LBM_ERR_ARG, "lbm_nn_conv3d_wgrad: bad arguments");
-    // the tcgen05 GEMMs over packed operands where the shape allows, else the
-    // gather kernel below; both leave per-chunk partial sums that are added in
-    // chunk order (the result does not depend on the order blocks finish in)
+    // per-chunk partial sums that are added in chunk order (the result does
+    // not depend on the order blocks finish in)
     int rc = wgrad_tc(x, dy, n, d, h, w, cin, cout, wrap, dw, S(stream));
     const long long M = (long long)n * d * h * w;
-    if (rc == 1) {
-        const int K = 27 * cin;
-        const long long vpb = 8192;
-        int nz = 0;
-        const int nf = pick_nf(cout, &nz);
-        const dim3 grid((unsigned)((K + BM - 1) / BM), (unsigned)((M + vpb - 1) / vpb), (unsigned)nz);
-        float* part = chunk_scratch((size_t)grid.y * K * cout);
-        if (!part) return fail(LBM_ERR_OOM, "weight-gradient partial sums");
-        auto go = [&](auto kern) {
-            kern<<<grid, 128, 0, S(stream)>>>(static_cast<const bf16*>(x), static_cast<const bf16*>(dy), n, d, h, w,
-                                              cin, cout, wrap, part, vpb);
-        };
-        switch (nf) {
-            case 1: go(k_wgrad<1>); break;
-            case 2: go(k_wgrad<2>); break;
-            case 4: go(k_wgrad<4>); break;
-            case 6: go(k_wgrad<6>); break;
-            case 8: go(k_wgrad<8>); break;
-            case 12: go(k_wgrad<12>); break;
-            default: go(k_wgrad<16>); break;
-        }
-        rc = check(cudaGetLastError(), "k_wgrad launch");
-        if (!rc) rc = sum_chunks(part, grid.y, (long long)K * cout, dw, S(stream));
-    }
     if (rc || !dbias) return rc;
     // two blocks per SM, and at least 64 rows each
     long long rpb = (M + 303) / 304;

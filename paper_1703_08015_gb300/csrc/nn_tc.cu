@@ -3,7 +3,7 @@
 // the FP32 accumulator in tensor memory (TMEM), one thread issuing the MMAs
 // and an mbarrier reporting their completion.  A plain BF16 GEMM, the 3x3x3
 // convolution (as an implicit GEMM, and reading a shared-memory halo tile)
-// and its weight gradient (one GEMM per tap over packed operands).  See
+// and its weight gradient (reducing over the voxels of such tiles).  See
 // include/lbm_nn.h.
 #include <cuda_bf16.h>
 
@@ -479,225 +479,267 @@ __global__ void __launch_bounds__(128) k_conv_halo(const bf16* __restrict__ x, i
 
 // ---- weight gradient on the tensor cores ------------------------------------
 //
-// dw[tap][ci][co] = sum_p x[p + off(tap)][ci] dy[p][co] as 27 K-major GEMMs
-// over voxels.  x and dy are first packed channel-major over a padded grid
-// (D + 2) x (H + 2) x Wp, Wp >= W + 2 a multiple of 8: padded voxel q holds x
-// at q minus one voxel on each axis (wrapped on periodic axes, zero outside),
-// dy only at interior voxels (zero on the padding).  With flat indices, the
-// voxel p + off(tap) is q + dz Hp Wp + dy Wp + dx; the dz and dy parts are
-// multiples of 8 values (16 bytes), and dx in {-1, 0, 1} is taken from one of
-// three copies of packed x shifted by one value, so every operand row starts
-// 16-byte aligned.  Rows are Lp values long, the data G values in, with zero
-// guards of G values (G > Hp Wp + Wp) before and after.
+// dw[tap][ci][co] = sum_p x[p + off(tap)][ci] dy[p][co]: GEMMs that reduce over
+// voxels, with both operands read by the tensor cores where the channels-last
+// tensors put them.  A stage holds one brick of 8 (x) x 16 (y) x MB (z) voxels:
+// a halo tile of x, 10 x 18 x (MB + 2) cells of 8 channels (16 bytes) laid out
+// [z][channel group][y][x], and the brick of dy laid out [channel
+// group][z][y][x].  8 consecutive cells along x are one core matrix of an
+// MN-major operand (8 voxels of K by 8 channels), so no transposed or shifted
+// copy is made: a tap is a start address.  Planes (z, channel group) are one
+// stride apart, so the groups from z plane m on are the rows (dz, ci) of all
+// three dz taps of output plane m: one MMA of K = 16 (8 x by 2 y voxels) gives
+// the sums of 3 cc (dz, ci) rows by NT output channels for one (dy, dx), into
+// that tap's TMEM columns.  (Rows past 3 cc groups read whatever lies behind;
+// their sums are not used.)  Eight warps copy the stages, one issues the MMAs,
+// two stages in flight; each block keeps its sums over all of its bricks in
+// TMEM and stores them once.
 //
-//   xp[(dx + 1) Cp + ci][G + q] = xpad[ci][q + dx],   dyp[co][G + q] = dypad[co][q]
-//
-// with Cp the input channels rounded up to 16 (the rows past Cin zero).
-constexpr int WG_STAGES = 3;
-constexpr int WG_THREADS = 256;  // two warps per TMEM lane quadrant
+// What bounds it: the tensor cores' reads of the 128 or 64 (dz, ci) rows from
+// shared memory, once per (dy, dx), and the L2 reads of the halo.  With
+// operands packed channel-major in memory (three copies of x) a layer wrote and
+// read 4 to 8 times its tensors: 16 -> 16 channels on 8 x 64^3 voxels 1082 us,
+// now 147; 48 -> 16 2636, now 424; 96 -> 32 on 8 x 32^3 914, now 155; 192 ->
+// 128 on 8 x 48^3 5012, now 3978; and 2 -> 16 on 8 x 64^3 (gathered for
+// mma.sync, 1275) 152.
+constexpr int WG_X = 10, WG_Y = 18;       // halo tile extent in x and y (z: MB + 2)
+constexpr int WG_FILL = 256;              // copying threads (eight warps)
+constexpr int WG_THREADS = WG_FILL + 32;  // and the warp that issues the MMAs
 
-// One block per padded row (sample, z, y): the row's values go through shared
-// memory ([voxel][channel], an odd number of 32-bit words per voxel so that
-// the channel-major reads do not collide in banks) and out channel-major,
-// one warp per output row.  x has Cin channels, written as Cp >= Cin rows per
-// copy (the rows past Cin zero).
-__host__ __device__ constexpr int wg_pack_stride(int c) { return 2 * (((c + 1) / 2) | 1); }
+// Shape of one launch, shared by the host and the kernel.
+struct WgShape {
+    int cc;       // input channels per block: 8, 16 or 32
+    int ncg;      // cc / 8
+    int nt;       // output channels per block: 16, 32, 48 or 64
+    int mb;       // z planes of a brick
+    int tg;       // tap groups: 1 (all nine (dy, dx)) or 2 (five and four)
+    int plane;    // cells from one (z, channel group) plane of the x tile to the next
+    int gstride;  // cells from one channel group of the dy brick to the next
+    uint32_t a_bytes, stage_bytes, smem, ncols;
+};
 
-__global__ void k_wgrad_pack(const bf16* __restrict__ x, const bf16* __restrict__ dy, int D, int H, int W, int Cin,
-                             int Cp, int Cout, int wrap, int Hp, int Wp, long long G, long long Lp, bf16* __restrict__ xp,
-                             bf16* __restrict__ dyp) {
-    extern __shared__ __align__(16) unsigned char pack_smem[];
-    const int sx = wg_pack_stride(Cp), sd = wg_pack_stride(Cout);
-    bf16* xs = reinterpret_cast<bf16*>(pack_smem);
-    bf16* ds = xs + (size_t)Wp * sx;
-    const long long r = blockIdx.x;  // padded row
-    const int Dp = D + 2;
-    const int yp = (int)(r % Hp), zp = (int)((r / Hp) % Dp);
-    const long long n = r / ((long long)Hp * Dp);
-    const bool wx = wrap & 1, wy = wrap & 2, wz = wrap & 4;
-    const int zs = halo_nb(zp - 1, D, wz), ys = halo_nb(yp - 1, H, wy);
-    const bool interior = zp >= 1 && zp <= D && yp >= 1 && yp <= H;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const bf16 z0 = __float2bfloat16(0.f);
-    // one 16-byte load per 8 channels where the channel count and alignment
-    // allow (every load of the block in flight at once), else one per value
-    auto load_row = [&](const bf16* base, int C, int Cw, bf16* dst, int sdst, bool vec, auto src_ok) {
-        if (vec) {
-            const int g8 = Cw / 8;
-            for (int e = threadIdx.x; e < Wp * g8; e += blockDim.x) {
-                const int v = e / g8, c8 = e - v * g8;
-                uint4 val = make_uint4(0, 0, 0, 0);
-                const long long off = src_ok(v);
-                if (off >= 0 && c8 * 8 < C) val = *reinterpret_cast<const uint4*>(base + off * C + c8 * 8);
-                const bf16* h8 = reinterpret_cast<const bf16*>(&val);
+// The plane and group strides put the 16-byte cells that a warp stores
+// together (channel groups fastest) into different banks: 8 / ncg mod 8 cells.
+__host__ __device__ inline WgShape wg_shape(int cin, int cout) {
+    WgShape s;
+    s.cc = cin <= 8 ? 8 : ((cin <= 16 || (cin % 32 && cin % 32 <= 16)) ? 16 : 32);
+    s.ncg = s.cc / 8;
+    s.nt = cout >= 64 ? 64 : (cout + 15) / 16 * 16;
+    s.mb = s.nt > 32 ? 2 : 4;
+    s.tg = 9 * s.nt > 512 ? 2 : 1;
+    const int base = WG_X * WG_Y;  // 180 = 4 mod 8
+    s.plane = s.ncg == 4 ? base + 6 : base;
+    s.gstride = s.mb * 128 + (s.nt / 8 == 2 ? 4 : (s.nt / 8 == 4 ? 2 : 1));
+    s.a_bytes = (uint32_t)((s.mb + 2) * s.ncg * s.plane) * 16;
+    const uint32_t g_bytes = (uint32_t)(s.nt / 8 * s.gstride) * 16;
+    s.stage_bytes = (s.a_bytes + g_bytes + 127) / 128 * 128;
+    // the unused rows of the last plane's MMAs reach past the x tile
+    const int rows8 = 3 * s.ncg > 8 ? 16 : 8;
+    const int over = (s.mb - 1) * s.ncg + rows8 - (s.mb + 2) * s.ncg;
+    const uint32_t over_bytes = over > 0 ? (uint32_t)(over * s.plane) * 16 : 0;
+    s.smem = 2 * s.stage_bytes + (over_bytes > g_bytes ? over_bytes - g_bytes : 0);
+    const int cols = (s.tg == 2 ? 5 : 9) * s.nt;
+    s.ncols = 32;
+    while ((int)s.ncols < cols) s.ncols <<= 1;
+    return s;
+}
+
+// The MMAs of one stage for the (dy, dx) taps T0 .. T0 + NTAP - 1: nz planes,
+// ny2 pairs of lines.  The whole warp runs the loop, one lane issues.
+template <int T0, int NTAP>
+__device__ __forceinline__ void wg_issue(uint32_t tmem, uint64_t a0, uint64_t g0, int nz, int ny2, uint32_t aplane,
+                                         int nt, uint32_t idesc, bool first, bool leader) {
+    for (int m = 0; m < nz; m++) {
+        for (int y2 = 0; y2 < ny2; y2++) {
+            const uint64_t a = a0 + (uint64_t)(m * aplane + (uint32_t)y2 * (2 * WG_X));
+            const uint64_t g = g0 + (uint64_t)(m * 128 + y2 * 16);
+            const bool acc = !(first && m == 0 && y2 == 0);
 #pragma unroll
-                for (int k = 0; k < 8; k++) dst[(size_t)v * sdst + c8 * 8 + k] = h8[k];
-            }
-        } else {
-            for (int e = threadIdx.x; e < Wp * Cw; e += blockDim.x) {
-                const int v = e / Cw, c = e - v * Cw;
-                const long long off = src_ok(v);
-                dst[(size_t)v * sdst + c] = (off >= 0 && c < C) ? base[off * C + c] : z0;
-            }
-        }
-    };
-    const long long xrow = ((n * D + zs) * H + ys) * W;  // voxel index of (zs, ys, 0)
-    load_row(x, Cin, Cp, xs, sx, Cin % 8 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0, [&](int v) -> long long {
-        const int xs_ = halo_nb(v - 1, W, wx);
-        return (zs | ys | xs_) >= 0 ? xrow + xs_ : -1;
-    });
-    const long long drow = ((n * D + zp - 1) * H + yp - 1) * W;
-    load_row(dy, Cout, Cout, ds, sd, Cout % 8 == 0 && (reinterpret_cast<uintptr_t>(dy) & 15) == 0,
-             [&](int v) -> long long { return interior && v >= 1 && v <= W ? drow + v - 1 : -1; });
-    __syncthreads();
-    // two values per 32-bit store (rows start at even offsets: G, Lp, Wp even)
-    const long long row0 = G + r * Wp;
-    const int wh = Wp / 2;
-    for (int rc = warp; rc < 3 * Cp; rc += nw) {  // rc = (dx + 1) Cp + ci
-        const int sh = rc / Cp - 1, ci = rc - (sh + 1) * Cp;
-        uint32_t* dst = reinterpret_cast<uint32_t*>(xp + (size_t)rc * Lp + row0);
-        for (int vp = lane; vp < wh; vp += 32) {
-            const int s0 = 2 * vp + sh, s1 = s0 + 1;
-            __nv_bfloat162 pr;
-            pr.x = (s0 >= 0 && s0 < Wp) ? xs[(size_t)s0 * sx + ci] : z0;
-            pr.y = (s1 >= 0 && s1 < Wp) ? xs[(size_t)s1 * sx + ci] : z0;
-            dst[vp] = *reinterpret_cast<const uint32_t*>(&pr);
-        }
-    }
-    for (int co = warp; co < Cout; co += nw) {
-        uint32_t* dst = reinterpret_cast<uint32_t*>(dyp + (size_t)co * Lp + row0);
-        for (int vp = lane; vp < wh; vp += 32) {
-            __nv_bfloat162 pr;
-            pr.x = ds[(size_t)(2 * vp) * sd + co];
-            pr.y = ds[(size_t)(2 * vp + 1) * sd + co];
-            dst[vp] = *reinterpret_cast<const uint32_t*>(&pr);
+            for (int t = T0; t < T0 + NTAP; t++)
+                tc::mma_bf16_if(tmem + (uint32_t)((t - T0) * nt), a + (uint64_t)((t / 3) * WG_X + t % 3), g, idesc, acc,
+                                leader);
         }
     }
 }
 
-// One block: 128 output channels (from blockIdx.z * 128; rows past Cout are
-// zero) x the Cp columns of each of TG taps (from blockIdx.y * TG), summed
-// over the voxel steps [blockIdx.x * spc, ..) of 64 values.  Each stage holds
-// the dy tile (A, 128 x 64) and the TG shifted x tiles (B, Cp x 64 each),
-// K-major; the x tiles lie back to back with one 8-row stride, so one MMA
-// covers up to 256 / Cp taps, one TMEM accumulator column range per tap.  The
-// two warps of each TMEM lane quadrant split the fills (taps of one parity
-// each) and the epilogue's column chunks; the three-stage ring and the bounded
-// waits are those of tc_pipeline.  The block's sums go to the partial sums of
-// its voxel chunk, part[blockIdx.x][tap][ci][co] (plain stores, NaN when a
-// wait ran out); k_sum_chunks adds the chunks to dw in a fixed order, so the
-// gradient does not depend on the order in which blocks finish.
-__global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict__ xp, const bf16* __restrict__ dyp, int Cin,
-                                                  int Cp, int Cout, int Hp, int Wp, long long G, long long Lp,
-                                                  long long nsteps, long long spc, int TG, float* __restrict__ part) {
+// Grid: x = voxel chunks (bricks blockIdx.x, + gridDim.x, ..), y = input-channel
+// chunks x tap groups, z = output-channel tiles.  part[blockIdx.x][tap][ci][co]
+// takes the block's sums (NaN when a wait ran out); k_sum_chunks adds the
+// chunks to dw in a fixed order, so the gradient does not depend on the order
+// in which blocks finish.
+template <bool VX, bool VG>
+__global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict__ x, const bf16* __restrict__ dy, int N,
+                                                         int D, int H, int W, int Cin, int Cout, int wrap, WgShape sh,
+                                                         float* __restrict__ part) {
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ uint64_t mbar[WG_STAGES];
+    __shared__ uint64_t full[2], empty[2], done;
     __shared__ uint32_t tmem_slot;
+    __shared__ int failed;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int t0 = blockIdx.y * TG, ntap = 27 - t0 < TG ? 27 - t0 : TG;
-    const int m0 = blockIdx.z * TC_M;
-    const long long s0 = (long long)blockIdx.x * spc, s1 = s0 + spc < nsteps ? s0 + spc : nsteps;
-    const int nk = (int)(s1 - s0);
-    const uint32_t a_bytes = TC_M * TC_BK * 2, b_bytes = (uint32_t)Cp * TC_BK * 2;
-    const uint32_t stage_bytes = a_bytes + (uint32_t)TG * b_bytes;
-    uint32_t ncols = 32;
-    while (ncols < (uint32_t)(TG * Cp)) ncols <<= 1;
-    if (warp == 0) tc::tmem_alloc(&tmem_slot, ncols);
-    if (tid == 0)
-        for (int s = 0; s < WG_STAGES; s++) tc::mbar_init(&mbar[s], 1);
+    const int c0 = ((int)blockIdx.y / sh.tg) * sh.cc, tgi = (int)blockIdx.y % sh.tg;
+    const int n0 = blockIdx.z * sh.nt;
+    const int BX = (W + 7) / 8, BY = (H + 15) / 16, BZ = (D + sh.mb - 1) / sh.mb;
+    const long long tiles = (long long)N * BZ * BY * BX;
+    const bool wx = wrap & 1, wy = wrap & 2, wz = wrap & 4;
+    if (warp == 0) tc::tmem_alloc(&tmem_slot, sh.ncols);
+    if (tid == 0) {
+        for (int s = 0; s < 2; s++) {
+            tc::mbar_init(&full[s], WG_FILL / 32);
+            tc::mbar_init(&empty[s], 1);
+        }
+        tc::mbar_init(&done, 1);
+        failed = 0;
+    }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = tmem_slot;
-    const int tpm = 256 / Cp;  // taps per MMA
+    const int rows = 3 * sh.ncg > 8 ? 128 : 64;  // (dz, ci) rows of an MMA
     bool ok = true;
-    // this thread's 16-byte segment g of rows r0, r0 + 16, .. (of the taps of
-    // its parity): fixed bases, per tap one offset (the copy for dx and the
-    // dz, dy shift)
-    const int th = tid & 127, par = tid >> 7;
-    const int g = th & 7, r0 = th >> 3;
-    const uint32_t so = tc::tile_off(r0, g, TC_KGAP, TC_RGAP), so16 = 2 * TC_RGAP;  // + 16 rows
-    const bf16* xb = xp + (size_t)r0 * Lp + g * 8;
-    const bf16* ab = dyp + g * 8;
-    const long long copy = (long long)Cp * Lp, plane = (long long)Hp * Wp;
-    auto fill = [&](unsigned char* st, int kc) {
-        const long long q = G + (s0 + kc) * TC_BK;
-#pragma unroll
-        for (int j = par; j < TC_M / 16; j += 2) {
-            const int co = m0 + r0 + 16 * j;
-            tc::cp_async16(st + so + j * so16, ab + (size_t)(co < Cout ? co : 0) * Lp + q, co < Cout);
-        }
-        unsigned char* sb = st + a_bytes + so + par * b_bytes;
-#pragma unroll 1
-        for (int t = par; t < ntap; t += 2, sb += 2 * b_bytes) {
-            const int tap = t0 + t;
-            const bf16* src = xb + (tap % 3) * copy + (tap / 9 - 1) * plane + (long long)((tap / 3) % 3 - 1) * Wp + q;
-            for (int ci = r0, k = 0; ci < Cp; ci += 16, k++)
-                tc::cp_async16(sb + k * so16, src + (size_t)(ci - r0) * Lp, true);
-        }
-    };
-    for (int p = 0; p < WG_STAGES - 1; p++) {
-        if (p < nk) fill(smem + p * stage_bytes, p);
-        tc::cp_async_commit();
-    }
-    for (int kc = 0; kc < nk; kc++) {
-        const int s = kc % WG_STAGES;
-        unsigned char* st = smem + s * stage_bytes;
-        tc::cp_async_wait<WG_STAGES - 2>();
-        tc::fence_smem_to_async();
-        __syncthreads();
-        if (tid == 0) {
-            tc::fence_after_sync();
-            const uint32_t a0 = tc::smem_u32(st);
-            // the taps' x tiles follow each other with the same 8-row stride:
-            // one MMA covers up to 256 / Cp taps (N = their Cp columns each)
-            for (int t = 0; t < ntap; t += tpm) {
-                const int nn = (ntap - t < tpm ? ntap - t : tpm) * Cp;
-                const uint32_t id = tc::idesc_bf16_f32(TC_M, nn);
-                const uint32_t b0 = a0 + a_bytes + (uint32_t)t * b_bytes;
-#pragma unroll
-                for (int j = 0; j < TC_BK / 16; j++)
-                    tc::mma_bf16(tmem + (uint32_t)(t * Cp), tc::smem_desc(a0 + 2 * j * TC_KGAP, TC_KGAP, TC_RGAP),
-                                 tc::smem_desc(b0 + 2 * j * TC_KGAP, TC_KGAP, TC_RGAP), id, kc > 0 || j > 0);
+    if (warp == 0) {
+        const bool leader = tc::elect_one();
+        const uint32_t idesc = tc::idesc_bf16_f32(rows, sh.nt) | tc::IDESC_MN_MAJOR;
+        int it = 0;
+        for (long long t = blockIdx.x; t < tiles; t += gridDim.x, it++) {
+            const int s = it & 1;
+            if (!tc::mbar_wait(&full[s], (it >> 1) & 1, TC_WAIT)) {
+                ok = false;
+                break;
             }
-            tc::mma_commit(&mbar[s]);
+            tc::fence_after_sync();
+            const long long q = t / BX / BY;
+            const int y0 = (int)(t / BX % BY) * 16, z0 = (int)(q % BZ) * sh.mb;
+            const int nz = D - z0 < sh.mb ? D - z0 : sh.mb, ny2 = H - y0 < 16 ? (H - y0 + 1) / 2 : 8;
+            const uint32_t st = tc::smem_u32(smem + s * sh.stage_bytes);
+            const uint64_t a0 = tc::smem_desc(st, WG_X * 16, (uint32_t)sh.plane * 16);
+            const uint64_t g0 = tc::smem_desc(st + sh.a_bytes, 128, (uint32_t)sh.gstride * 16);
+            const uint32_t ap = (uint32_t)(sh.ncg * sh.plane);
+            if (sh.tg == 1)
+                wg_issue<0, 9>(tmem, a0, g0, nz, ny2, ap, sh.nt, idesc, it == 0, leader);
+            else if (tgi == 0)
+                wg_issue<0, 5>(tmem, a0, g0, nz, ny2, ap, sh.nt, idesc, it == 0, leader);
+            else
+                wg_issue<5, 4>(tmem, a0, g0, nz, ny2, ap, sh.nt, idesc, it == 0, leader);
+            if (leader) tc::mma_commit(&empty[s]);
+            __syncwarp();
         }
-        const int nxt = kc + WG_STAGES - 1;
-        if (nxt < nk) {
-            const int r = nxt % WG_STAGES;
-            if (kc >= 1) ok &= tc::mbar_wait(&mbar[r], ((kc - 1) / WG_STAGES) & 1, TC_WAIT);
-            fill(smem + r * stage_bytes, nxt);
+        if (leader) tc::mma_commit(&done);
+        __syncwarp();
+    } else {
+        const int ft = tid - 32;
+        const int acells = (sh.mb + 2) * WG_X * WG_Y * sh.ncg;
+        const int ashift = sh.ncg == 4 ? 2 : sh.ncg - 1;  // log2 ncg
+        const int gcg = sh.nt / 8, gcells = sh.mb * 128 * gcg;
+        int it = 0;
+        for (long long t = blockIdx.x; t < tiles; t += gridDim.x, it++) {
+            const int s = it & 1;
+            if (it >= 2 && !tc::mbar_wait(&empty[s], ((it >> 1) - 1) & 1, TC_WAIT)) {
+                ok = false;
+                break;
+            }
+            unsigned char* sa = smem + s * sh.stage_bytes;
+            unsigned char* sg = sa + sh.a_bytes;
+            long long q = t;
+            const int x0 = (int)(q % BX) * 8;
+            q /= BX;
+            const int y0 = (int)(q % BY) * 16;
+            q /= BY;
+            const int z0 = (int)(q % BZ) * sh.mb, n = (int)(q / BZ);
+            // the halo tile of x (zero outside the box, wrapped on periodic axes), channel groups fastest
+#pragma unroll 4
+            for (int e = ft; e < acells; e += WG_FILL) {
+                const int cg = e & (sh.ncg - 1), cell = e >> ashift;
+                const int hx = cell % WG_X, hy = (cell / WG_X) % WG_Y, hz = cell / (WG_X * WG_Y);
+                const int zz = halo_nb(z0 + hz - 1, D, wz), yy = halo_nb(y0 + hy - 1, H, wy),
+                          xx = halo_nb(x0 + hx - 1, W, wx);
+                const int ci = c0 + cg * 8;
+                const bool in = (zz | yy | xx) >= 0;
+                unsigned char* dst = sa + (size_t)((hz * sh.ncg + cg) * sh.plane + hy * WG_X + hx) * 16;
+                const bf16* src = x + ((((long long)n * D + zz) * H + yy) * W + xx) * Cin + ci;
+                if constexpr (VX) {
+                    const bool get = in && ci < Cin;
+                    tc::cp_async16(dst, get ? src : x, get);
+                } else {
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (in) v = tc::load8(src, Cin - ci);
+                    *reinterpret_cast<uint4*>(dst) = v;
+                }
+            }
+            // the brick of dy, zero outside the box and past Cout
+#pragma unroll 4
+            for (int e = ft; e < gcells; e += WG_FILL) {
+                const int cell = e / gcg, cg = e - cell * gcg;
+                const int xx = x0 + (cell & 7), yy = y0 + ((cell >> 3) & 15), zz = z0 + (cell >> 7);
+                const int co = n0 + cg * 8;
+                const bool in = xx < W && yy < H && zz < D;
+                unsigned char* dst = sg + (size_t)(cg * sh.gstride + cell) * 16;
+                const bf16* src = dy + ((((long long)n * D + zz) * H + yy) * W + xx) * Cout + co;
+                if constexpr (VG) {
+                    const bool get = in && co < Cout;
+                    tc::cp_async16(dst, get ? src : dy, get);
+                } else {
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (in) v = tc::load8(src, Cout - co);
+                    *reinterpret_cast<uint4*>(dst) = v;
+                }
+            }
+            tc::cp_async_commit();
+            if (it > 0) {  // the stage before this one has landed
+                tc::cp_async_wait<1>();
+                tc::fence_smem_to_async();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&full[s ^ 1]);
+            }
         }
-        tc::cp_async_commit();
+        tc::cp_async_wait<0>();
+        tc::fence_smem_to_async();
+        __syncwarp();
+        if (lane == 0 && it > 0) tc::mbar_arrive(&full[(it - 1) & 1]);
     }
-    if (nk > 0) {
-        const int last = nk - 1;
-        bool done = tc::mbar_wait(&mbar[last % WG_STAGES], (last / WG_STAGES) & 1, TC_WAIT);
-        if (!done) done = tc::mbar_wait(&mbar[last % WG_STAGES], (last / WG_STAGES) & 1, TC_WAIT);
-        ok &= done;
+    bool fin = tc::mbar_wait(&done, 0, TC_WAIT);
+    if (!fin) fin = tc::mbar_wait(&done, 0, TC_WAIT);
+    ok &= fin;
+    if (!ok && lane == 0) {
+        atomicAdd(&g_tc_timeouts, 1u);
+        failed = 1;
     }
-    tc::cp_async_wait<0>();
-    if (!ok && lane == 0) atomicAdd(&g_tc_timeouts, 1u);
+    __syncthreads();
+    const bool good = failed == 0;
     tc::fence_after_sync();
-    // warps w and w + 4 read the same TMEM lanes (32 (w % 4) ..), alternate chunks
-    const int quad = warp & 3;
-    const int co = m0 + quad * 32 + lane;
-    if (nk > 0)
-        for (int c0 = 16 * par; c0 < ntap * Cp; c0 += 32) {
+    if (warp > 0) {
+        // row r of the accumulator lies in TMEM lane r (128 rows) or 32 (r / 16) + r % 16 (64 rows); the
+        // two copying warps of a lane quadrant alternate between chunks of 16 columns
+        const int quad = warp & 3, half = (warp - 1) >> 2;
+        const int r = rows == 128 ? quad * 32 + lane : (lane < 16 ? quad * 16 + lane : 128);
+        const int dz = r / sh.cc, ci = c0 + r % sh.cc;
+        const int t0 = tgi ? 5 : 0, ntap = sh.tg == 1 ? 9 : (tgi ? 4 : 5);
+        const bool mine = r < 3 * sh.cc && ci < Cin;
+        for (int col = half * 16; col < ntap * sh.nt; col += 32) {
             float v[16];
-            tc::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0, v);
-            if (co >= Cout) continue;
-            const int t = c0 / Cp, ci0 = c0 - t * Cp;  // Cp % 16 == 0: one tap per 16 columns
-            float* dst = part + (size_t)blockIdx.x * 27 * Cin * Cout + ((size_t)(t0 + t) * Cin + ci0) * Cout + co;
+            tc::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)col, v);
+            const int t = col / sh.nt, co0 = n0 + col - t * sh.nt;
+            if (!mine || co0 >= Cout) continue;
+            float* dst = part + (((size_t)blockIdx.x * 27 + dz * 9 + t0 + t) * Cin + ci) * Cout + co0;
+            if (Cout % 4 == 0) {
 #pragma unroll
-            for (int k = 0; k < 16; k++)
-                if (ci0 + k < Cin) dst[(size_t)k * Cout] = ok ? v[k] : __int_as_float(0x7fc00000);
+                for (int k = 0; k < 16; k += 4)
+                    if (co0 + k < Cout)
+                        *reinterpret_cast<float4*>(dst + k) =
+                            good ? make_float4(v[k], v[k + 1], v[k + 2], v[k + 3])
+                                 : make_float4(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000),
+                                               __int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
+            } else {
+#pragma unroll
+                for (int k = 0; k < 16; k++)
+                    if (co0 + k < Cout) dst[k] = good ? v[k] : __int_as_float(0x7fc00000);
+            }
         }
+    }
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, ncols);
+        tc::tmem_dealloc(tmem, sh.ncols);
     }
 }
 
@@ -841,13 +883,9 @@ int conv3d_halo(const void* x, int n, int d, int h, int w, int cin, const void* 
 
 namespace lbm {
 namespace nn {
-// Packed operands of the tensor-core weight gradient: one buffer kept for the
-// process and grown on demand (calls on one stream reuse it in order).
-static unsigned char* g_wg_buf = nullptr;
-static size_t g_wg_bytes = 0;
-// Per-chunk partial sums of the weight gradients (k_wgrad_tc, k_wgrad,
+// Per-chunk partial sums of the weight and bias gradients (k_wgrad_tc,
 // k_bias_grad), summed in chunk order by k_sum_chunks: kept for the process
-// and grown on demand, like the packed operands.
+// and grown on demand (calls on one stream reuse it in order).
 static float* g_part_buf = nullptr;
 static size_t g_part_floats = 0;
 
@@ -906,66 +944,35 @@ int sum_chunks(const float* part, long long chunks, long long E, float* dst, cud
     return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_sum_chunks launch");
 }
 
-// dw += the weight gradient on the tensor cores (input channels padded to a
-// multiple of 16, 8 <= cin <= 256: below 8 the padding would multiply the
-// work); returns 1, launching nothing, for other shapes or when the packed
-// operands do not fit.
+// dw += the weight gradient: any channel counts and alignment (16-byte copies
+// where a tensor's channels and address allow, else value by value).
 int wgrad_tc(const void* x, const void* dy, int n, int d, int h, int w, int cin, int cout, int wrap, float* dw,
              cudaStream_t s) {
-    const int cp = (cin + 15) / 16 * 16;
-    if (cin < 8 || cp > 256) return 1;
-    const int Dp = d + 2, Hp = h + 2, Wp = (w + 2 + 7) / 8 * 8;
-    const long long plane = (long long)Hp * Wp;
-    const long long G = (plane + Wp + 8 + 63) / 64 * 64;
-    const long long L = (long long)n * Dp * plane;
-    const long long nsteps = (L + TC_BK - 1) / TC_BK;
-    const long long Lp = 2 * G + nsteps * TC_BK;
-    const size_t rows = 3 * (size_t)cp + (size_t)cout;
-    const size_t bytes = rows * (size_t)Lp * 2;
-    const uint32_t pack_smem = (uint32_t)Wp * (uint32_t)(wg_pack_stride(cp) + wg_pack_stride(cout)) * 2;
-    if (pack_smem > 200u * 1024u || (long long)n * Dp * Hp > 0x7fffffff) return 1;
-    if (bytes > g_wg_bytes) {
-        if (g_wg_buf) cudaFree(g_wg_buf);
-        g_wg_buf = nullptr;
-        g_wg_bytes = 0;
-        if (cudaMalloc(&g_wg_buf, bytes) != cudaSuccess) {
-            (void)cudaGetLastError();
-            g_wg_buf = nullptr;
-            return 1;  // no room: the gather kernel needs none
-        }
-        g_wg_bytes = bytes;
-    }
-    bf16* xpk = reinterpret_cast<bf16*>(g_wg_buf);
-    bf16* dypk = xpk + (size_t)3 * cp * Lp;
-    cudaError_t e = cudaMemset2DAsync(g_wg_buf, (size_t)Lp * 2, 0, (size_t)G * 2, rows, s);
-    if (e == cudaSuccess)
-        e = cudaMemset2DAsync(g_wg_buf + (size_t)(G + L) * 2, (size_t)Lp * 2, 0, (size_t)(Lp - G - L) * 2, rows, s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemset2DAsync (weight-gradient guards)");
-    int rc = tc_launch_ok((const void*)k_wgrad_pack, pack_smem, "cudaFuncSetAttribute(k_wgrad_pack)");
-    if (rc) return rc;
-    k_wgrad_pack<<<(unsigned)(n * (long long)Dp * Hp), 256, pack_smem, s>>>(
-        static_cast<const bf16*>(x), static_cast<const bf16*>(dy), d, h, w, cin, cp, cout, wrap, Hp, Wp, G, Lp, xpk, dypk);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "k_wgrad_pack launch");
-    // taps per block: the stage (dy tile + TG x tiles) within 72 KB, TG Cin <= 448 TMEM columns
-    const int TG = 448 / cp < 27 ? 448 / cp : 27;
-    const int groups = (27 + TG - 1) / TG, mt = (cout + TC_M - 1) / TC_M;
-    long long chunks = sm_count() / (groups * mt);
+    const WgShape sh = wg_shape(cin, cout);
+    const long long tiles = (long long)n * ((d + sh.mb - 1) / sh.mb) * ((h + 15) / 16) * ((w + 7) / 8);
+    const long long groups = (long long)((cin + sh.cc - 1) / sh.cc) * sh.tg, mt = (cout + sh.nt - 1) / sh.nt;
+    if (groups > 65535 || mt > 65535)
+        return fail(LBM_ERR_ARG, "weight gradient: %d x %d channels exceed the grid", cin, cout);
+    // one resident block per SM, two where shared memory and TMEM hold them; each block's sums are one partial sum
+    const int per_sm = 2 * (sh.smem + 1024) <= (228u << 10) && 2 * sh.ncols <= 512 ? 2 : 1;
+    long long chunks = (long long)per_sm * sm_count() / (groups * mt);
     if (chunks < 1) chunks = 1;
-    if (chunks > nsteps) chunks = nsteps;
-    const long long spc = (nsteps + chunks - 1) / chunks;
-    chunks = (nsteps + spc - 1) / spc;
-    const uint32_t smem = WG_STAGES * (uint32_t)(TC_M * TC_BK * 2 + TG * cp * TC_BK * 2);
-    rc = tc_launch_ok((const void*)k_wgrad_tc, smem, "cudaFuncSetAttribute(k_wgrad_tc)");
-    if (rc) return rc;
+    if (chunks > tiles) chunks = tiles;
     const long long E = 27LL * cin * cout;
     float* part = chunk_scratch((size_t)(chunks * E));
     if (!part) return fail(LBM_ERR_OOM, "weight-gradient partial sums: %lld floats", chunks * E);
-    k_wgrad_tc<<<dim3((unsigned)chunks, (unsigned)groups, (unsigned)mt), WG_THREADS, smem, s>>>(xpk, dypk, cin, cp, cout, Hp, Wp,
-                                                                                       G, Lp, nsteps, spc, TG, part);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "k_wgrad_tc launch");
-    return sum_chunks(part, chunks, E, dw, s);
+    auto go = [&](auto kern) -> int {
+        int rc = tc_launch_ok((const void*)kern, sh.smem, "cudaFuncSetAttribute(k_wgrad_tc)");
+        if (rc) return rc;
+        kern<<<dim3((unsigned)chunks, (unsigned)groups, (unsigned)mt), WG_THREADS, sh.smem, s>>>(
+            static_cast<const bf16*>(x), static_cast<const bf16*>(dy), n, d, h, w, cin, cout, wrap, sh, part);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_wgrad_tc launch");
+    };
+    const bool vx = cin % 8 == 0 && (uintptr_t)x % 16 == 0, vg = cout % 8 == 0 && (uintptr_t)dy % 16 == 0;
+    const int rc = vx ? (vg ? go(k_wgrad_tc<true, true>) : go(k_wgrad_tc<true, false>))
+                      : (vg ? go(k_wgrad_tc<false, true>) : go(k_wgrad_tc<false, false>));
+    return rc ? rc : sum_chunks(part, chunks, E, dw, s);
 }
 }  // namespace nn
 }  // namespace lbm

@@ -10,6 +10,8 @@
 // a device counter and the kernel still frees its TMEM before it returns.
 #pragma once
 
+#include <cuda_bf16.h>
+
 #include <cstdint>
 
 namespace lbm {
@@ -57,6 +59,30 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
         : "memory");
 }
 
+// Instruction-descriptor bits of MN-major A and B (bits 15, 16 = 1): a core
+// matrix is 8 rows of K by 16 bytes of 8 consecutive M or N values; without
+// swizzle the leading byte offset then runs between core matrices adjacent
+// along K and the stride byte offset between those adjacent along M or N.
+constexpr uint32_t IDESC_MN_MAJOR = (1u << 15) | (1u << 16);
+
+// One lane of a converged warp (the same one on every call).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+    return p != 0;
+}
+
+// mma_bf16 executed by a whole warp, issued where `issue` is set (one lane):
+// the descriptors stay uniform over the warp.
+__device__ __forceinline__ void mma_bf16_if(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                            bool accumulate, bool issue) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate), "r"((uint32_t)issue)
+        : "memory");
+}
+
 // The mbarrier receives one arrival once every MMA this thread issued before
 // has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* mbar) {
@@ -68,6 +94,10 @@ __device__ __forceinline__ void mma_commit(uint64_t* mbar) {
 __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
 
 // Wait until the phase of parity `parity` has completed; false after `limit`
@@ -119,6 +149,16 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int PENDING>
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+
+// Up to eight consecutive BF16 values, zero past the first `count`, for tensors whose channels allow no
+// 16-byte load.
+__device__ __forceinline__ uint4 load8(const __nv_bfloat16* p, int count) {
+    unsigned short h[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) h[k] = k < count ? __ldg(reinterpret_cast<const unsigned short*>(p) + k) : 0;
+    return make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
+                      h[6] | (uint32_t)h[7] << 16);
 }
 
 // Byte offset of the 16-byte row segment (row r, K group g) of a K-major tile

@@ -417,3 +417,40 @@ def test_training_is_deterministic(nn):
     for a, b in zip(*states):
         assert np.array_equal(a, b)
     assert nn.lbm_nn_tc_timeouts() == 0
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("case", [
+    # n, d, h, w, cin, cout, wrap: one voxel on periodic axes, a brick's edges plus one voxel, channel counts
+    # at the edges of the input chunks (8, 16, 32) and of the output tiles (16, 32, 48, 64, two tap groups)
+    (1, 1, 1, 1, 1, 1, 7),
+    (1, 5, 17, 9, 2, 16, 1),
+    (2, 4, 16, 8, 24, 20, 0),
+    (1, 3, 33, 17, 40, 48, 2),
+    (1, 9, 5, 7, 33, 65, 4),
+    (1, 2, 18, 10, 48, 128, 5),
+    (1, 3, 4, 5, 300, 24, 1),
+])
+def test_conv_weight_gradient_tile_edges(nn, case, offset):
+    """The weight gradient where its bricks and channel tiles end, from aligned tensors (16-byte copies) and from
+    ones that start one value past it; the tolerance is that of the cases above."""
+    n, d, h, w, cin, cout, wrap = case
+    rng = np.random.default_rng(17 + hash(case) % 2**31)
+    x = rand_bf16(rng, (n, d, h, w, cin))
+    dy = rand_bf16(rng, (n, d, h, w, cout))
+
+    def dev(a):
+        t = torch.empty(a.size + offset, dtype=torch.bfloat16, device="cuda")
+        t[offset:] = bf16_dev(a).reshape(-1)
+        return t[offset:]
+
+    dw = torch.full((27 * cin * cout,), 0.25, dtype=torch.float32, device="cuda")
+    db = torch.full((cout,), -0.5, dtype=torch.float32, device="cuda")
+    nn.lbm_nn_conv3d_wgrad(dev(x), dev(dy), n, d, h, w, cin, cout, wrap, dw, db)
+    torch.cuda.synchronize()
+    assert nn.lbm_nn_tc_timeouts() == 0
+    ref_w, ref_b = R.conv3d_bwd_weight(x, dy, wrap)
+    tol_w = 2.0 ** -16 * R.conv3d_bwd_weight(np.abs(x), np.abs(dy), wrap)[0] + 1e-6
+    err = np.abs(f64(dw).reshape(27, cin, cout) - 0.25 - ref_w)
+    assert np.all(err <= tol_w), float(np.max(err / tol_w))
+    assert np.allclose(f64(db) + 0.5, ref_b, rtol=1e-5, atol=1e-4)
