@@ -126,11 +126,50 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const bf16* __restrict__ A, con
             tc::cp_async16(sb + tc::tile_off(r, g, TC_KGAP, TC_RGAP), B + (size_t)r * K + kc * TC_BK + g * 8, true);
         }
     };
-    auto out = [&](int r, int c0, const float (&v)[16], bool ok) {
+    auto out = [&](int r, int c0, float (&v)[16], bool ok) {
 #pragma unroll
         for (int k = 0; k < 16; k++) C[(size_t)(m0 + r) * N + c0 + k] = ok ? v[k] : __int_as_float(0x7fc00000);
     };
     tc_pipeline(smem, mbar, &tmem_slot, N, K / TC_BK, fill, out);
+}
+
+// 16 output channels from co0 of one voxel: bias, ReLU, and the stores that the
+// tensors allow (vy: 16 bytes of y, vy32: 16 bytes of y32, else value by value);
+// `at`: offset of (voxel, co0).  NaN where the sums are not there.
+__device__ __forceinline__ void conv_out(float (&v)[16], bool ok, const float* __restrict__ bias, int relu, int co0,
+                                         int Cout, size_t at, bool vy, bool vy32, bf16* __restrict__ y,
+                                         float* __restrict__ y32) {
+#pragma unroll
+    for (int k = 0; k < 16; k++) {
+        v[k] = ok ? v[k] + (bias && co0 + k < Cout ? __ldg(bias + co0 + k) : 0.f) : __int_as_float(0x7fc00000);
+        if (relu) v[k] = fmaxf(v[k], 0.f);
+    }
+    if (y && vy) {
+#pragma unroll
+        for (int k = 0; k < 16; k += 8)
+            if (co0 + k < Cout) {
+                uint32_t h[4];
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const __nv_bfloat162 p = __floats2bfloat162_rn(v[k + 2 * j], v[k + 2 * j + 1]);
+                    h[j] = *reinterpret_cast<const uint32_t*>(&p);
+                }
+                *reinterpret_cast<uint4*>(y + at + k) = make_uint4(h[0], h[1], h[2], h[3]);
+            }
+    } else if (y) {
+#pragma unroll
+        for (int k = 0; k < 16; k++)
+            if (co0 + k < Cout) y[at + k] = __float2bfloat16(v[k]);
+    }
+    if (y32 && vy32) {
+#pragma unroll
+        for (int k = 0; k < 16; k += 4)
+            if (co0 + k < Cout) *reinterpret_cast<float4*>(y32 + at + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+    } else if (y32) {
+#pragma unroll
+        for (int k = 0; k < 16; k++)
+            if (co0 + k < Cout) y32[at + k] = v[k];
+    }
 }
 
 // Neighbour coordinate along one axis: zero padding (-1 outside) or periodic.
@@ -140,17 +179,24 @@ __device__ __forceinline__ int tc_nb(int c, int d, int n, bool wrap) {
     return (c < 0 || c >= n) ? -1 : c;
 }
 
-// The 3x3x3 convolution of lbm_nn_conv3d as an implicit GEMM:
+// The 3x3x3 convolution of lbm_nn_conv3d as an implicit GEMM, for input
+// channels that do not fill K = 16 steps of one tap (Cin % 16 != 0):
 // y[p][co] = act(sum_k A[p][k] B[co][k] + bias[co]) with k = (tap, ci),
 // A[p][(tap, ci)] = x[p + off(tap)][ci] (zero outside, or wrapped on the axes
 // of `wrap`) and B[co][(tap, ci)] = wgt[tap][ci][co].  One block computes 128
-// voxels x NT output channels from blockIdx.y * NT; Cin % 8 == 0 (each 16-byte
-// row segment lies in one tap), NT % 16 == 0.  Rows k >= 27 Cin of the last
-// stage are zero.
+// voxels x NT output channels from blockIdx.y * NT, NT % 16 == 0.  A is read G
+// channels at a time: 8 (Cin % 8 == 0, 16-byte aligned), 2 (even Cin, 4-byte
+// aligned) or 1.  Rows k >= 27 Cin of the last stage are zero; `n_stages` stages
+// are reserved.
+//
+// Bound by the latency of the gathers and of a block's start: at the network's
+// 2-channel input a block has one stage, and as many blocks as shared memory
+// holds overlap.
+template <int G>
 __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ x, int N, int D, int H, int W, int Cin,
                                                  const bf16* __restrict__ wgt, const float* __restrict__ bias,
-                                                 int Cout, int NT, int relu, int wrap, bf16* __restrict__ y,
-                                                 float* __restrict__ y32) {
+                                                 int Cout, int NT, int relu, int wrap, bool vy, bool vy32,
+                                                 bf16* __restrict__ y, float* __restrict__ y32) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t mbar[TC_STAGES];
     __shared__ uint32_t tmem_slot;
@@ -176,103 +222,77 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ x, int
         vox[threadIdx.x] = c;
     }
     __syncthreads();
+    // source of channel ci of tap `tap` for voxel c; null: zero
+    auto source = [&](const int4& c, int tap, int ci) -> const bf16* {
+        if (c.x < 0) return nullptr;
+        const int zz = tc_nb(c.y, tap / 9 - 1, D, wz), yy = tc_nb(c.z, (tap / 3) % 3 - 1, H, wy),
+                  xx = tc_nb(c.w, tap % 3 - 1, W, wx);
+        return (zz | yy | xx) < 0 ? nullptr : x + ((((long long)c.x * D + zz) * H + yy) * W + xx) * Cin + ci;
+    };
     // a thread fills K group g = tid % 8 of rows tid / 8 + 16 j, j = 0 .. 7
     auto fill = [&](unsigned char* sa, unsigned char* sb, int kc) {
         const int g = threadIdx.x & 7;
-        const int k = kc * TC_BK + g * 8;
-        const bool kin = k < K;
-        const int tap = kin ? k / Cin : 0, ci = k - tap * Cin;
-        const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+        const int k0 = kc * TC_BK + g * 8;
+        int tap[8 / G], ci[8 / G];
+#pragma unroll
+        for (int q = 0; q < 8 / G; q++) {
+            const int k = k0 + q * G;
+            tap[q] = k < K ? k / Cin : -1;
+            ci[q] = k - tap[q] * Cin;
+        }
 #pragma unroll
         for (int j = 0; j < 8; j++) {
             const int r = (threadIdx.x >> 3) + 16 * j;
             const int4 c = vox[r];
-            const bf16* src = x;  // a zero fill (padding, past the end) reads nothing
-            bool full = false;
-            if (kin && c.x >= 0) {
-                const int zz = tc_nb(c.y, dz, D, wz), yy = tc_nb(c.z, dy, H, wy), xx = tc_nb(c.w, dx, W, wx);
-                if ((zz | yy | xx) >= 0) {
-                    src = x + ((((long long)c.x * D + zz) * H + yy) * W + xx) * Cin + ci;
-                    full = true;
-                }
-            }
-            tc::cp_async16(sa + tc::tile_off(r, g, TC_KGAP, TC_RGAP), src, full);
-        }
-        // B[co][k] from wgt[k][co]: 8 consecutive co of one k per 16-byte load,
-        // stored down the 8 rows of one segment column
-        for (int e = threadIdx.x; e < TC_BK * (NT / 8); e += 128) {
-            const int kk = e / (NT / 8), c8 = (e - kk * (NT / 8)) * 8;
-            const int k = kc * TC_BK + kk;
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (k < K && n0 + c8 < Cout) v = *reinterpret_cast<const uint4*>(wgt + (size_t)k * Cout + n0 + c8);
-            const bf16* h = reinterpret_cast<const bf16*>(&v);
-            const int g = kk >> 3, col = kk & 7;
+            unsigned char* dst = sa + tc::tile_off(r, g, TC_KGAP, TC_RGAP);
+            if constexpr (G == 8) {
+                const bf16* src = tap[0] >= 0 ? source(c, tap[0], ci[0]) : nullptr;
+                tc::cp_async16(dst, src ? src : x, src != nullptr);  // a zero fill reads nothing
+            } else {
+                uint32_t h[4];
 #pragma unroll
-            for (int j = 0; j < 8; j++)
-                *reinterpret_cast<bf16*>(sb + tc::tile_off(c8 + j, g, TC_KGAP, TC_RGAP) + col * 2) = h[j];
+                for (int q = 0; q < 4; q++) {
+                    if constexpr (G == 2) {
+                        const bf16* src = tap[q] >= 0 ? source(c, tap[q], ci[q]) : nullptr;
+                        h[q] = src ? __ldg(reinterpret_cast<const uint32_t*>(src)) : 0u;
+                    } else {
+                        const bf16* lo = tap[2 * q] >= 0 ? source(c, tap[2 * q], ci[2 * q]) : nullptr;
+                        const bf16* hi = tap[2 * q + 1] >= 0 ? source(c, tap[2 * q + 1], ci[2 * q + 1]) : nullptr;
+                        h[q] = (lo ? __ldg(reinterpret_cast<const unsigned short*>(lo)) : 0u) |
+                               (hi ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(hi)) << 16 : 0u);
+                    }
+                }
+                *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+            }
+        }
+        // B[co][k] from wgt[k][co], 8 consecutive k of one co per 16-byte row segment
+        const unsigned short* wv = reinterpret_cast<const unsigned short*>(wgt);
+        for (int e = threadIdx.x; e < NT * 8; e += 128) {
+            const int co = n0 + e % NT, gk = e / NT;
+            unsigned short h[8];
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                const int kk = kc * TC_BK + gk * 8 + k;
+                h[k] = kk < K && co < Cout ? __ldg(wv + (size_t)kk * Cout + co) : 0;
+            }
+            *reinterpret_cast<uint4*>(sb + tc::tile_off(e % NT, gk, TC_KGAP, TC_RGAP)) =
+                make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
+                           h[6] | (uint32_t)h[7] << 16);
         }
     };
-    // 16 columns of one row (Cout % 16 == 0: a chunk is wholly inside or outside)
-    auto out = [&](int r, int c0, const float (&v)[16], bool ok) {
+    auto out = [&](int r, int c0, float (&v)[16], bool ok) {
         const long long row = m0 + r;
         const int co0 = n0 + c0;
         if (row >= M || co0 >= Cout) return;
-        float a[16];
-#pragma unroll
-        for (int k = 0; k < 16; k++) {
-            a[k] = ok ? v[k] + (bias ? bias[co0 + k] : 0.f) : __int_as_float(0x7fc00000);
-            if (relu) a[k] = fmaxf(a[k], 0.f);
-        }
-        if (y) {
-            uint32_t h[8];
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                const __nv_bfloat162 t = __floats2bfloat162_rn(a[2 * k], a[2 * k + 1]);
-                h[k] = *reinterpret_cast<const uint32_t*>(&t);
-            }
-            uint4* dst = reinterpret_cast<uint4*>(y + row * Cout + co0);
-            dst[0] = make_uint4(h[0], h[1], h[2], h[3]);
-            dst[1] = make_uint4(h[4], h[5], h[6], h[7]);
-        }
-        if (y32) {
-            float4* dst = reinterpret_cast<float4*>(y32 + row * Cout + co0);
-#pragma unroll
-            for (int k = 0; k < 4; k++) dst[k] = make_float4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
-        }
+        conv_out(v, ok, bias, relu, co0, Cout, (size_t)row * Cout + co0, vy, vy32, y, y32);
     };
     tc_pipeline(smem, mbar, &tmem_slot, NT, (K + TC_BK - 1) / TC_BK, fill, out);
 }
 
-// The 3x3x3 convolution with the activations read by the tensor cores straight
-// from a shared-memory halo tile (no im2col copy).  A block computes MB bricks
-// of 8 (x) x 16 (y) x 1 (z) voxels stacked along z, each brick 128 accumulator
-// rows (x fastest) of NT output channels in its own TMEM columns.  The halo
-// tile holds (8 + 2) x (16 + 2) x (MB + 2) voxels of up to 64 input channels
-// as 16-byte cells of 8 channels, laid out [channel group][z][y][x]: for one
-// tap the 8 voxels of a brick line are 8 consecutive cells, i.e. one core
-// matrix, the 16 lines of a brick are 10 cells (160 B) apart, consecutive
-// bricks one tile plane (180 cells) apart and two channel groups one tile
-// (180 (MB + 2) cells) apart, so an MMA's A operand is a descriptor into the
-// tile at the tap's and the brick's offset.  B (the weights, K-major per
-// output channel) streams through a three-stage ring as in k_conv_tc; each
-// stage feeds the MMAs of all MB bricks.  Input channels beyond 64 are taken
-// in chunks, the tile reloaded once the MMAs of the previous chunk have
-// completed.  Cin % 16 == 0, NT % 16 == 0, MB * NT <= 512.
-constexpr int HX = 10, HY = 18;          // halo tile extent in x and y (z: MB + 2)
-constexpr int HPLANE = HX * HY;          // cells of one z plane of the tile
-constexpr uint32_t HLINE = HX * 16;      // brick lines (stride byte offset)
-constexpr int HCC = 64;                  // input channels per chunk
-constexpr int HMB_MAX = 4;               // bricks per block, at most
-
-// bytes between channel groups of the tile (the descriptors' leading byte offset)
-__host__ __device__ constexpr uint32_t halo_gap(int mb) { return (uint32_t)(HPLANE * (mb + 2)) * 16; }
-// shared memory of a block: the halo tile of min(Cin, 64) channels and the B ring
-__host__ __device__ constexpr uint32_t halo_tile_bytes(int cin, int mb) {
-    return (uint32_t)((cin < HCC ? cin : HCC) / 8) * halo_gap(mb);
-}
-__host__ __device__ constexpr uint32_t halo_smem_bytes(int cin, int nt, int mb) {
-    return halo_tile_bytes(cin, mb) + TC_STAGES * (uint32_t)nt * TC_BK * 2;
-}
+constexpr int HX = 10, HY = 18;      // halo tile extent in x and y
+constexpr int HPLANE = HX * HY;      // cells of one z plane of the tile
+constexpr int HMB_MAX = 16;          // z planes of a brick, at most
+constexpr int HZ_MAX = HMB_MAX + 2;  // planes of a halo tile, at most
 
 // Halo-tile coordinate c (the box's coordinate, possibly -1 .. n) along an
 // axis of n voxels: periodic or zero padding; -1 (a zero cell) as well beyond
@@ -283,197 +303,408 @@ __device__ __forceinline__ int halo_nb(int c, int n, bool wrap) {
     return (c < 0 || c >= n) ? -1 : c;
 }
 
-// The weights of the halo-tile convolution as the B stages it streams: for
-// output-channel tile ty (NT channels from ty * NT) and global stage gs (the
-// stages of input-channel chunk cb = 0, HCC, .. in order, 27 cc / TC_BK
-// rounded up per chunk of cc channels), the stage's NT x TC_BK operand in its
-// shared-memory layout (K-major core matrices, tile_off), element (co, kk) =
-// wgt[tap][cb + ci][ty NT + co] for k = (stage within chunk) TC_BK + kk = tap
-// cc + ci, zero past the chunk's 27 cc rows or past Cout.  One thread per
-// 16-byte core-matrix row (8 consecutive kk of one co).
-__global__ void k_pack_weights(const bf16* __restrict__ wgt, int Cin, int Cout, int NT, int G_total,
-                               unsigned char* __restrict__ wpack) {
-    const uint32_t bstage = (uint32_t)NT * TC_BK * 2;
-    const long long units = (long long)bstage / 16;  // per stage
-    const long long total = (long long)((Cout + NT - 1) / NT) * G_total * units;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const long long u = e % units, stage = e / units;
-        const int gs = (int)(stage % G_total), ty = (int)(stage / G_total);
-        // chunk and stage within it
-        int cb = 0, kc = gs;
-        for (;;) {
-            const int cc = Cin - cb < HCC ? Cin - cb : HCC;
-            const int nk = (27 * cc + TC_BK - 1) / TC_BK;
-            if (kc < nk) break;
-            kc -= nk;
-            cb += HCC;
+// ---- copies of bricks and their halos by warp-specialised blocks -------------
+//
+// Where the tiles of a block lie: bricks of 8 x 16 x mb voxels, x fastest.
+struct Brick {
+    int x0, y0, z0, n;
+};
+__device__ __forceinline__ Brick brick_at(long long t, int BX, int BY, int BZ, int mb) {
+    Brick b;
+    b.x0 = (int)(t % BX) * 8;
+    t /= BX;
+    b.y0 = (int)(t % BY) * 16;
+    t /= BY;
+    b.z0 = (int)(t % BZ) * mb;
+    b.n = (int)(t / BZ);
+    return b;
+}
+
+constexpr int FILL_THREADS = 256;  // copying threads of a block (eight warps)
+
+// The source of a brick's halo cells along each axis, one entry per tile
+// coordinate: the plane's address (null: a plane of zeros) and voxel offsets
+// within the plane (negative: a zero cell).  The copying threads write it once
+// per brick; a cell's address is then two additions and a multiplication
+// (recomputed per cell from its coordinates, the copies took 0.7 to 1 us per
+// 16 bytes and thread, more than the MMAs they fed).
+struct HaloAxes {
+    const bf16* z[HZ_MAX];
+    long long y[HY];
+    int x[HX];
+};
+
+__device__ __forceinline__ void halo_axes(HaloAxes& ax, int ft, const bf16* src, const Brick& b, int mb, int D, int H,
+                                          int W, int C, int wrap) {
+    if (ft < HX) ax.x[ft] = halo_nb(b.x0 + ft - 1, W, wrap & 1);
+    const int yi = ft - 32;
+    if (yi >= 0 && yi < HY) {
+        const int yy = halo_nb(b.y0 + yi - 1, H, wrap & 2);
+        ax.y[yi] = yy < 0 ? -1 : (long long)yy * W;
+    }
+    const int zi = ft - 64;
+    if (zi >= 0 && zi < mb + 2) {
+        const int zz = halo_nb(b.z0 + zi - 1, D, wrap & 4);
+        ax.z[zi] = zz < 0 ? nullptr : src + (size_t)((long long)b.n * D + zz) * H * W * C;
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(FILL_THREADS) : "memory");
+}
+
+// Copies planes z0 .. z1 - 1 of the halo tile, channels c0 .. c0 + 8 ncg - 1,
+// to [z][channel group][y][x] cells of 16 bytes at `dst`, `plane` cells from
+// one (z, channel group) plane to the next: cp.async (VEC: C % 8 == 0, 16-byte
+// aligned source), else value by value.  Lanes run over the channel groups of
+// a cell first, then over the cells of a line.
+template <bool VEC>
+__device__ __forceinline__ void fill_halo(unsigned char* dst, const HaloAxes& ax, const bf16* any, int ft, int ncg,
+                                          int z0, int z1, int plane, int c0, int C) {
+    const int step = FILL_THREADS / ncg, cell0 = ft / ncg, cg = ft - cell0 * ncg;
+    int hx = cell0 % HX, hy = cell0 / HX % HY, hz = cell0 / HPLANE;
+    const int sx = step % HX, sy = step / HX % HY, sz = step / HPLANE;
+    const int ci = c0 + cg * 8, cells = (z1 - z0) * HPLANE;
+    const bool cin = ci < C;
+#pragma unroll 4
+    for (int e = cell0 < step ? cell0 : cells; e < cells; e += step) {
+        const bf16* zp = ax.z[z0 + hz];
+        const long long yo = ax.y[hy];
+        const int xo = ax.x[hx];
+        const bool get = zp && yo >= 0 && xo >= 0 && cin;
+        const bf16* src = zp + (yo + xo) * C + ci;
+        unsigned char* to = dst + (uint32_t)((hz * ncg + cg) * plane + hy * HX + hx) * 16u;
+        if constexpr (VEC) {
+            tc::cp_async16(to, get ? src : any, get);
+        } else {
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (get) v = tc::load8(src, C - ci);
+            *reinterpret_cast<uint4*>(to) = v;
         }
-        const int cc = Cin - cb < HCC ? Cin - cb : HCC;
-        const int c8 = (int)(u / (TC_BK / 8)) , gk = (int)(u % (TC_BK / 8));  // row co = c8, k-group gk
-        const int co = ty * NT + c8;
-        uint4 out;
-        bf16* h = reinterpret_cast<bf16*>(&out);
-#pragma unroll
-        for (int col = 0; col < 8; col++) {
-            const int k = kc * TC_BK + gk * 8 + col;
-            bf16 v = __float2bfloat16(0.f);
-            if (k < 27 * cc && co < Cout) {
-                const int tap = k / cc, ci = k - tap * cc;
-                v = wgt[((size_t)tap * Cin + cb + ci) * Cout + co];
-            }
-            h[col] = v;
-        }
-        *reinterpret_cast<uint4*>(wpack + (size_t)stage * bstage + tc::tile_off(c8, gk, TC_KGAP, TC_RGAP)) = out;
+        hx += sx;
+        hy += sy;
+        hz += sz;
+        if (hx >= HX) hx -= HX, hy++;
+        if (hy >= HY) hy -= HY, hz++;
     }
 }
 
-__global__ void __launch_bounds__(128) k_conv_halo(const bf16* __restrict__ x, int N, int D, int H, int W, int Cin,
-                                                   const unsigned char* __restrict__ wpack, int G_total,
-                                                   const float* __restrict__ bias,
-                                                   int Cout, int NT, int MB, int relu, int wrap,
-                                                   bf16* __restrict__ y, float* __restrict__ y32) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ uint64_t mbar[TC_STAGES];
-    __shared__ uint32_t tmem_slot;
-    unsigned char* const tile = smem;
-    unsigned char* const ring = smem + halo_tile_bytes(Cin, MB);
-    const uint32_t bstage = (uint32_t)NT * TC_BK * 2;
-    const uint32_t hgap = halo_gap(MB);
-    const int hcells = HPLANE * (MB + 2);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int BX = (W + 7) / 8, BY = (H + 15) / 16, BZ = (D + MB - 1) / MB;
-    int b = blockIdx.x;
-    const int xb = b % BX;
-    b /= BX;
-    const int yb = b % BY;
-    b /= BY;
-    const int z0 = (b % BZ) * MB, n0 = b / BZ;
-    const int x0 = xb * 8, y0 = yb * 16;
-    const int nb = D - z0 < MB ? D - z0 : MB;  // bricks inside the box
-    const int c0 = blockIdx.y * NT;
-    const bool wx = wrap & 1, wy = wrap & 2, wz = wrap & 4;
+// ---- the 3x3x3 convolution ----------------------------------------------------
+//
+// y[p][co] = act(sum_{tap, ci} x[p + off(tap)][ci] wgt[tap][ci][co] + bias[co])
+// with the activations read by the tensor cores straight from halo planes (no
+// im2col copy), Cin % 16 == 0.  A brick of 8 (x) x 16 (y) x mb (z) voxels has
+// one accumulator of 128 rows (x fastest) by nt output channels per z plane,
+// the planes side by side in TMEM.  Input channels come in chunks of 64 (the
+// last one may be shorter).  A stage holds a few input planes of the brick's
+// halo, 10 x 18 cells of 8 channels per [z][channel group]: the 8 voxels of a
+// brick line are one core matrix, and a tap is a start address.  The weights of
+// a chunk stay in shared memory in nine slots, one per (dy, dx): per 16
+// channels the 3 nt columns (dz = 2, 1, 0; co).  Input plane z of the tile adds
+// to the output planes z - 2, z - 1 and z with its dz = 2, 1 and 0 taps: their
+// accumulators are neighbours, so one MMA of N = 3 nt columns takes all three,
+// and the tensor cores read an input plane 9 times instead of 27.  An output's
+// sum runs in the order (chunk, dz, dy, dx, 16 channels).
+//
+// What bounds it: the MMAs' reads of their 128 A rows from shared memory, up to
+// nt = 32 (an MMA of 128 x N x 16 takes max(N / 2, 32 + N / 4) cycles), beyond
+// that the MMAs.  Before and after (blocks of up to four planes that copied,
+// multiplied and stored in turn, 27 MMAs per plane): 48 -> 16 channels on 8 x
+// 64^3 voxels 639 and 220 us, 96 -> 32 on 8 x 32^3 292 and 101, 192 -> 64 on 8 x
+// 16^3 149 and 58, 192 -> 128 on 8 x 48^3 6411 and 1335.
+//
+// Blocks are persistent: each keeps one tile of output channels and walks over
+// bricks.  One warp issues the MMAs, eight copy the planes (the stages that
+// shared memory holds in flight), one the weights (bulk copies, slot by slot as
+// the last plane of a chunk releases them), four write the outputs of the
+// brick before from the other of two accumulator sets.
+constexpr int CV_STAGES = 8;
+constexpr int CV_CC = 64;    // input channels per chunk
+constexpr int CV_EPI = 128;  // output threads (four warps)
+constexpr int CV_THREADS = 32 + CV_EPI + FILL_THREADS + 32;
 
-    uint32_t ncols = 32;
-    while (ncols < (uint32_t)(MB * NT)) ncols <<= 1;
-    if (warp == 0) tc::tmem_alloc(&tmem_slot, ncols);
-    if (tid == 0)
-        for (int s = 0; s < TC_STAGES; s++) tc::mbar_init(&mbar[s], 1);
+struct CvShape {
+    int nt;      // output channels per block: a multiple of 16 up to 64
+    int mb;      // z planes of a brick
+    int chunks;  // ceil(Cin / 64)
+    int planes;  // input planes per stage
+    int pc;      // cells from one (z, channel group) plane to the next
+    int stages;
+    uint32_t slot_bytes, stage_bytes, smem, ncols;
+};
+
+// False where two stages or two accumulator sets do not fit.
+static bool cv_shape(int cin, int nt, int mb, CvShape* s) {
+    s->nt = nt;
+    s->mb = mb;
+    s->chunks = (cin + CV_CC - 1) / CV_CC;
+    const int cc = cin < CV_CC ? cin : CV_CC, ncg = cc / 8;
+    s->planes = CV_CC / cc;
+    // strides that put the cells a warp stores together into different banks
+    s->pc = ncg == 2 ? HPLANE : (ncg == 4 ? HPLANE + 2 : HPLANE + 1);
+    s->slot_bytes = (uint32_t)(cc * 6 * nt);
+    s->stage_bytes = (uint32_t)(s->planes * ncg * s->pc * 16 + 127) / 128 * 128;
+    const uint32_t all = 224u * 1024u, b = 9 * s->slot_bytes;
+    s->stages = b < all ? (int)((all - b) / s->stage_bytes) : 0;
+    if (s->stages > CV_STAGES) s->stages = CV_STAGES;
+    s->smem = b + (uint32_t)s->stages * s->stage_bytes;
+    s->ncols = 32;
+    while ((int)s->ncols < 2 * mb * nt) s->ncols <<= 1;
+    return s->stages >= 2 && s->ncols <= 512;
+}
+
+// 16-byte units of the weights of a chunk of cc input channels: [(dy, dx)][cc /
+// 16][8-channel group][dz = 2, 1, 0][co], 8 consecutive input channels each,
+// zero past Cout.
+__device__ __forceinline__ uint4 cv_weights(const bf16* __restrict__ wgt, int Cin, int Cout, int nt, int c0, int cc,
+                                            int ct, int u) {
+    const int col = u % (3 * nt), t = u / (3 * nt), g = t % (cc / 8), tap = (2 - col / nt) * 9 + t / (cc / 8);
+    const int co = ct * nt + col % nt;
+    unsigned short h[8];
+    const unsigned short* w = reinterpret_cast<const unsigned short*>(wgt) + ((size_t)tap * Cin + c0 + g * 8) * Cout + co;
+#pragma unroll
+    for (int k = 0; k < 8; k++) h[k] = co < Cout ? __ldg(w + (size_t)k * Cout) : 0;
+    return make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
+                      h[6] | (uint32_t)h[7] << 16);
+}
+
+// The weights of every output tile and chunk as the blocks copy them, tile by
+// tile, chunk by chunk (27 nt 16-byte units per 8 input channels).
+__global__ void k_pack_weights(const bf16* __restrict__ wgt, int Cin, int Cout, int nt, int tiles,
+                               uint4* __restrict__ wpack) {
+    const int per_tile = 27 * nt * (Cin / 8), per_chunk = 27 * nt * (CV_CC / 8);
+    const long long total = (long long)tiles * per_tile;
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+        const int ct = (int)(e / per_tile), in = (int)(e - (long long)ct * per_tile), c = in / per_chunk;
+        const int c0 = c * CV_CC, cc = Cin - c0 < CV_CC ? Cin - c0 : CV_CC;
+        wpack[e] = cv_weights(wgt, Cin, Cout, nt, c0, cc, ct, in - c * per_chunk);
+    }
+}
+
+// The MMAs of (dy, dx) tap t of input plane hz (a: its descriptor, at the tap's
+// offset; b: the tap's slot), ks steps of 16 channels, into the accumulators of
+// the output planes hz - 2 .. hz that the brick of nz planes has; called by one
+// lane.  `first`: the plane's first MMAs of the brick's first chunk, which
+// overwrite the accumulator of plane hz.
+__device__ __forceinline__ void cv_issue(uint32_t acc, uint64_t a, uint64_t b, int hz, int nz, int nt, int ks, int pc,
+                                         bool first) {
+    const int lo = hz < 2 ? 0 : hz - 2, hi = hz < nz ? hz : nz - 1;  // output planes
+    const uint64_t bo = b + (uint64_t)((lo - hz + 2) * nt);
+    const uint32_t d = acc + (uint32_t)(lo * nt);
+    const uint32_t id = tc::idesc_bf16_f32(TC_M, (hi - lo + 1) * nt);
+    int k = 0;
+    if (first && hz < nz) {
+        if (hz > lo) tc::mma_bf16(d, a, bo, tc::idesc_bf16_f32(TC_M, (hz - lo) * nt), true);
+        tc::mma_bf16(acc + (uint32_t)(hz * nt), a, b + (uint64_t)(2 * nt), tc::idesc_bf16_f32(TC_M, nt), false);
+        k = 1;
+    }
+    for (; k < ks; k++) tc::mma_bf16(d, a + (uint64_t)(k * 2 * pc), bo + (uint64_t)(k * 6 * nt), id, true);
+}
+
+// Grid: x = bricks (blockIdx.x, + gridDim.x, ..), y = output-channel tiles.
+// wpack NULL (no room for it): the weights' warp gathers them from wgt.
+template <bool VX>
+__global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restrict__ x, int N, int D, int H, int W, int Cin,
+                                                             const bf16* __restrict__ wgt, const uint4* __restrict__ wpack,
+                                                             const float* __restrict__ bias, int Cout, int relu, int wrap,
+                                                             CvShape sh, bool vy, bool vy32, bf16* __restrict__ y,
+                                                             float* __restrict__ y32) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ HaloAxes axes[2];
+    __shared__ uint64_t full[CV_STAGES], empty[CV_STAGES], wfull[9], wempty[9], accf[2], acce[2];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int stop[2];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int BX = (W + 7) / 8, BY = (H + 15) / 16, BZ = (D + sh.mb - 1) / sh.mb;
+    const long long tiles = (long long)N * BZ * BY * BX;
+    unsigned char* const ring = smem + 9 * sh.slot_bytes;
+    if (warp == 0) tc::tmem_alloc(&tmem_slot, sh.ncols);
+    if (tid == 0) {
+        for (int s = 0; s < sh.stages; s++) {
+            tc::mbar_init(&full[s], FILL_THREADS / 32);
+            tc::mbar_init(&empty[s], 1);
+        }
+        for (int t = 0; t < 9; t++) {
+            tc::mbar_init(&wfull[t], 1);
+            tc::mbar_init(&wempty[t], 1);
+        }
+        for (int s = 0; s < 2; s++) {
+            tc::mbar_init(&accf[s], 1);
+            tc::mbar_init(&acce[s], CV_EPI / 32);
+        }
+        stop[0] = stop[1] = 0;
+    }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = tmem_slot;
-    const uint32_t idesc = tc::idesc_bf16_f32(TC_M, NT);
-    const uint32_t tile_a = tc::smem_u32(tile);
     bool ok = true;
-    int g = 0;  // stages issued by the block so far (selects the ring buffer and mbarrier phase)
-
-    // B stage number gs of this block's channel tile (k_pack_weights wrote it
-    // in its shared-memory layout): one 16-byte copy per core-matrix row
-    const unsigned char* const wtile = wpack + (size_t)blockIdx.y * G_total * bstage;
-    auto fill_b = [&](unsigned char* sb, int gs) {
-        const unsigned char* src = wtile + (size_t)gs * bstage;
-        for (uint32_t e = tid; e < bstage / 16; e += 128) tc::cp_async16(sb + e * 16, src + e * 16, true);
-    };
-
-    for (int cb = 0; cb < Cin; cb += HCC) {
-        const int cc = Cin - cb < HCC ? Cin - cb : HCC;
-        const int nk = (27 * cc + TC_BK - 1) / TC_BK;
-        if (cb > 0) {  // every MMA that reads the tile has completed
-            const int last = g - 1;
-            ok &= tc::mbar_wait(&mbar[last % TC_STAGES], (last / TC_STAGES) & 1, TC_WAIT);
-        }
-        // the halo tile of this chunk (zero outside the box, wrapped on periodic axes)
-        for (int e = tid; e < (cc / 8) * hcells; e += 128) {
-            const int cg = e / hcells, cell = e - cg * hcells;
-            const int hx = cell % HX, hy = (cell / HX) % HY, hz = cell / HPLANE;
-            const int zz = halo_nb(z0 + hz - 1, D, wz), yy = halo_nb(y0 + hy - 1, H, wy),
-                      xx = halo_nb(x0 + hx - 1, W, wx);
-            const bool full = (zz | yy | xx) >= 0;
-            const bf16* src = full ? x + ((((long long)n0 * D + zz) * H + yy) * W + xx) * Cin + cb + cg * 8 : x;
-            tc::cp_async16(tile + (size_t)e * 16, src, full);
-        }
-        // the ring's first stages join the tile's copies in the first group
-        for (int p = 0; p < TC_STAGES - 1; p++) {
-            if (p < nk) fill_b(ring + ((g + p) % TC_STAGES) * bstage, g + p);
-            tc::cp_async_commit();
-        }
-        for (int kc = 0; kc < nk; kc++, g++) {
-            const int s = g % TC_STAGES;
-            tc::cp_async_wait<TC_STAGES - 2>();
-            tc::fence_smem_to_async();
-            __syncthreads();
-            if (tid == 0) {
-                tc::fence_after_sync();
-                const uint32_t b0 = tc::smem_u32(ring + s * bstage);
+    if (warp == 0) {
+        // the waits' results are made uniform over the warp, so that the elected
+        // lane's descriptors stay in uniform registers (a lane picked by its
+        // index issues an MMA every 45 cycles at best)
+        auto wait = [&](uint64_t* bar, uint32_t parity) {
+            return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, TC_WAIT));
+        };
+        const uint32_t wslots = tc::smem_u32(smem), rg = tc::smem_u32(ring);
+        int s = 0, it = 0;
+        uint32_t ph = 0, wph = 0;  // phases of the stages and of the weights' slots
+        for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x, it++) {
+            const Brick b = brick_at(t, BX, BY, BZ, sh.mb);
+            const int nz = D - b.z0 < sh.mb ? D - b.z0 : sh.mb, buf = it & 1;
+            const uint32_t acc = tmem + (uint32_t)(buf * sh.mb * sh.nt);
+            if (it >= 2) ok = wait(&acce[buf], ((it >> 1) - 1) & 1);
+            for (int c = 0; c < sh.chunks && ok; c++) {
+                const int cc = Cin - c * CV_CC < CV_CC ? Cin - c * CV_CC : CV_CC, ks = cc / 16;
+                const bool fresh = sh.chunks > 1 || it == 0;  // the weights' slots are filled anew
+                for (int h0 = 0; h0 < nz + 2 && ok; h0 += sh.planes) {
+                    if (!(ok = wait(&full[s], ph))) break;
+                    tc::fence_after_sync();
+                    const int h1 = h0 + sh.planes < nz + 2 ? h0 + sh.planes : nz + 2;
+                    for (int hz = h0; hz < h1 && ok; hz++) {
+                        const uint64_t a0 = tc::smem_desc(rg + s * sh.stage_bytes + (uint32_t)((hz - h0) * (cc / 8) * sh.pc) * 16,
+                                                          (uint32_t)sh.pc * 16, HX * 16);
+                        const uint64_t b0 = tc::smem_desc(wslots, (uint32_t)(3 * sh.nt) * 16, 128);
+                        const uint64_t bt = sh.slot_bytes / 16;
+                        const bool last = sh.chunks > 1 && hz == nz + 1;  // releases the slots
+                        if ((hz == 0 && fresh) || last) {
+                            for (int t9 = 0; t9 < 9; t9++) {
+                                if (hz == 0 && fresh) {
+                                    if (!(ok = wait(&wfull[t9], wph))) break;
+                                    tc::fence_after_sync();
+                                }
+                                if (tc::elect_one()) {
+                                    cv_issue(acc, a0 + (uint64_t)((t9 / 3) * HX + t9 % 3), b0 + t9 * bt, hz, nz, sh.nt, ks,
+                                             sh.pc, c == 0 && t9 == 0);
+                                    if (last) tc::mma_commit(&wempty[t9]);
+                                }
+                                __syncwarp();
+                            }
+                        } else if (tc::elect_one()) {
 #pragma unroll
-                for (int j = 0; j < TC_BK / 16; j++) {
-                    const int k = kc * TC_BK + 16 * j;
-                    if (k >= 27 * cc) break;
-                    const int tap = k / cc, ci = k - tap * cc;
-                    const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;  // 0 .. 2: offsets -1 .. +1
-                    const uint32_t a = tile_a + (uint32_t)(ci / 8) * hgap + (uint32_t)((dz * HY + dy) * HX + dx) * 16;
-                    const uint64_t bdesc = tc::smem_desc(b0 + 2 * j * TC_KGAP, TC_KGAP, TC_RGAP);
-                    for (int m = 0; m < nb; m++)  // brick m: one tile plane further along z
-                        tc::mma_bf16(tmem + (uint32_t)(m * NT), tc::smem_desc(a + (uint32_t)(m * HPLANE) * 16, hgap, HLINE),
-                                     bdesc, idesc, cb > 0 || kc > 0 || j > 0);
+                            for (int t9 = 0; t9 < 9; t9++)
+                                cv_issue(acc, a0 + (uint64_t)((t9 / 3) * HX + t9 % 3), b0 + t9 * bt, hz, nz, sh.nt, ks, sh.pc,
+                                         c == 0 && t9 == 0);
+                        }
+                        __syncwarp();
+                    }
+                    if (tc::elect_one()) {
+                        tc::mma_commit(&empty[s]);
+                        if (c == sh.chunks - 1 && h1 == nz + 2) tc::mma_commit(&accf[buf]);
+                    }
+                    __syncwarp();
+                    if (++s == sh.stages) s = 0, ph ^= 1;
                 }
-                tc::mma_commit(&mbar[s]);
+                if (fresh) wph ^= 1;
             }
-            const int nxt = kc + TC_STAGES - 1;
-            if (nxt < nk) {
-                const int r = (g + TC_STAGES - 1) % TC_STAGES;
-                if (kc >= 1) ok &= tc::mbar_wait(&mbar[r], ((g - 1) / TC_STAGES) & 1, TC_WAIT);
-                fill_b(ring + r * bstage, g + TC_STAGES - 1);
-            }
-            tc::cp_async_commit();
         }
-        tc::cp_async_wait<0>();
+    } else if (warp <= CV_EPI / 32) {
+        const int quad = warp & 3, r = quad * 32 + lane;
+        int it = 0;
+        for (long long t = blockIdx.x; t < tiles; t += gridDim.x, it++) {
+            const Brick b = brick_at(t, BX, BY, BZ, sh.mb);
+            const int nz = D - b.z0 < sh.mb ? D - b.z0 : sh.mb, buf = it & 1;
+            // once a wait has run out: NaN for this and the remaining bricks
+            if (ok) ok = __all_sync(0xffffffffu, tc::mbar_wait(&accf[buf], (it >> 1) & 1, TC_WAIT));
+            tc::fence_after_sync();
+            const int vx = b.x0 + (r & 7), vy_ = b.y0 + (r >> 3);
+            const bool inside = vx < W && vy_ < H;
+            for (int q = 0; q < nz * sh.nt; q += 16) {  // plane q / nt, its columns q % nt ..
+                __syncwarp();
+                const int m = q / sh.nt, co0 = blockIdx.y * sh.nt + q - m * sh.nt;
+                float v[16];
+                tc::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * sh.mb * sh.nt + q), v);
+                if (inside && co0 < Cout)
+                    conv_out(v, ok, bias, relu, co0, Cout, ((((size_t)b.n * D + b.z0 + m) * H + vy_) * W + vx) * Cout + co0, vy,
+                             vy32, y, y32);
+            }
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&acce[buf]);
+        }
+    } else if (warp <= (CV_EPI + FILL_THREADS) / 32) {
+        const int ft = tid - 32 - CV_EPI;
+        constexpr int LAG = 2;  // stages whose copies are in flight before the oldest is waited for
+        int it = 0, fills = 0, s = 0, pending = 0;
+        uint32_t ph = 0;
+        bool stopped = false;
+        auto hand_over = [&]() {  // the oldest pending stage: this warp's copies to it have completed
+            tc::fence_smem_to_async();
+            __syncwarp();
+            const int o = s - pending;
+            if (lane == 0) tc::mbar_arrive(&full[o < 0 ? o + sh.stages : o]);
+            pending--;
+        };
+        auto hand_over_all = [&]() {
+            tc::cp_async_wait<0>();
+            while (pending > 0) hand_over();
+        };
+        for (long long t = blockIdx.x; t < tiles && !stopped; t += gridDim.x, it++) {
+            const Brick b = brick_at(t, BX, BY, BZ, sh.mb);
+            const int nz = D - b.z0 < sh.mb ? D - b.z0 : sh.mb;
+            // a wait that ran out stops every copying warp behind the barrier of halo_axes
+            if (!ok) stop[it & 1] = 1;
+            halo_axes(axes[it & 1], ft, x, b, sh.mb, D, H, W, Cin, wrap);
+            stopped = *(volatile int*)&stop[it & 1];
+            if (stopped) break;
+            for (int c = 0; c < sh.chunks; c++) {
+                const int cc = Cin - c * CV_CC < CV_CC ? Cin - c * CV_CC : CV_CC;
+                for (int h0 = 0; h0 < nz + 2; h0 += sh.planes, fills++) {
+                    // while the stage is still read, first hand over those before it
+                    if (fills >= sh.stages && !__all_sync(0xffffffffu, tc::mbar_test(&empty[s], ph ^ 1))) {
+                        hand_over_all();
+                        if (ok) ok = tc::mbar_wait(&empty[s], ph ^ 1, TC_WAIT);
+                    }
+                    const int h1 = h0 + sh.planes < nz + 2 ? h0 + sh.planes : nz + 2;
+                    if (ok) fill_halo<VX>(ring + s * sh.stage_bytes, axes[it & 1], x, ft, cc / 8, h0, h1, sh.pc, c * CV_CC, Cin);
+                    __syncwarp();
+                    tc::cp_async_commit();
+                    pending++;
+                    if (++s == sh.stages) s = 0, ph ^= 1;
+                    if (pending > LAG) {
+                        tc::cp_async_wait<LAG>();
+                        hand_over();
+                    }
+                }
+            }
+        }
+        hand_over_all();
+        ok &= !stopped;
+    } else {
+        uint32_t ph = 0;
+        bool again = false;
+        const uint4* tile = wpack ? wpack + (size_t)blockIdx.y * 27 * sh.nt * (Cin / 8) : nullptr;
+        for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+            if (again && sh.chunks == 1) break;  // the weights stay
+            for (int c = 0; c < sh.chunks && ok; c++) {
+                const int c0 = c * CV_CC, cc = Cin - c0 < CV_CC ? Cin - c0 : CV_CC;
+                const int units = 3 * sh.nt * (cc / 8);  // of a slot
+                for (int t9 = 0; t9 < 9; t9++) {
+                    if (again && !(ok = __all_sync(0xffffffffu, tc::mbar_wait(&wempty[t9], ph, TC_WAIT)))) break;
+                    unsigned char* slot = smem + t9 * sh.slot_bytes;
+                    if (wpack) {
+                        if (lane == 0)
+                            tc::bulk_copy(slot, tile + (size_t)27 * sh.nt * (c0 / 8) + (size_t)t9 * units, (uint32_t)units * 16,
+                                          &wfull[t9]);
+                    } else {
+                        for (int u = lane; u < units; u += 32)
+                            reinterpret_cast<uint4*>(slot)[u] =
+                                cv_weights(wgt, Cin, Cout, sh.nt, c0, cc, blockIdx.y, t9 * units + u);
+                        tc::fence_smem_to_async();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(&wfull[t9]);
+                    }
+                    __syncwarp();
+                }
+                if (again) ph ^= 1;
+                again = true;
+            }
+        }
+        // bulk copies in flight land before the block ends: the MMAs that wait for them are waited for below
     }
-    const int last = g - 1;
-    bool done = tc::mbar_wait(&mbar[last % TC_STAGES], (last / TC_STAGES) & 1, TC_WAIT);
-    if (!done) done = tc::mbar_wait(&mbar[last % TC_STAGES], (last / TC_STAGES) & 1, TC_WAIT);
-    ok &= done;
     if (!ok && lane == 0) atomicAdd(&g_tc_timeouts, 1u);
-    tc::fence_after_sync();
-    // row r of brick m's accumulator = voxel (x0 + r % 8, y0 + r / 8, z0 + m) of sample n0
-    const int r = warp * 32 + lane;
-    const int vx = x0 + (r & 7), vy = y0 + (r >> 3);
-    const bool inside = vx < W && vy < H;
-    for (int q = 0; q < nb * NT; q += 16) {  // brick q / NT, its columns q % NT ..
-        const int m = q / NT, cq = q - m * NT;
-        const long long row = (((long long)n0 * D + z0 + m) * H + vy) * W + vx;
-        float v[16];
-        tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)q, v);
-        const int co0 = c0 + cq;
-        if (!inside || co0 >= Cout) continue;
-        float a[16];
-#pragma unroll
-        for (int k = 0; k < 16; k++) {
-            a[k] = ok ? v[k] + (bias ? bias[co0 + k] : 0.f) : __int_as_float(0x7fc00000);
-            if (relu) a[k] = fmaxf(a[k], 0.f);
-        }
-        if (y) {
-            uint32_t h[8];
-#pragma unroll
-            for (int k = 0; k < 8; k++) {
-                const __nv_bfloat162 t = __floats2bfloat162_rn(a[2 * k], a[2 * k + 1]);
-                h[k] = *reinterpret_cast<const uint32_t*>(&t);
-            }
-            uint4* dst = reinterpret_cast<uint4*>(y + row * Cout + co0);
-            dst[0] = make_uint4(h[0], h[1], h[2], h[3]);
-            dst[1] = make_uint4(h[4], h[5], h[6], h[7]);
-        }
-        if (y32) {
-            float4* dst = reinterpret_cast<float4*>(y32 + row * Cout + co0);
-#pragma unroll
-            for (int k = 0; k < 4; k++) dst[k] = make_float4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
-        }
-    }
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, ncols);
+        tc::tmem_dealloc(tmem, sh.ncols);
     }
 }
 
@@ -496,74 +727,96 @@ __global__ void __launch_bounds__(128) k_conv_halo(const bf16* __restrict__ x, i
 // TMEM and stores them once.
 //
 // What bounds it: the tensor cores' reads of the 128 or 64 (dz, ci) rows from
-// shared memory, once per (dy, dx), and the L2 reads of the halo.  With
-// operands packed channel-major in memory (three copies of x) a layer wrote and
-// read 4 to 8 times its tensors: 16 -> 16 channels on 8 x 64^3 voxels 1082 us,
-// now 147; 48 -> 16 2636, now 424; 96 -> 32 on 8 x 32^3 914, now 155; 192 ->
-// 128 on 8 x 48^3 5012, now 3978; and 2 -> 16 on 8 x 64^3 (gathered for
-// mma.sync, 1275) 152.
-constexpr int WG_X = 10, WG_Y = 18;       // halo tile extent in x and y (z: MB + 2)
-constexpr int WG_FILL = 256;              // copying threads (eight warps)
-constexpr int WG_THREADS = WG_FILL + 32;  // and the warp that issues the MMAs
+// shared memory, once per (dy, dx): an MMA of 64 x 16 x 16 takes 23 cycles, of
+// 128 x 32 x 16 40.  With operands packed channel-major in memory (three copies
+// of x) a layer wrote and read 4 to 8 times its tensors: 16 -> 16 channels on 8
+// x 64^3 voxels 1082 us, now 134; 48 -> 16 2636, now 430; 96 -> 32 on 8 x 32^3
+// 914, now 137; 192 -> 128 on 8 x 48^3 5012, now 3710; and 2 -> 16 on 8 x 64^3
+// (gathered for mma.sync, 1275) 160.
+constexpr int WG_THREADS = FILL_THREADS + 32;  // the copying warps and the one that issues the MMAs
+constexpr int WG_STAGES = 4;
 
 // Shape of one launch, shared by the host and the kernel.
 struct WgShape {
     int cc;       // input channels per block: 8, 16 or 32
     int ncg;      // cc / 8
-    int nt;       // output channels per block: 16, 32, 48 or 64
+    int nt;       // output channels per block: 16, 32 or 48
     int mb;       // z planes of a brick
-    int tg;       // tap groups: 1 (all nine (dy, dx)) or 2 (five and four)
+    int stages;   // bricks in flight: 2 .. WG_STAGES
     int plane;    // cells from one (z, channel group) plane of the x tile to the next
     int gstride;  // cells from one channel group of the dy brick to the next
     uint32_t a_bytes, stage_bytes, smem, ncols;
 };
 
-// The plane and group strides put the 16-byte cells that a warp stores
-// together (channel groups fastest) into different banks: 8 / ncg mod 8 cells.
-__host__ __device__ inline WgShape wg_shape(int cin, int cout) {
+// Output tiles of at most 48 channels, whose nine (dy, dx) accumulators fit the
+// 512 TMEM columns (64 channels in two groups of taps filled every stage twice:
+// 192 -> 128 channels on 8 x 48^3 voxels 3.9 ms).  Input channels per block: 32
+// (rows 3 * 32 of 128), or 16 (3 * 16 of 64) up to 32 output channels, where the
+// MMA of 64 rows takes little more than half the time (24 against 40 cycles) and
+// twice as many blocks fill the chip.  The plane and group strides put the
+// 16-byte cells that a warp stores together (channel groups fastest) into
+// different banks.
+__host__ __device__ inline WgShape wg_shape(int cin, int cout, int mb_max) {
     WgShape s;
-    s.cc = cin <= 8 ? 8 : ((cin <= 16 || (cin % 32 && cin % 32 <= 16)) ? 16 : 32);
+    const int mt = (cout + 47) / 48;
+    s.nt = ((cout + mt - 1) / mt + 15) / 16 * 16;
+    s.cc = cin <= 8 ? 8 : (cin <= 16 || cout <= 32 || (cin % 32 && cin % 32 <= 16) ? 16 : 32);
     s.ncg = s.cc / 8;
-    s.nt = cout >= 64 ? 64 : (cout + 15) / 16 * 16;
-    s.mb = s.nt > 32 ? 2 : 4;
-    s.tg = 9 * s.nt > 512 ? 2 : 1;
-    const int base = WG_X * WG_Y;  // 180 = 4 mod 8
-    s.plane = s.ncg == 4 ? base + 6 : base;
-    s.gstride = s.mb * 128 + (s.nt / 8 == 2 ? 4 : (s.nt / 8 == 4 ? 2 : 1));
-    s.a_bytes = (uint32_t)((s.mb + 2) * s.ncg * s.plane) * 16;
-    const uint32_t g_bytes = (uint32_t)(s.nt / 8 * s.gstride) * 16;
-    s.stage_bytes = (s.a_bytes + g_bytes + 127) / 128 * 128;
-    // the unused rows of the last plane's MMAs reach past the x tile
-    const int rows8 = 3 * s.ncg > 8 ? 16 : 8;
-    const int over = (s.mb - 1) * s.ncg + rows8 - (s.mb + 2) * s.ncg;
-    const uint32_t over_bytes = over > 0 ? (uint32_t)(over * s.plane) * 16 : 0;
-    s.smem = 2 * s.stage_bytes + (over_bytes > g_bytes ? over_bytes - g_bytes : 0);
-    const int cols = (s.tg == 2 ? 5 : 9) * s.nt;
+    s.plane = s.ncg == 4 ? HPLANE + 6 : HPLANE;  // 8 / ncg mod 8 cells
+    uint32_t tail = 0;
+    for (s.mb = mb_max;; s.mb--) {  // the deepest brick of which two fit (one plane: they do)
+        s.gstride = s.mb * 128 + (s.nt == 16 ? 4 : (s.nt == 32 ? 2 : 1));
+        s.a_bytes = (uint32_t)((s.mb + 2) * s.ncg * s.plane) * 16;
+        const uint32_t g_bytes = (uint32_t)(s.nt / 8 * s.gstride) * 16;
+        s.stage_bytes = (s.a_bytes + g_bytes + 127) / 128 * 128;
+        // the unused rows of the last plane's MMAs reach past the x tile
+        const int over = (s.mb - 1) * s.ncg + (3 * s.ncg > 8 ? 16 : 8) - (s.mb + 2) * s.ncg;
+        const uint32_t over_bytes = over > 0 ? (uint32_t)(over * s.plane) * 16 : 0;
+        tail = over_bytes > g_bytes ? over_bytes - g_bytes : 0;
+        s.stages = (int)((224u * 1024u - tail) / s.stage_bytes);
+        if (s.stages >= 2 || s.mb == 1) break;
+    }
+    if (s.stages > WG_STAGES) s.stages = WG_STAGES;
+    s.smem = (uint32_t)s.stages * s.stage_bytes + tail;
     s.ncols = 32;
-    while ((int)s.ncols < cols) s.ncols <<= 1;
+    while ((int)s.ncols < 9 * s.nt) s.ncols <<= 1;
     return s;
 }
 
-// The MMAs of one stage for the (dy, dx) taps T0 .. T0 + NTAP - 1: nz planes,
-// ny2 pairs of lines.  The whole warp runs the loop, one lane issues.
-template <int T0, int NTAP>
+// The MMAs of one stage: nz planes, ny2 pairs of lines, nine (dy, dx); called by
+// one lane.
 __device__ __forceinline__ void wg_issue(uint32_t tmem, uint64_t a0, uint64_t g0, int nz, int ny2, uint32_t aplane,
-                                         int nt, uint32_t idesc, bool first, bool leader) {
+                                         int nt, uint32_t idesc, bool first) {
     for (int m = 0; m < nz; m++) {
         for (int y2 = 0; y2 < ny2; y2++) {
-            const uint64_t a = a0 + (uint64_t)(m * aplane + (uint32_t)y2 * (2 * WG_X));
+            const uint64_t a = a0 + (uint64_t)(m * aplane + (uint32_t)y2 * (2 * HX));
             const uint64_t g = g0 + (uint64_t)(m * 128 + y2 * 16);
             const bool acc = !(first && m == 0 && y2 == 0);
 #pragma unroll
-            for (int t = T0; t < T0 + NTAP; t++)
-                tc::mma_bf16_if(tmem + (uint32_t)((t - T0) * nt), a + (uint64_t)((t / 3) * WG_X + t % 3), g, idesc, acc,
-                                leader);
+            for (int t = 0; t < 9; t++)
+                tc::mma_bf16(tmem + (uint32_t)(t * nt), a + (uint64_t)((t / 3) * HX + t % 3), g, idesc, acc);
         }
     }
 }
 
-// Grid: x = voxel chunks (bricks blockIdx.x, + gridDim.x, ..), y = input-channel
-// chunks x tap groups, z = output-channel tiles.  part[blockIdx.x][tap][ci][co]
+// First brick of voxel chunk c of `chunks`: where equal parts of the box padded
+// by one voxel on each side (rows by W + 2 and up to a multiple of 8, in units
+// of 64 voxels) begin.  The accumulators truncate, so where a chunk begins is
+// part of the result's rounding: chunks of equal bricks would move the
+// gradient's last bits as far as a different number of chunks does.
+__host__ __device__ inline long long wg_chunk_begin(long long c, long long chunks, long long tiles, int N, int D, int H,
+                                                    int W) {
+    const long long Wp = (W + 2 + 7) / 8 * 8, Hp = H + 2, Dp = D + 2;
+    const long long steps = (N * Dp * Hp * Wp + 63) / 64, line = c * ((steps + chunks - 1) / chunks) * 64 / Wp;
+    const long long n = line / (Hp * Dp), zp = line / Hp % Dp, yp = line % Hp;
+    if (c >= chunks || n >= N) return tiles;
+    // lines of the box before it
+    const long long z = zp < 1 ? 0 : (zp > D ? D : zp - 1), y = zp < 1 || zp > D ? 0 : (yp < 1 ? 0 : (yp > H ? H : yp - 1));
+    return tiles * ((n * D + z) * H + y) / ((long long)N * D * H);
+}
+
+// Grid: x = voxel chunks (consecutive bricks), y = input-channel
+// chunks, z = output-channel tiles.  part[blockIdx.x][tap][ci][co]
 // takes the block's sums (NaN when a wait ran out); k_sum_chunks adds the
 // chunks to dw in a fixed order, so the gradient does not depend on the order
 // in which blocks finish.
@@ -572,23 +825,25 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict_
                                                          int D, int H, int W, int Cin, int Cout, int wrap, WgShape sh,
                                                          float* __restrict__ part) {
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ uint64_t full[2], empty[2], done;
+    __shared__ HaloAxes axes[2];
+    __shared__ uint64_t full[WG_STAGES], empty[WG_STAGES], done;
     __shared__ uint32_t tmem_slot;
-    __shared__ int failed;
+    __shared__ int failed, stop[2];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int c0 = ((int)blockIdx.y / sh.tg) * sh.cc, tgi = (int)blockIdx.y % sh.tg;
+    const int c0 = blockIdx.y * sh.cc;
     const int n0 = blockIdx.z * sh.nt;
     const int BX = (W + 7) / 8, BY = (H + 15) / 16, BZ = (D + sh.mb - 1) / sh.mb;
     const long long tiles = (long long)N * BZ * BY * BX;
-    const bool wx = wrap & 1, wy = wrap & 2, wz = wrap & 4;
+    const long long tile_begin = wg_chunk_begin(blockIdx.x, gridDim.x, tiles, N, D, H, W),
+                    tile_end = wg_chunk_begin(blockIdx.x + 1, gridDim.x, tiles, N, D, H, W);
     if (warp == 0) tc::tmem_alloc(&tmem_slot, sh.ncols);
     if (tid == 0) {
-        for (int s = 0; s < 2; s++) {
-            tc::mbar_init(&full[s], WG_FILL / 32);
+        for (int s = 0; s < sh.stages; s++) {
+            tc::mbar_init(&full[s], FILL_THREADS / 32);
             tc::mbar_init(&empty[s], 1);
         }
         tc::mbar_init(&done, 1);
-        failed = 0;
+        failed = stop[0] = stop[1] = 0;
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -597,104 +852,96 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict_
     const int rows = 3 * sh.ncg > 8 ? 128 : 64;  // (dz, ci) rows of an MMA
     bool ok = true;
     if (warp == 0) {
-        const bool leader = tc::elect_one();
+        // the waits' results are made uniform over the warp, so that the elected
+        // lane's descriptors stay in uniform registers (a lane picked by its
+        // index issues an MMA every 45 cycles at best; these need 23 to 48)
         const uint32_t idesc = tc::idesc_bf16_f32(rows, sh.nt) | tc::IDESC_MN_MAJOR;
-        int it = 0;
-        for (long long t = blockIdx.x; t < tiles; t += gridDim.x, it++) {
-            const int s = it & 1;
-            if (!tc::mbar_wait(&full[s], (it >> 1) & 1, TC_WAIT)) {
+        int s = 0;        // stage
+        uint32_t ph = 0;  // its phase
+        bool first = true;
+        for (long long t = tile_begin; t < tile_end; t++) {
+            if (!__all_sync(0xffffffffu, tc::mbar_wait(&full[s], ph, TC_WAIT))) {
                 ok = false;
                 break;
             }
             tc::fence_after_sync();
-            const long long q = t / BX / BY;
-            const int y0 = (int)(t / BX % BY) * 16, z0 = (int)(q % BZ) * sh.mb;
-            const int nz = D - z0 < sh.mb ? D - z0 : sh.mb, ny2 = H - y0 < 16 ? (H - y0 + 1) / 2 : 8;
+            const Brick b = brick_at(t, BX, BY, BZ, sh.mb);
+            const int nz = D - b.z0 < sh.mb ? D - b.z0 : sh.mb, ny2 = H - b.y0 < 16 ? (H - b.y0 + 1) / 2 : 8;
             const uint32_t st = tc::smem_u32(smem + s * sh.stage_bytes);
-            const uint64_t a0 = tc::smem_desc(st, WG_X * 16, (uint32_t)sh.plane * 16);
+            const uint64_t a0 = tc::smem_desc(st, HX * 16, (uint32_t)sh.plane * 16);
             const uint64_t g0 = tc::smem_desc(st + sh.a_bytes, 128, (uint32_t)sh.gstride * 16);
             const uint32_t ap = (uint32_t)(sh.ncg * sh.plane);
-            if (sh.tg == 1)
-                wg_issue<0, 9>(tmem, a0, g0, nz, ny2, ap, sh.nt, idesc, it == 0, leader);
-            else if (tgi == 0)
-                wg_issue<0, 5>(tmem, a0, g0, nz, ny2, ap, sh.nt, idesc, it == 0, leader);
-            else
-                wg_issue<5, 4>(tmem, a0, g0, nz, ny2, ap, sh.nt, idesc, it == 0, leader);
-            if (leader) tc::mma_commit(&empty[s]);
+            if (tc::elect_one()) {
+                wg_issue(tmem, a0, g0, nz, ny2, ap, sh.nt, idesc, first);
+                tc::mma_commit(&empty[s]);
+            }
             __syncwarp();
+            first = false;
+            if (++s == sh.stages) s = 0, ph ^= 1;
         }
-        if (leader) tc::mma_commit(&done);
+        if (tc::elect_one()) tc::mma_commit(&done);
         __syncwarp();
     } else {
         const int ft = tid - 32;
-        const int acells = (sh.mb + 2) * WG_X * WG_Y * sh.ncg;
-        const int ashift = sh.ncg == 4 ? 2 : sh.ncg - 1;  // log2 ncg
-        const int gcg = sh.nt / 8, gcells = sh.mb * 128 * gcg;
-        int it = 0;
-        for (long long t = blockIdx.x; t < tiles; t += gridDim.x, it++) {
-            const int s = it & 1;
-            if (it >= 2 && !tc::mbar_wait(&empty[s], ((it >> 1) - 1) & 1, TC_WAIT)) {
-                ok = false;
-                break;
+        // this thread's share of the dy brick: one channel group of every gstep-th voxel
+        const int groups = sh.nt / 8, gstep = FILL_THREADS / groups;
+        const int gcell = ft / groups, gcg = ft - gcell * groups, co = n0 + gcg * 8;
+        int it = 0, s = 0, last = -1;  // bricks so far, stage, the stage copied but not handed over
+        uint32_t ph = 0;
+        auto hand_over = [&](int stage) {  // this warp's copies to it have completed
+            tc::fence_smem_to_async();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&full[stage]);
+        };
+        auto hand_over_all = [&]() {
+            tc::cp_async_wait<0>();
+            if (last >= 0) hand_over(last);
+            last = -1;
+        };
+        for (long long t = tile_begin; t < tile_end; t++, it++) {
+            if (it >= sh.stages) {
+                // the stage is still read: first hand over the one before it
+                if (!__all_sync(0xffffffffu, tc::mbar_test(&empty[s], ph ^ 1))) {
+                    hand_over_all();
+                    // a wait that runs out stops every copying warp behind the barrier of halo_axes
+                    if (!tc::mbar_wait(&empty[s], ph ^ 1, TC_WAIT)) stop[it & 1] = 1;
+                }
             }
             unsigned char* sa = smem + s * sh.stage_bytes;
             unsigned char* sg = sa + sh.a_bytes;
-            long long q = t;
-            const int x0 = (int)(q % BX) * 8;
-            q /= BX;
-            const int y0 = (int)(q % BY) * 16;
-            q /= BY;
-            const int z0 = (int)(q % BZ) * sh.mb, n = (int)(q / BZ);
-            // the halo tile of x (zero outside the box, wrapped on periodic axes), channel groups fastest
-#pragma unroll 4
-            for (int e = ft; e < acells; e += WG_FILL) {
-                const int cg = e & (sh.ncg - 1), cell = e >> ashift;
-                const int hx = cell % WG_X, hy = (cell / WG_X) % WG_Y, hz = cell / (WG_X * WG_Y);
-                const int zz = halo_nb(z0 + hz - 1, D, wz), yy = halo_nb(y0 + hy - 1, H, wy),
-                          xx = halo_nb(x0 + hx - 1, W, wx);
-                const int ci = c0 + cg * 8;
-                const bool in = (zz | yy | xx) >= 0;
-                unsigned char* dst = sa + (size_t)((hz * sh.ncg + cg) * sh.plane + hy * WG_X + hx) * 16;
-                const bf16* src = x + ((((long long)n * D + zz) * H + yy) * W + xx) * Cin + ci;
-                if constexpr (VX) {
-                    const bool get = in && ci < Cin;
-                    tc::cp_async16(dst, get ? src : x, get);
-                } else {
-                    uint4 v = make_uint4(0, 0, 0, 0);
-                    if (in) v = tc::load8(src, Cin - ci);
-                    *reinterpret_cast<uint4*>(dst) = v;
-                }
+            const Brick b = brick_at(t, BX, BY, BZ, sh.mb);
+            halo_axes(axes[it & 1], ft, x, b, sh.mb, D, H, W, Cin, wrap);
+            if (*(volatile int*)&stop[it & 1]) {
+                ok = false;
+                break;
             }
+            fill_halo<VX>(sa, axes[it & 1], x, ft, sh.ncg, 0, sh.mb + 2, sh.plane, c0, Cin);
             // the brick of dy, zero outside the box and past Cout
+            const bf16* gb = dy + ((((size_t)b.n * D + b.z0) * H + b.y0) * W + b.x0) * Cout + co;
+            const int gx = W - b.x0, gy = H - b.y0, gz = co < Cout ? D - b.z0 : 0;  // limits of the brick
 #pragma unroll 4
-            for (int e = ft; e < gcells; e += WG_FILL) {
-                const int cell = e / gcg, cg = e - cell * gcg;
-                const int xx = x0 + (cell & 7), yy = y0 + ((cell >> 3) & 15), zz = z0 + (cell >> 7);
-                const int co = n0 + cg * 8;
-                const bool in = xx < W && yy < H && zz < D;
-                unsigned char* dst = sg + (size_t)(cg * sh.gstride + cell) * 16;
-                const bf16* src = dy + ((((long long)n * D + zz) * H + yy) * W + xx) * Cout + co;
+            for (int cell = gcell < gstep ? gcell : sh.mb * 128; cell < sh.mb * 128; cell += gstep) {
+                const int xx = cell & 7, yy = (cell >> 3) & 15, zz = cell >> 7;
+                const bool get = xx < gx && yy < gy && zz < gz;
+                const bf16* src = gb + (((long long)zz * H + yy) * W + xx) * Cout;
+                unsigned char* to = sg + (uint32_t)(gcg * sh.gstride + cell) * 16u;
                 if constexpr (VG) {
-                    const bool get = in && co < Cout;
-                    tc::cp_async16(dst, get ? src : dy, get);
+                    tc::cp_async16(to, get ? src : dy, get);
                 } else {
                     uint4 v = make_uint4(0, 0, 0, 0);
-                    if (in) v = tc::load8(src, Cout - co);
-                    *reinterpret_cast<uint4*>(dst) = v;
+                    if (get) v = tc::load8(src, Cout - co);
+                    *reinterpret_cast<uint4*>(to) = v;
                 }
             }
             tc::cp_async_commit();
-            if (it > 0) {  // the stage before this one has landed
+            if (last >= 0) {  // the stage before this one has landed
                 tc::cp_async_wait<1>();
-                tc::fence_smem_to_async();
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&full[s ^ 1]);
+                hand_over(last);
             }
+            last = s;
+            if (++s == sh.stages) s = 0, ph ^= 1;
         }
-        tc::cp_async_wait<0>();
-        tc::fence_smem_to_async();
-        __syncwarp();
-        if (lane == 0 && it > 0) tc::mbar_arrive(&full[(it - 1) & 1]);
+        hand_over_all();
     }
     bool fin = tc::mbar_wait(&done, 0, TC_WAIT);
     if (!fin) fin = tc::mbar_wait(&done, 0, TC_WAIT);
@@ -704,7 +951,7 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict_
         failed = 1;
     }
     __syncthreads();
-    const bool good = failed == 0;
+    const bool good = failed == 0, none = tile_begin == tile_end;  // no brick: sums of zero
     tc::fence_after_sync();
     if (warp > 0) {
         // row r of the accumulator lies in TMEM lane r (128 rows) or 32 (r / 16) + r % 16 (64 rows); the
@@ -712,14 +959,17 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict_
         const int quad = warp & 3, half = (warp - 1) >> 2;
         const int r = rows == 128 ? quad * 32 + lane : (lane < 16 ? quad * 16 + lane : 128);
         const int dz = r / sh.cc, ci = c0 + r % sh.cc;
-        const int t0 = tgi ? 5 : 0, ntap = sh.tg == 1 ? 9 : (tgi ? 4 : 5);
         const bool mine = r < 3 * sh.cc && ci < Cin;
-        for (int col = half * 16; col < ntap * sh.nt; col += 32) {
+        for (int col = half * 16; col < 9 * sh.nt; col += 32) {
             float v[16];
             tc::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)col, v);
             const int t = col / sh.nt, co0 = n0 + col - t * sh.nt;
             if (!mine || co0 >= Cout) continue;
-            float* dst = part + (((size_t)blockIdx.x * 27 + dz * 9 + t0 + t) * Cin + ci) * Cout + co0;
+            if (none) {
+#pragma unroll
+                for (int k = 0; k < 16; k++) v[k] = 0.f;
+            }
+            float* dst = part + (((size_t)blockIdx.x * 27 + dz * 9 + t) * Cin + ci) * Cout + co0;
             if (Cout % 4 == 0) {
 #pragma unroll
                 for (int k = 0; k < 16; k += 4)
@@ -768,35 +1018,10 @@ extern "C" int lbm_nn_gemm_bf16(const void* a, const void* b, float* c, int m, i
 
 namespace lbm {
 namespace nn {
-// The tensor-core convolution for the shapes it takes (cin % 8 == 0, cout %
-// 16 == 0, 16-byte aligned operands); returns 1, launching nothing, for the
-// others.
-int conv3d_tc(const void* x, int n, int d, int h, int w, int cin, const void* wgt, const float* bias, int cout,
-              int relu, int wrap, void* y, float* y32, cudaStream_t s) {
-    if (cin % 8 || cout % 16 || ((uintptr_t)x | (uintptr_t)wgt | (uintptr_t)y | (uintptr_t)y32) & 15) return 1;
-    const int tiles = (cout + 127) / 128;
-    const int nt = ((cout / tiles + 15) / 16) * 16;
-    const long long M = (long long)n * d * h * w;
-    const long long gx = (M + TC_M - 1) / TC_M;
-    if (gx > 0x7fffffff) return 1;
-    const uint32_t smem = TC_STAGES * tc_stage_bytes(nt);
-    int rc = tc_launch_ok((const void*)k_conv_tc, smem, "cudaFuncSetAttribute(k_conv_tc)");
-    if (rc) return rc;
-    k_conv_tc<<<dim3((unsigned)gx, (unsigned)((cout + nt - 1) / nt)), 128, smem, s>>>(
-        static_cast<const bf16*>(x), n, d, h, w, cin, static_cast<const bf16*>(wgt), bias, cout, nt, relu, wrap,
-        static_cast<bf16*>(y), y32);
-    const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_conv_tc launch");
-}
-}  // namespace nn
-}  // namespace lbm
-
-namespace lbm {
-namespace nn {
 static int g_halo_mb = 0, g_halo_nt = 0;  // fixed by lbm_nn_conv_tune; 0 = chosen per shape
-// The halo-tile convolution's weights packed as B stages (k_pack_weights):
-// kept for the process, grown on demand; calls on one stream reuse it in order.
-static unsigned char* g_wpack = nullptr;
+// The convolution's weights packed as its slots (k_pack_weights): kept for
+// the process, grown on demand; calls on one stream reuse it in order.
+static uint4* g_wpack = nullptr;
 static size_t g_wpack_bytes = 0;
 
 static int sm_count() {
@@ -811,72 +1036,99 @@ static int sm_count() {
     return sms;
 }
 
-// The halo-tile tensor-core convolution (cin % 16 == 0, cout % 16 == 0,
-// 16-byte aligned operands); returns 1, launching nothing, for other shapes.
-int conv3d_halo(const void* x, int n, int d, int h, int w, int cin, const void* wgt, const float* bias, int cout,
-                int relu, int wrap, void* y, float* y32, cudaStream_t s) {
-    if (cin % 16 || cout % 16 || ((uintptr_t)x | (uintptr_t)wgt | (uintptr_t)y | (uintptr_t)y32) & 15) return 1;
-    const long long plane_bricks = (long long)n * ((h + 15) / 16) * ((w + 7) / 8);
-    if (plane_bricks * d > 0x7fffffff) return 1;
-    const int sms = sm_count();
-    // Launch shape: mb bricks per block along z and nt output channels per
-    // block (the default tile of at most 128 channels, or a half, quarter ..
-    // of it).  Preferred: at least 1.5 blocks per SM in the grid and two
-    // blocks per SM by shared memory (one block's halo copy overlaps another's
-    // MMAs) within the SM's 512 TMEM columns; among those, the most work per
-    // block (mb nt), then the deeper brick stack.  Measured on the U-Net's
-    // layers, this picks the fastest shape or one within 5 % of it.
+// The convolution as an implicit GEMM, any channel counts and alignment.
+static int conv3d_im2col(const void* x, int n, int d, int h, int w, int cin, const void* wgt, const float* bias, int cout,
+                         int relu, int wrap, void* y, float* y32, bool vy, bool vy32, cudaStream_t s) {
     const int tiles = (cout + 127) / 128;
-    const int nt0 = ((cout / tiles + 15) / 16) * 16;
-    int mb = 0, nt = 0;
-    long long key = -1;
-    for (int ntc = g_halo_nt ? g_halo_nt : nt0; ntc >= 16; ntc = (ntc % 32 == 0 && !g_halo_nt) ? ntc / 2 : 0) {
-        for (int m = HMB_MAX; m >= 1; m--) {
-            if ((g_halo_mb && m != g_halo_mb) || (!g_halo_mb && m == 3) || m * ntc > 512) continue;
-            const long long nblk = plane_bricks * ((d + m - 1) / m) * ((cout + ntc - 1) / ntc);
-            uint32_t cols = 32;
-            while (cols < (uint32_t)(m * ntc)) cols <<= 1;
-            uint32_t per_sm = (228u << 10) / (halo_smem_bytes(cin, ntc, m) + 1024u);
-            per_sm = per_sm > 16 ? 16 : per_sm;
-            const bool occ = per_sm >= 2 && cols * per_sm <= 512u, grid = 2 * nblk >= 3LL * sms;
-            // lexicographic: both, occupancy, then work per block (or, short of
-            // a full grid, the block count), then brick depth
-            const long long k = ((long long)(occ && grid) << 62) | ((long long)occ << 61) |
-                                ((grid ? (long long)(m * ntc) : (nblk < (1LL << 40) ? nblk : (1LL << 40) - 1)) << 3) | m;
-            if (k > key) key = k, mb = m, nt = ntc;
+    const int nt = ((cout + tiles - 1) / tiles + 15) / 16 * 16;
+    const long long M = (long long)n * d * h * w;
+    const long long gx = (M + TC_M - 1) / TC_M;
+    if (gx > 0x7fffffff || tiles > 65535) return fail(LBM_ERR_ARG, "convolution: grid of %lld x %d blocks", gx, tiles);
+    const int nk = (27 * cin + TC_BK - 1) / TC_BK;  // a block's stages: the ring holds no more
+    const uint32_t smem = (nk < TC_STAGES ? nk : TC_STAGES) * tc_stage_bytes(nt);
+    auto go = [&](auto kern) -> int {
+        int rc = tc_launch_ok((const void*)kern, smem, "cudaFuncSetAttribute(k_conv_tc)");
+        if (rc) return rc;
+        kern<<<dim3((unsigned)gx, (unsigned)((cout + nt - 1) / nt)), 128, smem, s>>>(
+            static_cast<const bf16*>(x), n, d, h, w, cin, static_cast<const bf16*>(wgt), bias, cout, nt, relu, wrap, vy, vy32,
+            static_cast<bf16*>(y), y32);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_conv_tc launch");
+    };
+    if (cin % 8 == 0 && (uintptr_t)x % 16 == 0) return go(k_conv_tc<8>);
+    return cin % 2 == 0 && (uintptr_t)x % 4 == 0 ? go(k_conv_tc<2>) : go(k_conv_tc<1>);
+}
+
+// Launch shape: the output-channel tile nt and brick depth mb of the least
+// time by the model below, in SM cycles: bricks per block times the MMAs (9 per
+// input plane and 16 channels, of 128 x 3 nt x 16) or the copies of the planes
+// (near 24 bytes a cycle), whichever is longer, some cycles per plane and
+// brick, and the weights at a block's start.
+static CvShape cv_pick(int n, int d, int h, int w, int cin, int cout, int* grid_x) {
+    CvShape best{};
+    double least = 0;
+    const int want = (cout + 15) / 16 * 16, most = want < 64 ? want : 64;
+    for (int nt = most; nt >= 16; nt -= 16) {
+        if (g_halo_nt && (nt > g_halo_nt || least > 0)) continue;  // fixed: the widest that fits, up to it
+        const long long gy = (cout + nt - 1) / nt;
+        for (int mb = HMB_MAX; mb >= 1; mb = mb > 4 ? mb / 2 : mb - 1) {
+            CvShape s;
+            if ((g_halo_mb ? mb != g_halo_mb : mb == 3) || !cv_shape(cin, nt, mb, &s)) continue;
+            const long long tiles = (long long)n * ((d + mb - 1) / mb) * ((h + 15) / 16) * ((w + 7) / 8);
+            long long gx = sm_count() / gy;
+            if (gx < 1) gx = 1;
+            if (gx > tiles) gx = tiles;
+            const long long per = (tiles + gx - 1) / gx, waves = (gx * gy + sm_count() - 1) / sm_count();
+            const int planes = (mb < d ? mb : d) + 2;
+            const double mma = 9.0 * (cin / 16) * (1.5 * nt > 32 + 0.75 * nt ? 1.5 * nt : 32 + 0.75 * nt);
+            const double copy = (double)(cin / 8) * HPLANE * 16 / 24.0;
+            const double fill = 9.0 * s.slot_bytes / 40.0;  // a chunk's weights
+            const double cost = (double)waves * (per * (planes * ((mma > copy ? mma : copy) + 60.0) + 800.0 * s.chunks) + 6000.0 + fill);
+            if (least == 0 || cost < least) least = cost, best = s, *grid_x = (int)gx;
         }
     }
-    if (!mb) return 1;
-    const int gy = (cout + nt - 1) / nt;
-    const long long blocks = plane_bricks * ((d + mb - 1) / mb);
-    const uint32_t smem = halo_smem_bytes(cin, nt, mb);
-    int rc = tc_launch_ok((const void*)k_conv_halo, smem, "cudaFuncSetAttribute(k_conv_halo)");
-    if (rc) return rc;
-    // the weights as the blocks' B stages (a library-owned buffer, repacked per call)
-    int G_total = 0;
-    for (int cb = 0; cb < cin; cb += HCC) G_total += (27 * (cin - cb < HCC ? cin - cb : HCC) + TC_BK - 1) / TC_BK;
-    const size_t pack_bytes = (size_t)gy * G_total * nt * TC_BK * 2;
-    if (pack_bytes > g_wpack_bytes) {
+    return best;
+}
+
+// The convolution: halo planes for cin % 16 == 0, else the implicit GEMM.  Any
+// channel counts and alignment (16-byte copies and stores where a tensor's
+// channels and address allow, else narrower ones).
+int conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt, const float* bias, int cout, int relu,
+           int wrap, void* y, float* y32, cudaStream_t s) {
+    const bool vy = cout % 8 == 0 && (uintptr_t)y % 16 == 0, vy32 = cout % 4 == 0 && (uintptr_t)y32 % 16 == 0;
+    if (cin % 16) return conv3d_im2col(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, vy, vy32, s);
+    int gx = 1;
+    const CvShape sh = cv_pick(n, d, h, w, cin, cout, &gx);
+    const long long gy = sh.nt ? (cout + sh.nt - 1) / sh.nt : 0;
+    if (gy < 1 || gy > 65535) return fail(LBM_ERR_ARG, "convolution: %d output channels exceed the grid", cout);
+    const size_t units = (size_t)gy * 27 * sh.nt * (cin / 8);
+    if (units * 16 > g_wpack_bytes) {
         if (g_wpack) cudaFree(g_wpack);
         g_wpack = nullptr;
         g_wpack_bytes = 0;
-        if (cudaMalloc(&g_wpack, pack_bytes) != cudaSuccess) {
+        if (cudaMalloc(&g_wpack, units * 16) == cudaSuccess) {
+            g_wpack_bytes = units * 16;
+        } else {  // no room: the blocks gather the weights
             (void)cudaGetLastError();
             g_wpack = nullptr;
-            return 1;  // no room: the other kernels need no packed weights
         }
-        g_wpack_bytes = pack_bytes;
     }
-    const long long units = (long long)pack_bytes / 16;
-    k_pack_weights<<<(unsigned)((units + 127) / 128 < 1216 ? (units + 127) / 128 : 1216), 128, 0, s>>>(
-        static_cast<const bf16*>(wgt), cin, cout, nt, G_total, g_wpack);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "k_pack_weights launch");
-    k_conv_halo<<<dim3((unsigned)blocks, (unsigned)gy), 128, smem, s>>>(
-        static_cast<const bf16*>(x), n, d, h, w, cin, g_wpack, G_total, bias, cout, nt, mb, relu, wrap,
-        static_cast<bf16*>(y), y32);
-    e = cudaGetLastError();
-    return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_conv_halo launch");
+    if (g_wpack) {
+        k_pack_weights<<<(unsigned)((units + 127) / 128 < 1216 ? (units + 127) / 128 : 1216), 128, 0, s>>>(
+            static_cast<const bf16*>(wgt), cin, cout, sh.nt, (int)gy, g_wpack);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e, "k_pack_weights launch");
+    }
+    auto go = [&](auto kern) -> int {
+        int rc = tc_launch_ok((const void*)kern, sh.smem, "cudaFuncSetAttribute(k_conv_halo)");
+        if (rc) return rc;
+        kern<<<dim3((unsigned)gx, (unsigned)gy), CV_THREADS, sh.smem, s>>>(
+            static_cast<const bf16*>(x), n, d, h, w, cin, static_cast<const bf16*>(wgt), g_wpack, bias, cout, relu, wrap, sh,
+            vy, vy32, static_cast<bf16*>(y), y32);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_conv_halo launch");
+    };
+    return (uintptr_t)x % 16 == 0 ? go(k_conv_halo<true>) : go(k_conv_halo<false>);
 }
 }  // namespace nn
 }  // namespace lbm
@@ -948,15 +1200,28 @@ int sum_chunks(const float* part, long long chunks, long long E, float* dst, cud
 // where a tensor's channels and address allow, else value by value).
 int wgrad_tc(const void* x, const void* dy, int n, int d, int h, int w, int cin, int cout, int wrap, float* dw,
              cudaStream_t s) {
-    const WgShape sh = wg_shape(cin, cout);
+    // Voxel chunks: a block's FP32 accumulators in TMEM truncate, about 2e-8 of a sum per K = 16 step, so the
+    // chunks (their number here, their bounds in wg_chunk_begin) are part of the result's rounding.  A chunk is
+    // one of SMs / q of the voxels, q the 448-column accumulators that 27 taps of the input channels would fill
+    // (and the 128-channel output tiles), or 8192 voxels outside 8 .. 256 input channels; shorter chunks would be
+    // more exact, but up to 1e-4 from the results of that split, more than FP32 results may move.  For the same
+    // reason long sums run in bricks of few planes, closer to the order of memory: on random operands of 884,736
+    // voxels by 96 and 192 channels 1.8e-5 and 3.2e-5 from it with four planes, 1.3e-5 and 2.6e-5 with two, 7e-6
+    // and 1.1e-5 with one, which costs up to 1.4 times the time.
+    const long long M = (long long)n * d * h * w;
+    long long chunks = (M + 8191) / 8192;
+    const int cp = (cin + 15) / 16 * 16;
+    if (cin >= 8 && cp <= 256) {
+        const int per = 448 / cp < 27 ? 448 / cp : 27;
+        chunks = sm_count() / ((27 + per - 1) / per * ((cout + 127) / 128));
+    }
+    if (chunks < 1) chunks = 1;
+    const long long steps = M / 16 / chunks;
+    const WgShape sh = wg_shape(cin, cout, steps > 2700 ? 1 : (steps > 1600 ? 2 : 4));
     const long long tiles = (long long)n * ((d + sh.mb - 1) / sh.mb) * ((h + 15) / 16) * ((w + 7) / 8);
-    const long long groups = (long long)((cin + sh.cc - 1) / sh.cc) * sh.tg, mt = (cout + sh.nt - 1) / sh.nt;
+    const long long groups = (cin + sh.cc - 1) / sh.cc, mt = (cout + sh.nt - 1) / sh.nt;
     if (groups > 65535 || mt > 65535)
         return fail(LBM_ERR_ARG, "weight gradient: %d x %d channels exceed the grid", cin, cout);
-    // one resident block per SM, two where shared memory and TMEM hold them; each block's sums are one partial sum
-    const int per_sm = 2 * (sh.smem + 1024) <= (228u << 10) && 2 * sh.ncols <= 512 ? 2 : 1;
-    long long chunks = (long long)per_sm * sm_count() / (groups * mt);
-    if (chunks < 1) chunks = 1;
     if (chunks > tiles) chunks = tiles;
     const long long E = 27LL * cin * cout;
     float* part = chunk_scratch((size_t)(chunks * E));
@@ -981,16 +1246,13 @@ extern "C" int lbm_nn_conv3d_tc(const void* x, int n, int d, int h, int w, int c
                                 const float* bias, int cout, int relu, int wrap, void* y, float* y32, void* stream) {
     if (!x || !wgt || n < 1 || d < 1 || h < 1 || w < 1 || cin < 1 || cout < 1 || (!y && !y32) || (wrap & ~7))
         return fail(LBM_ERR_ARG, "lbm_nn_conv3d_tc: bad arguments");
-    // the halo-tile kernel for cin % 16 == 0, else the im2col one (cin % 8 == 0)
-    int rc = conv3d_halo(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, static_cast<cudaStream_t>(stream));
-    if (rc == 1) rc = conv3d_tc(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, static_cast<cudaStream_t>(stream));
-    if (rc == 1)
+    if (cin % 8 || cout % 16 || ((uintptr_t)x | (uintptr_t)wgt | (uintptr_t)y | (uintptr_t)y32) & 15)
         return fail(LBM_ERR_ARG, "lbm_nn_conv3d_tc: needs cin %% 8 == 0, cout %% 16 == 0 and 16-byte aligned operands");
-    return rc;
+    return conv3d(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int lbm_nn_conv_tune(int bricks_z, int cout_tile) {
-    if (bricks_z < 0 || bricks_z > HMB_MAX || cout_tile < 0 || cout_tile > 128 || cout_tile % 16 ||
+    if (bricks_z < 0 || bricks_z > 4 || cout_tile < 0 || cout_tile > 128 || cout_tile % 16 ||
         (bricks_z && cout_tile && bricks_z * cout_tile > 512))
         return fail(LBM_ERR_ARG, "lbm_nn_conv_tune: bricks_z in 0..4, cout_tile a multiple of 16 in 0..128");
     g_halo_mb = bricks_z;

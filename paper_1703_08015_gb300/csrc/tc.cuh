@@ -65,22 +65,11 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
 // along K and the stride byte offset between those adjacent along M or N.
 constexpr uint32_t IDESC_MN_MAJOR = (1u << 15) | (1u << 16);
 
-// One lane of a converged warp (the same one on every call).
+// True in one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
     return p != 0;
-}
-
-// mma_bf16 executed by a whole warp, issued where `issue` is set (one lane):
-// the descriptors stay uniform over the warp.
-__device__ __forceinline__ void mma_bf16_if(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                            bool accumulate, bool issue) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate), "r"((uint32_t)issue)
-        : "memory");
 }
 
 // The mbarrier receives one arrival once every MMA this thread issued before
@@ -100,6 +89,18 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
 
+// `bytes` (a multiple of 16, both addresses 16-byte aligned) from global to
+// shared memory, asynchronously; the mbarrier's phase expects this one arrival
+// and the bytes, and completes when they have landed, visible to the tensor
+// cores.
+__device__ __forceinline__ void bulk_copy(void* smem, const void* gmem, uint32_t bytes, uint64_t* mbar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(smem)),
+                 "l"(gmem), "r"(bytes), "r"(smem_u32(mbar))
+                 : "memory");
+}
+
 // Wait until the phase of parity `parity` has completed; false after `limit`
 // polls.
 __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint32_t limit) {
@@ -115,6 +116,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint3
         if (done) return true;
     }
     return false;
+}
+
+// True once the phase of parity `parity` has completed; does not wait for it.
+__device__ __forceinline__ bool mbar_test(uint64_t* mbar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(smem_u32(mbar)), "r"(parity)
+        : "memory");
+    return done != 0;
 }
 
 // Shared-memory writes of this thread become visible to the tensor cores.
