@@ -4,61 +4,71 @@
 #include <cuda_bf16.h>
 
 #include <cstdint>
-#include <type_traits>
 
 #include "internal.h"
 #include "lbm_nn.h"
+#include "tc.cuh"
 
 namespace lbm {
 namespace nn {
 
 using bf16 = __nv_bfloat16;
 
-// Partial bias gradients of row blocks: part[blockIdx.x][c] = sum of dy over the
-// block's rows.  Bound by reading dy once: a thread keeps V consecutive channels
-// (one 16- or 8-byte load per row) and takes every R-th row of the block, R =
-// kBiasThreads / (C / V) rows in flight, so that a warp reads consecutive
-// memory; the R partial sums of a channel are then added in row order.  (One
-// thread per channel walking 4096 rows kept 16 threads of a block busy on a
-// 16-channel layer: the 15 layers of a training step on 8 x 64^3 voxels took
-// 5.4 ms with their chunk sums, 0.2 ms this way.)
-// Channel groups beyond kBiasThreads go to further blocks along y.
+// Partial bias gradients of blocks of kBiasRows rows: part[blockIdx.x][c] = sum
+// of dy over the block's rows, in row order (one FP32 chain per channel: the
+// order is part of the result's rounding).  The block's threads bring the rows
+// to shared memory, tile after tile, 16 bytes at a time where VEC (C % 8 == 0,
+// aligned), the next tile in flight while one thread per channel walks the
+// last.  Bound by that chain, 4096 additions, about 10 us for any layer; walking
+// memory instead of shared memory the 15 layers of a training step on 8 x 64^3
+// voxels took 5.4 ms with their chunk sums.
 constexpr int kBiasThreads = 256;
+constexpr int kBiasRows = 4096;
+constexpr int kBiasTile = 8192;  // values of a tile, at most (a row wider than that takes several passes)
 
-template <int V>
+template <bool VEC>
 __global__ void __launch_bounds__(kBiasThreads) k_bias_grad(const bf16* __restrict__ dy, long long M, int C,
-                                                            float* __restrict__ part, long long rows_per_block) {
-    __shared__ float sm[kBiasThreads][V];
-    const int G = C / V;  // channel groups
-    const int g0 = blockIdx.y * kBiasThreads, gn = G - g0 < kBiasThreads ? G - g0 : kBiasThreads;
-    const int R = kBiasThreads / gn;
-    const int r = threadIdx.x / gn, g = threadIdx.x - r * gn;
-    const long long r0 = (long long)blockIdx.x * rows_per_block;
-    const long long r1 = r0 + rows_per_block < M ? r0 + rows_per_block : M;
-    float s[V];
-#pragma unroll
-    for (int k = 0; k < V; k++) s[k] = 0.f;
-    if (r < R) {
-        const bf16* src = dy + (size_t)(g0 + g) * V;
-#pragma unroll 8
-        for (long long row = r0 + r; row < r1; row += R) {
-            const bf16* p = src + row * C;
-            bf16 h[V];
-            if constexpr (V == 8) *reinterpret_cast<uint4*>(h) = __ldg(reinterpret_cast<const uint4*>(p));
-            else if constexpr (V == 4) *reinterpret_cast<uint2*>(h) = __ldg(reinterpret_cast<const uint2*>(p));
-            else h[0] = p[0];
-#pragma unroll
-            for (int k = 0; k < V; k++) s[k] += __bfloat162float(h[k]);
+                                                            float* __restrict__ part) {
+    __shared__ __align__(16) bf16 sm[2][kBiasTile];
+    const long long r0 = (long long)blockIdx.x * kBiasRows;
+    const int rows = (int)(M - r0 < kBiasRows ? M - r0 : kBiasRows);
+    // the channels from blockIdx.y * kBiasThreads, one per thread
+    const int c0 = blockIdx.y * kBiasThreads, cn = C - c0 < kBiasThreads ? C - c0 : kBiasThreads;
+    const int tr = kBiasTile / cn, tiles = (rows + tr - 1) / tr;
+    const bf16* src = dy + r0 * C + c0;
+    auto load = [&](int t) {
+        bf16* dst = sm[t & 1];
+        const int n = rows - t * tr < tr ? rows - t * tr : tr;
+        if constexpr (VEC) {
+            const int g8 = cn / 8;
+            for (int e = threadIdx.x; e < n * g8; e += kBiasThreads) {
+                const int r = e / g8, g = e - r * g8;
+                tc::cp_async16(dst + (size_t)e * 8, src + (long long)(t * tr + r) * C + g * 8, true);
+            }
+        } else {
+            for (int e = threadIdx.x; e < n * cn; e += kBiasThreads) {
+                const int r = e / cn, c = e - r * cn;
+                dst[e] = src[(long long)(t * tr + r) * C + c];
+            }
         }
+        tc::cp_async_commit();
+    };
+    float s = 0.f;
+    load(0);
+    for (int t = 0; t < tiles; t++) {
+        if (t + 1 < tiles) load(t + 1);
+        else tc::cp_async_commit();
+        tc::cp_async_wait<1>();
+        __syncthreads();
+        const int n = rows - t * tr < tr ? rows - t * tr : tr;
+        if ((int)threadIdx.x < cn) {
+            const bf16* p = sm[t & 1] + threadIdx.x;
+#pragma unroll 16
+            for (int r = 0; r < n; r++) s += __bfloat162float(p[r * cn]);
+        }
+        __syncthreads();
     }
-#pragma unroll
-    for (int k = 0; k < V; k++) sm[threadIdx.x][k] = s[k];
-    __syncthreads();
-    for (int c = threadIdx.x; c < gn * V; c += kBiasThreads) {
-        float t = 0.f;
-        for (int q = 0; q < R; q++) t += sm[q * gn + c / V][c % V];
-        part[(long long)blockIdx.x * C + (size_t)g0 * V + c] = t;
-    }
+    if ((int)threadIdx.x < cn) part[(long long)blockIdx.x * C + c0 + threadIdx.x] = s;
 }
 
 __global__ void k_weight_flip(const bf16* __restrict__ w, int Cin, int Cout, bf16* __restrict__ wt) {
@@ -267,7 +277,7 @@ namespace nn {
 int conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt, const float* bias, int cout, int relu,
            int wrap, void* y, float* y32, cudaStream_t s);
 float* chunk_scratch(size_t floats);
-int sum_chunks(const float* part, long long chunks, long long E, float* dst, cudaStream_t s);
+int sum_few(const float* part, long long chunks, long long E, float* dst, cudaStream_t s);
 int wgrad_tc(const void* x, const void* dy, int n, int d, int h, int w, int cin, int cout, int wrap, float* dw,
              cudaStream_t s);
 }  // namespace nn
@@ -296,24 +306,17 @@ extern "C" int lbm_nn_conv3d_wgrad(const void* x, const void* dy, int n, int d, 
     int rc = wgrad_tc(x, dy, n, d, h, w, cin, cout, wrap, dw, S(stream));
     const long long M = (long long)n * d * h * w;
     if (rc || !dbias) return rc;
-    // two blocks per SM, and at least 64 rows each
-    long long rpb = (M + 303) / 304;
-    if (rpb < 64) rpb = 64;
-    const long long nb = (M + rpb - 1) / rpb;
+    const long long nb = (M + kBiasRows - 1) / kBiasRows;
     float* part = chunk_scratch((size_t)nb * cout);  // the weight gradient's sums are already in dw
     if (!part) return fail(LBM_ERR_OOM, "bias-gradient partial sums");
-    auto bias = [&](auto V, auto kern) {
-        const int G = cout / decltype(V)::value;
-        kern<<<dim3((unsigned)nb, (unsigned)((G + kBiasThreads - 1) / kBiasThreads)), kBiasThreads, 0, S(stream)>>>(
-            static_cast<const bf16*>(dy), M, cout, part, rpb);
-    };
-    // the widest load that every row's channels allow (row starts are C values apart)
-    const uintptr_t at = reinterpret_cast<uintptr_t>(dy);
-    if (cout % 8 == 0 && at % 16 == 0) bias(std::integral_constant<int, 8>{}, k_bias_grad<8>);
-    else if (cout % 4 == 0 && at % 8 == 0) bias(std::integral_constant<int, 4>{}, k_bias_grad<4>);
-    else bias(std::integral_constant<int, 1>{}, k_bias_grad<1>);
+    const dim3 grid((unsigned)nb, (unsigned)((cout + kBiasThreads - 1) / kBiasThreads));
+    // 16-byte copies where every row's channels allow them (row starts are cout values apart)
+    if (cout % 8 == 0 && reinterpret_cast<uintptr_t>(dy) % 16 == 0)
+        k_bias_grad<true><<<grid, kBiasThreads, 0, S(stream)>>>(static_cast<const bf16*>(dy), M, cout, part);
+    else
+        k_bias_grad<false><<<grid, kBiasThreads, 0, S(stream)>>>(static_cast<const bf16*>(dy), M, cout, part);
     rc = check(cudaGetLastError(), "k_bias_grad launch");
-    return rc ? rc : sum_chunks(part, nb, cout, dbias, S(stream));
+    return rc ? rc : sum_few(part, nb, cout, dbias, S(stream));
 }
 
 extern "C" int lbm_nn_relu_mask(void* g, const void* act, size_t count, void* stream) {

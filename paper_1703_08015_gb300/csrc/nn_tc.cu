@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 #include "lbm_nn.h"
@@ -133,15 +134,15 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const bf16* __restrict__ A, con
     tc_pipeline(smem, mbar, &tmem_slot, N, K / TC_BK, fill, out);
 }
 
-// 16 output channels from co0 of one voxel: bias, ReLU, and the stores that the
-// tensors allow (vy: 16 bytes of y, vy32: 16 bytes of y32, else value by value);
+// 16 output channels from co0 of one voxel: their bias (in shared memory), ReLU,
+// and the stores that the tensors allow (vy: 16 bytes of y, vy32: 16 bytes of y32, else value by value);
 // `at`: offset of (voxel, co0).  NaN where the sums are not there.
-__device__ __forceinline__ void conv_out(float (&v)[16], bool ok, const float* __restrict__ bias, int relu, int co0,
+__device__ __forceinline__ void conv_out(float (&v)[16], bool ok, const float* bias, int relu, int co0,
                                          int Cout, size_t at, bool vy, bool vy32, bf16* __restrict__ y,
                                          float* __restrict__ y32) {
 #pragma unroll
     for (int k = 0; k < 16; k++) {
-        v[k] = ok ? v[k] + (bias && co0 + k < Cout ? __ldg(bias + co0 + k) : 0.f) : __int_as_float(0x7fc00000);
+        v[k] = ok ? v[k] + bias[k] : __int_as_float(0x7fc00000);
         if (relu) v[k] = fmaxf(v[k], 0.f);
     }
     if (y && vy) {
@@ -189,9 +190,7 @@ __device__ __forceinline__ int tc_nb(int c, int d, int n, bool wrap) {
 // aligned) or 1.  Rows k >= 27 Cin of the last stage are zero; `n_stages` stages
 // are reserved.
 //
-// Bound by the latency of the gathers and of a block's start: at the network's
-// 2-channel input a block has one stage, and as many blocks as shared memory
-// holds overlap.
+// Bound by the addresses and the latency of the gathers.
 template <int G>
 __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ x, int N, int D, int H, int W, int Cin,
                                                  const bf16* __restrict__ wgt, const float* __restrict__ bias,
@@ -207,6 +206,8 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ x, int
     const bool wx = wrap & 1, wy = wrap & 2, wz = wrap & 4;
     // voxel (n, z, y, x) of each of the block's rows (n < 0: past the end)
     __shared__ int4 vox[TC_M];
+    __shared__ float sbias[128];
+    sbias[threadIdx.x] = bias && n0 + (int)threadIdx.x < Cout ? bias[n0 + threadIdx.x] : 0.f;
     {
         const long long p = m0 + threadIdx.x;
         int4 c = make_int4(-1, 0, 0, 0);
@@ -284,7 +285,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ x, int
         const long long row = m0 + r;
         const int co0 = n0 + c0;
         if (row >= M || co0 >= Cout) return;
-        conv_out(v, ok, bias, relu, co0, Cout, (size_t)row * Cout + co0, vy, vy32, y, y32);
+        conv_out(v, ok, sbias + c0, relu, co0, Cout, (size_t)row * Cout + co0, vy, vy32, y, y32);
     };
     tc_pipeline(smem, mbar, &tmem_slot, NT, (K + TC_BK - 1) / TC_BK, fill, out);
 }
@@ -407,17 +408,19 @@ __device__ __forceinline__ void fill_halo(unsigned char* dst, const HaloAxes& ax
 // nt = 32 (an MMA of 128 x N x 16 takes max(N / 2, 32 + N / 4) cycles), beyond
 // that the MMAs.  Before and after (blocks of up to four planes that copied,
 // multiplied and stored in turn, 27 MMAs per plane): 48 -> 16 channels on 8 x
-// 64^3 voxels 639 and 220 us, 96 -> 32 on 8 x 32^3 292 and 101, 192 -> 64 on 8 x
-// 16^3 149 and 58, 192 -> 128 on 8 x 48^3 6411 and 1335.
+// 64^3 voxels 639 and 216 us, 96 -> 32 on 8 x 32^3 292 and 87, 192 -> 64 on 8 x
+// 16^3 149 and 50, 192 -> 128 on 8 x 48^3 6411 and 1304; 16 -> 16 on 8 x 64^3,
+// bound by its outputs, 136 and 134.
 //
 // Blocks are persistent: each keeps one tile of output channels and walks over
 // bricks.  One warp issues the MMAs, eight copy the planes (the stages that
 // shared memory holds in flight), one the weights (bulk copies, slot by slot as
-// the last plane of a chunk releases them), four write the outputs of the
-// brick before from the other of two accumulator sets.
+// the last plane of a chunk releases them), eight write the outputs plane by
+// plane as they complete, while the next brick uses the other of two accumulator
+// sets.
 constexpr int CV_STAGES = 8;
 constexpr int CV_CC = 64;    // input channels per chunk
-constexpr int CV_EPI = 128;  // output threads (four warps)
+constexpr int CV_EPI = 256;  // output threads (two warps per TMEM lane quadrant)
 constexpr int CV_THREADS = 32 + CV_EPI + FILL_THREADS + 32;
 
 struct CvShape {
@@ -508,7 +511,8 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
                                                              float* __restrict__ y32) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ HaloAxes axes[2];
-    __shared__ uint64_t full[CV_STAGES], empty[CV_STAGES], wfull[9], wempty[9], accf[2], acce[2];
+    __shared__ uint64_t full[CV_STAGES], empty[CV_STAGES], wfull[9], wempty[9], accf[2][HMB_MAX], acce[2];
+    __shared__ float sbias[64];
     __shared__ uint32_t tmem_slot;
     __shared__ int stop[2];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -516,6 +520,10 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
     const long long tiles = (long long)N * BZ * BY * BX;
     unsigned char* const ring = smem + 9 * sh.slot_bytes;
     if (warp == 0) tc::tmem_alloc(&tmem_slot, sh.ncols);
+    if (tid >= 64 && tid < 128) {
+        const int co = blockIdx.y * sh.nt + tid - 64;
+        sbias[tid - 64] = bias && co < Cout ? bias[co] : 0.f;
+    }
     if (tid == 0) {
         for (int s = 0; s < sh.stages; s++) {
             tc::mbar_init(&full[s], FILL_THREADS / 32);
@@ -526,7 +534,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
             tc::mbar_init(&wempty[t], 1);
         }
         for (int s = 0; s < 2; s++) {
-            tc::mbar_init(&accf[s], 1);
+            for (int m = 0; m < sh.mb; m++) tc::mbar_init(&accf[s][m], 1);
             tc::mbar_init(&acce[s], CV_EPI / 32);
         }
         stop[0] = stop[1] = 0;
@@ -584,11 +592,12 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
                                          c == 0 && t9 == 0);
                         }
                         __syncwarp();
+                        // output plane hz - 2 is complete (with the last one, those that the brick lacks)
+                        if (c == sh.chunks - 1 && hz >= 2 && tc::elect_one())
+                            for (int m = hz - 2; m < (hz == nz + 1 ? sh.mb : hz - 1); m++) tc::mma_commit(&accf[buf][m]);
+                        __syncwarp();
                     }
-                    if (tc::elect_one()) {
-                        tc::mma_commit(&empty[s]);
-                        if (c == sh.chunks - 1 && h1 == nz + 2) tc::mma_commit(&accf[buf]);
-                    }
+                    if (tc::elect_one()) tc::mma_commit(&empty[s]);
                     __syncwarp();
                     if (++s == sh.stages) s = 0, ph ^= 1;
                 }
@@ -596,24 +605,25 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
             }
         }
     } else if (warp <= CV_EPI / 32) {
-        const int quad = warp & 3, r = quad * 32 + lane;
+        const int quad = warp & 3, half = (warp - 1) >> 2, r = quad * 32 + lane;
         int it = 0;
         for (long long t = blockIdx.x; t < tiles; t += gridDim.x, it++) {
             const Brick b = brick_at(t, BX, BY, BZ, sh.mb);
             const int nz = D - b.z0 < sh.mb ? D - b.z0 : sh.mb, buf = it & 1;
-            // once a wait has run out: NaN for this and the remaining bricks
-            if (ok) ok = __all_sync(0xffffffffu, tc::mbar_wait(&accf[buf], (it >> 1) & 1, TC_WAIT));
-            tc::fence_after_sync();
             const int vx = b.x0 + (r & 7), vy_ = b.y0 + (r >> 3);
             const bool inside = vx < W && vy_ < H;
-            for (int q = 0; q < nz * sh.nt; q += 16) {  // plane q / nt, its columns q % nt ..
-                __syncwarp();
-                const int m = q / sh.nt, co0 = blockIdx.y * sh.nt + q - m * sh.nt;
-                float v[16];
-                tc::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * sh.mb * sh.nt + q), v);
-                if (inside && co0 < Cout)
-                    conv_out(v, ok, bias, relu, co0, Cout, ((((size_t)b.n * D + b.z0 + m) * H + vy_) * W + vx) * Cout + co0, vy,
-                             vy32, y, y32);
+            for (int m = half; m < nz; m += 2) {
+                // once a wait has run out: NaN for this and the remaining planes
+                if (ok) ok = __all_sync(0xffffffffu, tc::mbar_wait(&accf[buf][m], (it >> 1) & 1, TC_WAIT));
+                tc::fence_after_sync();
+                const size_t at = ((((size_t)b.n * D + b.z0 + m) * H + vy_) * W + vx) * Cout;
+                for (int q = 0; q < sh.nt; q += 16) {
+                    __syncwarp();
+                    const int co0 = blockIdx.y * sh.nt + q;
+                    float v[16];
+                    tc::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)((buf * sh.mb + m) * sh.nt + q), v);
+                    if (inside && co0 < Cout) conv_out(v, ok, sbias + q, relu, co0, Cout, at + co0, vy, vy32, y, y32);
+                }
             }
             tc::fence_before_sync();
             __syncwarp();
@@ -708,138 +718,253 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
     }
 }
 
+// ---- the 3x3x3 convolution of two or four input channels ---------------------
+//
+// The implicit GEMM of k_conv_tc, k = (tap, ci), where 27 CI fits one operand
+// tile: a block copies the halo of a column of 8 x 16 x FEW_Z voxels once, and
+// each thread puts one voxel's row together from it, plane by plane.  Bound by
+// the chain of a plane (rows, MMAs, outputs), which as many blocks as an SM
+// holds overlap; k_conv_tc spent it on the addresses of 27 CI separate loads per
+// voxel: 2 -> 16 channels on 8 x 64^3 voxels 334 and 53 us, 4 -> 16
+// 615 and 86.
+constexpr int FEW_Z = 8;
+__host__ __device__ constexpr int few_groups(int ci) { return (27 * ci + 15) / 16 * 2; }  // 8-value groups of a row
+__host__ __device__ constexpr uint32_t few_smem(int ci, int nt) {
+    return (uint32_t)((TC_M + nt) * few_groups(ci) * 16 + (FEW_Z + 2) * HPLANE * 2 * ci);
+}
+
+template <int CI>
+__global__ void __launch_bounds__(TC_M) k_conv_few(const bf16* __restrict__ x, int N, int D, int H, int W,
+                                                   const bf16* __restrict__ wgt, const float* __restrict__ bias, int Cout,
+                                                   int nt, int relu, int wrap, bool vy, bool vy32, bf16* __restrict__ y,
+                                                   float* __restrict__ y32) {
+    static_assert(CI == 2 || CI == 4, "a cell of 4 or 8 bytes");
+    using Cell = typename std::conditional<CI == 2, uint32_t, uint2>::type;
+    constexpr int KG = few_groups(CI), K = 27 * CI;
+    constexpr uint32_t RGAP = KG * 128;
+    extern __shared__ __align__(128) unsigned char smem[];
+    unsigned char* const sb = smem + TC_M * KG * 16;
+    Cell* const halo = reinterpret_cast<Cell*>(sb + nt * KG * 16);
+    __shared__ uint64_t mbar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ float sbias[64];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n0 = blockIdx.y * nt;
+    uint32_t ncols = 32;
+    while (ncols < (uint32_t)nt) ncols <<= 1;
+    if (warp == 0) tc::tmem_alloc(&tmem_slot, ncols);
+    if (tid == 0) tc::mbar_init(&mbar, 1);
+    if (tid < 64) sbias[tid] = bias && n0 + tid < Cout ? bias[n0 + tid] : 0.f;
+    const unsigned short* wv = reinterpret_cast<const unsigned short*>(wgt);
+    for (int e = tid; e < nt * KG; e += TC_M) {
+        const int c = e % nt, g = e / nt, co = n0 + c;
+        unsigned short h[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) h[k] = g * 8 + k < K && co < Cout ? __ldg(wv + (size_t)(g * 8 + k) * Cout + co) : 0;
+        *reinterpret_cast<uint4*>(sb + tc::tile_off(c, g, TC_KGAP, RGAP)) =
+            make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
+                       h[6] | (uint32_t)h[7] << 16);
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = tmem_slot, idesc = tc::idesc_bf16_f32(TC_M, nt);
+    const int BX = (W + 7) / 8, BY = (H + 15) / 16, BZ = (D + FEW_Z - 1) / FEW_Z;
+    const long long tiles = (long long)N * BZ * BY * BX;
+    const int lx = tid & 7, ly = tid >> 3;
+    bool ok = true;
+    uint32_t ph = 0;
+    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const Brick b = brick_at(t, BX, BY, BZ, FEW_Z);
+        const int nz = D - b.z0 < FEW_Z ? D - b.z0 : FEW_Z;
+#pragma unroll 4
+        for (int e = tid; e < (nz + 2) * HPLANE; e += TC_M) {
+            const int hx = e % HX, hy = e / HX % HY, hz = e / HPLANE;
+            const int xx = halo_nb(b.x0 + hx - 1, W, wrap & 1), yy = halo_nb(b.y0 + hy - 1, H, wrap & 2),
+                      zz = halo_nb(b.z0 + hz - 1, D, wrap & 4);
+            Cell v{};
+            if ((xx | yy | zz) >= 0)
+                v = __ldg(reinterpret_cast<const Cell*>(x) + (((long long)b.n * D + zz) * H + yy) * W + xx);
+            halo[e] = v;
+        }
+        __syncthreads();
+        const int vx = b.x0 + lx, vy_ = b.y0 + ly;
+        for (int z = 0; z < nz; z++) {
+            Cell w[KG * 8 / CI];
+#pragma unroll
+            for (int k = 0; k < KG * 8 / CI; k++)
+                w[k] = k < 27 ? halo[((z + k / 9) * HY + ly + k / 3 % 3) * HX + lx + k % 3] : Cell{};
+#pragma unroll
+            for (int g = 0; g < KG; g++) {
+                uint4 u;
+                if constexpr (CI == 2) u = make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
+                else u = make_uint4(w[2 * g].x, w[2 * g].y, w[2 * g + 1].x, w[2 * g + 1].y);
+                *reinterpret_cast<uint4*>(smem + tc::tile_off(tid, g, TC_KGAP, RGAP)) = u;
+            }
+            tc::fence_smem_to_async();
+            __syncthreads();
+            if (tid == 0) {
+                tc::fence_after_sync();
+                const uint32_t a0 = tc::smem_u32(smem), b0 = tc::smem_u32(sb);
+#pragma unroll
+                for (int j = 0; j < KG / 2; j++)
+                    tc::mma_bf16(tmem, tc::smem_desc(a0 + 2 * j * TC_KGAP, TC_KGAP, RGAP),
+                                 tc::smem_desc(b0 + 2 * j * TC_KGAP, TC_KGAP, RGAP), idesc, j > 0);
+                tc::mma_commit(&mbar);
+            }
+            if (ok) ok = __all_sync(0xffffffffu, tc::mbar_wait(&mbar, ph, TC_WAIT));
+            ph ^= 1;
+            tc::fence_after_sync();
+            const size_t at = ((((size_t)b.n * D + b.z0 + z) * H + vy_) * W + vx) * Cout;
+            for (int q = 0; q < nt; q += 16) {
+                float v[16];
+                __syncwarp();
+                tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)q, v);
+                if (vx < W && vy_ < H && n0 + q < Cout)
+                    conv_out(v, ok, sbias + q, relu, n0 + q, Cout, at + n0 + q, vy, vy32, y, y32);
+            }
+            tc::fence_before_sync();
+            __syncthreads();  // the rows and the accumulator are free
+            tc::fence_after_sync();
+        }
+    }
+    if (!ok && lane == 0) atomicAdd(&g_tc_timeouts, 1u);
+    if (warp == 0) tc::tmem_dealloc(tmem, ncols);
+}
+
 // ---- weight gradient on the tensor cores ------------------------------------
 //
 // dw[tap][ci][co] = sum_p x[p + off(tap)][ci] dy[p][co]: GEMMs that reduce over
-// voxels, with both operands read by the tensor cores where the channels-last
-// tensors put them.  A stage holds one brick of 8 (x) x 16 (y) x MB (z) voxels:
-// a halo tile of x, 10 x 18 x (MB + 2) cells of 8 channels (16 bytes) laid out
-// [z][channel group][y][x], and the brick of dy laid out [channel
-// group][z][y][x].  8 consecutive cells along x are one core matrix of an
-// MN-major operand (8 voxels of K by 8 channels), so no transposed or shifted
-// copy is made: a tap is a start address.  Planes (z, channel group) are one
-// stride apart, so the groups from z plane m on are the rows (dz, ci) of all
-// three dz taps of output plane m: one MMA of K = 16 (8 x by 2 y voxels) gives
-// the sums of 3 cc (dz, ci) rows by NT output channels for one (dy, dx), into
-// that tap's TMEM columns.  (Rows past 3 cc groups read whatever lies behind;
-// their sums are not used.)  Eight warps copy the stages, one issues the MMAs,
-// two stages in flight; each block keeps its sums over all of its bricks in
-// TMEM and stores them once.
+// the positions of a padded grid, (D + 2) x (H + 2) x Wp with Wp >= W + 2 a
+// multiple of 8: position q holds x at q minus one voxel on each axis (wrapped
+// on periodic axes, zero outside) and dy at interior positions (zero on the
+// padding), so a tap is a shift of q by (dz Hp + dy) Wp + dx.  Both operands
+// are read by the tensor cores where the channels-last tensors put them: a
+// stage holds T consecutive positions as cells of 8 channels (16 bytes), dy as
+// [channel group][q], x as [dz][channel group][q] with the rows that the dy and
+// dx shifts reach (one window of T + 2 Wp + 2 cells, or three of T + 2 for the
+// dy of wide rows).  8 consecutive cells are one core matrix of an MN-major
+// operand (8 positions of K by 8 channels): no transposed or shifted copy is
+// made, a tap is a start address.  The (dz, channel group) planes are one stride
+// apart, so one MMA of K = 16 positions gives the sums of 3 cc (dz, ci) rows by
+// NT output channels for one (dy, dx), into that tap's TMEM columns.  (Rows past
+// 3 cc read whatever lies behind; their sums are not used.)  Sixteen warps copy
+// the stages, one issues the MMAs; each block keeps its sums over its chunk of
+// positions in TMEM and stores them once.  Stages without an interior row are left
+// out.
 //
 // What bounds it: the tensor cores' reads of the 128 or 64 (dz, ci) rows from
-// shared memory, once per (dy, dx): an MMA of 64 x 16 x 16 takes 23 cycles, of
-// 128 x 32 x 16 40.  With operands packed channel-major in memory (three copies
-// of x) a layer wrote and read 4 to 8 times its tensors: 16 -> 16 channels on 8
-// x 64^3 voxels 1082 us, now 134; 48 -> 16 2636, now 430; 96 -> 32 on 8 x 32^3
-// 914, now 137; 192 -> 128 on 8 x 48^3 5012, now 3710; and 2 -> 16 on 8 x 64^3
-// (gathered for mma.sync, 1275) 160.
-constexpr int WG_THREADS = FILL_THREADS + 32;  // the copying warps and the one that issues the MMAs
+// shared memory, once per (dy, dx) (an MMA of 64 x 16 x 16 takes 23 cycles, of
+// 128 x 32 x 16 40), and the copies of x, three or more for its halo.
+// With operands packed channel-major in memory (three copies of x) a layer wrote
+// and read 4 to 8 times its tensors: 16 -> 16 channels on 8 x 64^3 voxels 1082
+// us, now 157; 48 -> 16 2636, now 417; 96 -> 32 on 8 x 32^3 914, now 181; 192 ->
+// 128 on 8 x 48^3 5012, now 4102; 2 -> 16 on 8 x 64^3 (gathered for mma.sync,
+// 1275) 189.
+constexpr int WG_FILL = 512;               // copying threads (16 warps)
+constexpr int WG_THREADS = WG_FILL + 32;  // and the warp that issues the MMAs
 constexpr int WG_STAGES = 4;
+constexpr int WG_T = 512;                // positions of a stage, at most
+constexpr int WG_ROWS = WG_T / 8 + 6;    // rows of the padded grid that a stage reaches, at most
 
 // Shape of one launch, shared by the host and the kernel.
 struct WgShape {
     int cc;       // input channels per block: 8, 16 or 32
     int ncg;      // cc / 8
     int nt;       // output channels per block: 16, 32 or 48
-    int mb;       // z planes of a brick
-    int stages;   // bricks in flight: 2 .. WG_STAGES
+    int T;        // positions of a stage: a multiple of 64
+    int win;      // windows of x: 1, or 3 (one per dy)
+    int len;      // cells of a window
     int plane;    // cells from one (z, channel group) plane of the x tile to the next
-    int gstride;  // cells from one channel group of the dy brick to the next
+    int gstride;  // cells from one channel group of the dy tile to the next
+    int stages;   // 2 .. WG_STAGES
     uint32_t a_bytes, stage_bytes, smem, ncols;
 };
 
 // Output tiles of at most 48 channels, whose nine (dy, dx) accumulators fit the
-// 512 TMEM columns (64 channels in two groups of taps filled every stage twice:
-// 192 -> 128 channels on 8 x 48^3 voxels 3.9 ms).  Input channels per block: 32
-// (rows 3 * 32 of 128), or 16 (3 * 16 of 64) up to 32 output channels, where the
-// MMA of 64 rows takes little more than half the time (24 against 40 cycles) and
-// twice as many blocks fill the chip.  The plane and group strides put the
-// 16-byte cells that a warp stores together (channel groups fastest) into
-// different banks.
-__host__ __device__ inline WgShape wg_shape(int cin, int cout, int mb_max) {
-    WgShape s;
+// 512 TMEM columns.  Input channels per block: 32 (rows 3 * 32 of 128), or 16
+// (3 * 16 of 64) up to 32 output channels, where the MMA of 64 rows takes little
+// more than half the time (24 against 40 cycles) and twice as many blocks fill
+// the chip.  Of the stage lengths and windows of which two stages fit, the one
+// that copies least per position.  The plane and group strides put the 16-byte
+// cells that a warp stores together (channel groups fastest) into different
+// banks.
+static WgShape wg_shape(int cin, int cout, int Wp) {
+    WgShape best{};
+    double least = 0;
     const int mt = (cout + 47) / 48;
-    s.nt = ((cout + mt - 1) / mt + 15) / 16 * 16;
-    s.cc = cin <= 8 ? 8 : (cin <= 16 || cout <= 32 || (cin % 32 && cin % 32 <= 16) ? 16 : 32);
-    s.ncg = s.cc / 8;
-    s.plane = s.ncg == 4 ? HPLANE + 6 : HPLANE;  // 8 / ncg mod 8 cells
-    uint32_t tail = 0;
-    for (s.mb = mb_max;; s.mb--) {  // the deepest brick of which two fit (one plane: they do)
-        s.gstride = s.mb * 128 + (s.nt == 16 ? 4 : (s.nt == 32 ? 2 : 1));
-        s.a_bytes = (uint32_t)((s.mb + 2) * s.ncg * s.plane) * 16;
-        const uint32_t g_bytes = (uint32_t)(s.nt / 8 * s.gstride) * 16;
-        s.stage_bytes = (s.a_bytes + g_bytes + 127) / 128 * 128;
-        // the unused rows of the last plane's MMAs reach past the x tile
-        const int over = (s.mb - 1) * s.ncg + (3 * s.ncg > 8 ? 16 : 8) - (s.mb + 2) * s.ncg;
-        const uint32_t over_bytes = over > 0 ? (uint32_t)(over * s.plane) * 16 : 0;
-        tail = over_bytes > g_bytes ? over_bytes - g_bytes : 0;
-        s.stages = (int)((224u * 1024u - tail) / s.stage_bytes);
-        if (s.stages >= 2 || s.mb == 1) break;
-    }
-    if (s.stages > WG_STAGES) s.stages = WG_STAGES;
-    s.smem = (uint32_t)s.stages * s.stage_bytes + tail;
-    s.ncols = 32;
-    while ((int)s.ncols < 9 * s.nt) s.ncols <<= 1;
-    return s;
-}
-
-// The MMAs of one stage: nz planes, ny2 pairs of lines, nine (dy, dx); called by
-// one lane.
-__device__ __forceinline__ void wg_issue(uint32_t tmem, uint64_t a0, uint64_t g0, int nz, int ny2, uint32_t aplane,
-                                         int nt, uint32_t idesc, bool first) {
-    for (int m = 0; m < nz; m++) {
-        for (int y2 = 0; y2 < ny2; y2++) {
-            const uint64_t a = a0 + (uint64_t)(m * aplane + (uint32_t)y2 * (2 * HX));
-            const uint64_t g = g0 + (uint64_t)(m * 128 + y2 * 16);
-            const bool acc = !(first && m == 0 && y2 == 0);
-#pragma unroll
-            for (int t = 0; t < 9; t++)
-                tc::mma_bf16(tmem + (uint32_t)(t * nt), a + (uint64_t)((t / 3) * HX + t % 3), g, idesc, acc);
+    for (int T = WG_T; T >= 64; T -= 64)
+        for (int win = 1; win <= 3; win += 2) {
+            WgShape s;
+            s.nt = ((cout + mt - 1) / mt + 15) / 16 * 16;
+            s.cc = cin <= 8 ? 8 : (cin <= 16 || cout <= 32 || (cin % 32 && cin % 32 <= 16) ? 16 : 32);
+            s.ncg = s.cc / 8;
+            s.T = T;
+            s.win = win;
+            const long long len = T + 2 + (win == 1 ? 2ll * Wp : 0);
+            if (len > 8192) continue;
+            s.len = (int)len;
+            const int at = s.ncg == 4 ? 2 : (s.ncg == 2 ? 4 : 0);
+            s.plane = (s.len + 7 - at) / 8 * 8 + at;
+            s.gstride = T + (s.nt == 16 ? 4 : (s.nt == 32 ? 2 : 1));
+            s.a_bytes = (uint32_t)(win * 3 * s.ncg * s.plane) * 16;
+            const uint32_t g_bytes = (uint32_t)(s.nt / 8 * s.gstride) * 16;
+            s.stage_bytes = (s.a_bytes + g_bytes + 127) / 128 * 128;
+            // the unused rows of an MMA reach past the last window's planes
+            const uint32_t over = (uint32_t)(((3 * s.ncg > 8 ? 16 : 8) - 3 * s.ncg) * s.plane) * 16;
+            const uint32_t tail = over > g_bytes ? over - g_bytes : 0;
+            if (tail >= 220u * 1024u) continue;
+            s.stages = (int)((220u * 1024u - tail) / s.stage_bytes);
+            if (s.stages < 2) continue;
+            if (s.stages > WG_STAGES) s.stages = WG_STAGES;
+            s.smem = (uint32_t)s.stages * s.stage_bytes + tail;
+            s.ncols = 32;
+            while ((int)s.ncols < 9 * s.nt) s.ncols <<= 1;
+            const double cost = (3.0 * win * s.ncg * s.len + s.nt / 8.0 * T + 400.0) / T;  // cells copied, and a stage's overhead
+            if (least == 0 || cost < least) least = cost, best = s;
         }
+    return best;
+}
+
+// The MMAs of one stage: ks K steps, nine (dy, dx) each (dy steps `dyoff`
+// descriptor units apart); called by one lane.
+__device__ __forceinline__ void wg_issue(uint32_t tmem, uint64_t a0, uint64_t g0, int ks, uint32_t dyoff, int nt,
+                                         uint32_t idesc, bool first) {
+    for (int k = 0; k < ks; k++) {
+        const uint64_t a = a0 + (uint64_t)(k * 16), g = g0 + (uint64_t)(k * 16);
+        const bool acc = !first || k > 0;
+#pragma unroll
+        for (int t = 0; t < 9; t++)
+            tc::mma_bf16(tmem + (uint32_t)(t * nt), a + (uint64_t)((t / 3) * dyoff + t % 3), g, idesc, acc);
     }
 }
 
-// First brick of voxel chunk c of `chunks`: where equal parts of the box padded
-// by one voxel on each side (rows by W + 2 and up to a multiple of 8, in units
-// of 64 voxels) begin.  The accumulators truncate, so where a chunk begins is
-// part of the result's rounding: chunks of equal bricks would move the
-// gradient's last bits as far as a different number of chunks does.
-__host__ __device__ inline long long wg_chunk_begin(long long c, long long chunks, long long tiles, int N, int D, int H,
-                                                    int W) {
-    const long long Wp = (W + 2 + 7) / 8 * 8, Hp = H + 2, Dp = D + 2;
-    const long long steps = (N * Dp * Hp * Wp + 63) / 64, line = c * ((steps + chunks - 1) / chunks) * 64 / Wp;
-    const long long n = line / (Hp * Dp), zp = line / Hp % Dp, yp = line % Hp;
-    if (c >= chunks || n >= N) return tiles;
-    // lines of the box before it
-    const long long z = zp < 1 ? 0 : (zp > D ? D : zp - 1), y = zp < 1 || zp > D ? 0 : (yp < 1 ? 0 : (yp > H ? H : yp - 1));
-    return tiles * ((n * D + z) * H + y) / ((long long)N * D * H);
-}
-
-// Grid: x = voxel chunks (consecutive bricks), y = input-channel
-// chunks, z = output-channel tiles.  part[blockIdx.x][tap][ci][co]
-// takes the block's sums (NaN when a wait ran out); k_sum_chunks adds the
-// chunks to dw in a fixed order, so the gradient does not depend on the order
-// in which blocks finish.
+// Grid: x = chunks of spc * 64 positions, y = input-channel chunks, z =
+// output-channel tiles.  part[blockIdx.x][tap][ci][co] takes the block's sums
+// (NaN when a wait ran out); k_sum_chunks adds the chunks to dw in order, so the
+// gradient does not depend on the order in which blocks finish.
 template <bool VX, bool VG>
-__global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict__ x, const bf16* __restrict__ dy, int N,
-                                                         int D, int H, int W, int Cin, int Cout, int wrap, WgShape sh,
-                                                         float* __restrict__ part) {
+__global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad_tc(const bf16* __restrict__ x, const bf16* __restrict__ dy, int N,
+                                                            int D, int H, int W, int Cin, int Cout, int wrap, int Wp,
+                                                            long long nsteps, long long spc, WgShape sh,
+                                                            float* __restrict__ part) {
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ HaloAxes axes[2];
+    // sources of the padded grid's rows near a stage: x for each dz, dy (null: zeros)
+    __shared__ const bf16* xrow[2][3][WG_ROWS];
+    __shared__ const bf16* grow[2][WG_ROWS];
+    __shared__ int used[WG_STAGES];  // the stage holds an interior row
     __shared__ uint64_t full[WG_STAGES], empty[WG_STAGES], done;
     __shared__ uint32_t tmem_slot;
     __shared__ int failed, stop[2];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int c0 = blockIdx.y * sh.cc;
     const int n0 = blockIdx.z * sh.nt;
-    const int BX = (W + 7) / 8, BY = (H + 15) / 16, BZ = (D + sh.mb - 1) / sh.mb;
-    const long long tiles = (long long)N * BZ * BY * BX;
-    const long long tile_begin = wg_chunk_begin(blockIdx.x, gridDim.x, tiles, N, D, H, W),
-                    tile_end = wg_chunk_begin(blockIdx.x + 1, gridDim.x, tiles, N, D, H, W);
+    const int Hp = H + 2, Dp = D + 2;
+    const long long begin = blockIdx.x * spc * 64, last_step = (blockIdx.x + 1) * spc,
+                    end = (last_step < nsteps ? last_step : nsteps) * 64;
     if (warp == 0) tc::tmem_alloc(&tmem_slot, sh.ncols);
     if (tid == 0) {
         for (int s = 0; s < sh.stages; s++) {
-            tc::mbar_init(&full[s], FILL_THREADS / 32);
+            tc::mbar_init(&full[s], WG_FILL / 32);
             tc::mbar_init(&empty[s], 1);
         }
         tc::mbar_init(&done, 1);
@@ -850,43 +975,52 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict_
     tc::fence_after_sync();
     const uint32_t tmem = tmem_slot;
     const int rows = 3 * sh.ncg > 8 ? 128 : 64;  // (dz, ci) rows of an MMA
-    bool ok = true;
+    bool ok = true, any = false;                 // any (the issuing warp): the accumulators were written
+    __shared__ int written;
     if (warp == 0) {
         // the waits' results are made uniform over the warp, so that the elected
         // lane's descriptors stay in uniform registers (a lane picked by its
         // index issues an MMA every 45 cycles at best; these need 23 to 48)
         const uint32_t idesc = tc::idesc_bf16_f32(rows, sh.nt) | tc::IDESC_MN_MAJOR;
+        const uint32_t dyoff = (uint32_t)(sh.win == 1 ? Wp : 3 * sh.ncg * sh.plane);
         int s = 0;        // stage
         uint32_t ph = 0;  // its phase
-        bool first = true;
-        for (long long t = tile_begin; t < tile_end; t++) {
+        for (long long q = begin; q < end; q += sh.T) {
             if (!__all_sync(0xffffffffu, tc::mbar_wait(&full[s], ph, TC_WAIT))) {
                 ok = false;
                 break;
             }
             tc::fence_after_sync();
-            const Brick b = brick_at(t, BX, BY, BZ, sh.mb);
-            const int nz = D - b.z0 < sh.mb ? D - b.z0 : sh.mb, ny2 = H - b.y0 < 16 ? (H - b.y0 + 1) / 2 : 8;
             const uint32_t st = tc::smem_u32(smem + s * sh.stage_bytes);
-            const uint64_t a0 = tc::smem_desc(st, HX * 16, (uint32_t)sh.plane * 16);
+            const uint64_t a0 = tc::smem_desc(st, 128, (uint32_t)sh.plane * 16);
             const uint64_t g0 = tc::smem_desc(st + sh.a_bytes, 128, (uint32_t)sh.gstride * 16);
-            const uint32_t ap = (uint32_t)(sh.ncg * sh.plane);
-            if (tc::elect_one()) {
-                wg_issue(tmem, a0, g0, nz, ny2, ap, sh.nt, idesc, first);
-                tc::mma_commit(&empty[s]);
+            const int ks = (int)(end - q < sh.T ? end - q : sh.T) / 16;
+            if (__any_sync(0xffffffffu, used[s])) {
+                if (tc::elect_one()) wg_issue(tmem, a0, g0, ks, dyoff, sh.nt, idesc, !any);
+                __syncwarp();
+                any = true;
             }
+            if (tc::elect_one()) tc::mma_commit(&empty[s]);
             __syncwarp();
-            first = false;
             if (++s == sh.stages) s = 0, ph ^= 1;
         }
         if (tc::elect_one()) tc::mma_commit(&done);
         __syncwarp();
+        if (lane == 0) written = any;
     } else {
         const int ft = tid - 32;
-        // this thread's share of the dy brick: one channel group of every gstep-th voxel
-        const int groups = sh.nt / 8, gstep = FILL_THREADS / groups;
-        const int gcell = ft / groups, gcg = ft - gcell * groups, co = n0 + gcg * 8;
-        int it = 0, s = 0, last = -1;  // bricks so far, stage, the stage copied but not handed over
+        // this thread's channel groups of x and dy, its first position and the step between its positions
+        const int xstep = WG_FILL / sh.ncg, xpos = ft / sh.ncg, xcg = ft - xpos * sh.ncg, ci = c0 + xcg * 8;
+        const int groups = sh.nt / 8, gstep = WG_FILL / groups;
+        const int gpos = ft / groups, gcg = ft - gpos * groups, co = n0 + gcg * 8;
+        const int xsi = xstep / Wp, xsx = xstep - xsi * Wp, gsi = gstep / Wp, gsx = gstep - gsi * Wp;
+        // row and position in it of the segment's start; rows are decoded in 32 bits where they fit
+        long long row0 = begin / Wp;
+        int x0 = (int)(begin - row0 * Wp);
+        const int ti = sh.T / Wp, tx = sh.T - ti * Wp;
+        const long long all_rows = (long long)N * Dp * Hp;
+        const bool small_rows = all_rows < 0x7fffffffll;
+        int it = 0, s = 0, last = -1;  // segments so far, stage, the stage copied but not handed over
         uint32_t ph = 0;
         auto hand_over = [&](int stage) {  // this warp's copies to it have completed
             tc::fence_smem_to_async();
@@ -898,41 +1032,102 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict_
             if (last >= 0) hand_over(last);
             last = -1;
         };
-        for (long long t = tile_begin; t < tile_end; t++, it++) {
-            if (it >= sh.stages) {
-                // the stage is still read: first hand over the one before it
-                if (!__all_sync(0xffffffffu, tc::mbar_test(&empty[s], ph ^ 1))) {
-                    hand_over_all();
-                    // a wait that runs out stops every copying warp behind the barrier of halo_axes
-                    if (!tc::mbar_wait(&empty[s], ph ^ 1, TC_WAIT)) stop[it & 1] = 1;
-                }
+        for (long long q = begin; q < end; q += sh.T, it++) {
+            // with two stages the one before is handed over as soon as it has landed (the MMAs
+            // would otherwise wait for the copies of this one as well), with more at the
+            // latest while this one is still read; a wait that runs out stops every copying
+            // warp behind the barrier below
+            if (sh.stages == 2) hand_over_all();
+            if (it >= sh.stages && !__all_sync(0xffffffffu, tc::mbar_test(&empty[s], ph ^ 1))) {
+                hand_over_all();
+                if (!tc::mbar_wait(&empty[s], ph ^ 1, TC_WAIT)) stop[it & 1] = 1;
             }
-            unsigned char* sa = smem + s * sh.stage_bytes;
-            unsigned char* sg = sa + sh.a_bytes;
-            const Brick b = brick_at(t, BX, BY, BZ, sh.mb);
-            halo_axes(axes[it & 1], ft, x, b, sh.mb, D, H, W, Cin, wrap);
+            const long long rb = row0 - 2;  // first row of the tables
+            const int off = x0 + 2 * Wp;    // the segment's start from there
+            const int nr = (x0 + sh.T - 1) / Wp + 5;
+            for (int e = ft; e < 3 * nr; e += WG_FILL) {
+                const int dz = e / nr, i = e - dz * nr;
+                const long long r = rb + i + (long long)(dz - 1) * Hp;
+                const bf16 *px = nullptr, *pg = nullptr;
+                if (r >= 0 && r < all_rows) {
+                    int yp, zp;
+                    long long n;
+                    if (small_rows) {
+                        const unsigned u = (unsigned)r, v = u / (unsigned)Hp;
+                        yp = (int)(u - v * (unsigned)Hp);
+                        n = v / (unsigned)Dp;
+                        zp = (int)(v - (unsigned)n * (unsigned)Dp);
+                    } else {
+                        yp = (int)(r % Hp);
+                        zp = (int)(r / Hp % Dp);
+                        n = r / Hp / Dp;
+                    }
+                    const int zs = halo_nb(zp - 1, D, wrap & 4), ys = halo_nb(yp - 1, H, wrap & 2);
+                    if ((zs | ys) >= 0) px = x + ((n * D + zs) * H + ys) * (long long)W * Cin;
+                    if (zp >= 1 && zp <= D && yp >= 1 && yp <= H) pg = dy + ((n * D + zp - 1) * H + yp - 1) * (long long)W * Cout;
+                }
+                xrow[it & 1][dz][i] = px;
+                if (dz == 1) grow[it & 1][i] = pg;
+            }
+            asm volatile("bar.sync 1, %0;" ::"n"(WG_FILL) : "memory");
             if (*(volatile int*)&stop[it & 1]) {
                 ok = false;
                 break;
             }
-            fill_halo<VX>(sa, axes[it & 1], x, ft, sh.ncg, 0, sh.mb + 2, sh.plane, c0, Cin);
-            // the brick of dy, zero outside the box and past Cout
-            const bf16* gb = dy + ((((size_t)b.n * D + b.z0) * H + b.y0) * W + b.x0) * Cout + co;
-            const int gx = W - b.x0, gy = H - b.y0, gz = co < Cout ? D - b.z0 : 0;  // limits of the brick
+            // nothing to copy or multiply where no row is interior
+            bool use = false;
+            for (int i = lane; i < nr; i += 32) use |= i >= 2 && i < nr - 2 && grow[it & 1][i] != nullptr;
+            use = __any_sync(0xffffffffu, use);
+            if (ft == 0) used[s] = use;
+            if (use) {
+                unsigned char* sa = smem + s * sh.stage_bytes;
+                unsigned char* sg = sa + sh.a_bytes;
+                const int held = end - q < sh.T ? (int)(end - q) : sh.T, cells = sh.len - (sh.T - held);  // of this segment
+                for (int pl = 0; pl < 3 * sh.win; pl++) {
+                    const int dz = pl % 3;
+                    // position of the window's first cell from the tables' first row
+                    const int rel = off - 1 + (sh.win == 1 ? -Wp : (pl / 3 - 1) * Wp) + xpos;
+                    int i = rel / Wp, xp = rel - i * Wp;
+                    unsigned char* to = sa + (uint32_t)((pl * sh.ncg + xcg) * sh.plane) * 16u;
 #pragma unroll 4
-            for (int cell = gcell < gstep ? gcell : sh.mb * 128; cell < sh.mb * 128; cell += gstep) {
-                const int xx = cell & 7, yy = (cell >> 3) & 15, zz = cell >> 7;
-                const bool get = xx < gx && yy < gy && zz < gz;
-                const bf16* src = gb + (((long long)zz * H + yy) * W + xx) * Cout;
-                unsigned char* to = sg + (uint32_t)(gcg * sh.gstride + cell) * 16u;
-                if constexpr (VG) {
-                    tc::cp_async16(to, get ? src : dy, get);
-                } else {
-                    uint4 v = make_uint4(0, 0, 0, 0);
-                    if (get) v = tc::load8(src, Cout - co);
-                    *reinterpret_cast<uint4*>(to) = v;
+                    for (int e = xpos < xstep ? xpos : cells; e < cells; e += xstep) {
+                        const bf16* row = xrow[it & 1][dz][i];
+                        const int xx = xp > W + 1 ? -1 : halo_nb(xp - 1, W, wrap & 1);
+                        const bool get = row && xx >= 0 && ci < Cin;
+                        const bf16* src = row + (long long)xx * Cin + ci;
+                        if constexpr (VX) {
+                            tc::cp_async16(to + (uint32_t)e * 16u, get ? src : x, get);
+                        } else {
+                            uint4 v = make_uint4(0, 0, 0, 0);
+                            if (get) v = tc::load8(src, Cin - ci);
+                            *reinterpret_cast<uint4*>(to + (uint32_t)e * 16u) = v;
+                        }
+                        xp += xsx;
+                        i += xsi;
+                        if (xp >= Wp) xp -= Wp, i++;
+                    }
+                }
+                const int rel = off + gpos;
+                int i = rel / Wp, xp = rel - i * Wp;
+                unsigned char* to = sg + (uint32_t)(gcg * sh.gstride) * 16u;
+#pragma unroll 4
+                for (int e = gpos < gstep ? gpos : held; e < held; e += gstep) {
+                    const bf16* row = grow[it & 1][i];
+                    const bool get = row && xp >= 1 && xp <= W && co < Cout;
+                    const bf16* src = row + (long long)(xp - 1) * Cout + co;
+                    if constexpr (VG) {
+                        tc::cp_async16(to + (uint32_t)e * 16u, get ? src : dy, get);
+                    } else {
+                        uint4 v = make_uint4(0, 0, 0, 0);
+                        if (get) v = tc::load8(src, Cout - co);
+                        *reinterpret_cast<uint4*>(to + (uint32_t)e * 16u) = v;
+                    }
+                    xp += gsx;
+                    i += gsi;
+                    if (xp >= Wp) xp -= Wp, i++;
                 }
             }
+            __syncwarp();
             tc::cp_async_commit();
             if (last >= 0) {  // the stage before this one has landed
                 tc::cp_async_wait<1>();
@@ -940,6 +1135,9 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict_
             }
             last = s;
             if (++s == sh.stages) s = 0, ph ^= 1;
+            row0 += ti;
+            x0 += tx;
+            if (x0 >= Wp) x0 -= Wp, row0++;
         }
         hand_over_all();
     }
@@ -951,37 +1149,32 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const bf16* __restrict_
         failed = 1;
     }
     __syncthreads();
-    const bool good = failed == 0, none = tile_begin == tile_end;  // no brick: sums of zero
+    const bool good = failed == 0, none = written == 0;  // none: sums of zero
     tc::fence_after_sync();
     if (warp > 0) {
         // row r of the accumulator lies in TMEM lane r (128 rows) or 32 (r / 16) + r % 16 (64 rows); the
-        // two copying warps of a lane quadrant alternate between chunks of 16 columns
+        // copying warps of a lane quadrant take turns with the chunks of 16 columns
         const int quad = warp & 3, half = (warp - 1) >> 2;
         const int r = rows == 128 ? quad * 32 + lane : (lane < 16 ? quad * 16 + lane : 128);
         const int dz = r / sh.cc, ci = c0 + r % sh.cc;
         const bool mine = r < 3 * sh.cc && ci < Cin;
-        for (int col = half * 16; col < 9 * sh.nt; col += 32) {
+        for (int col = half * 16; col < 9 * sh.nt; col += 16 * (WG_FILL / 128)) {
             float v[16];
+            __syncwarp();
             tc::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)col, v);
             const int t = col / sh.nt, co0 = n0 + col - t * sh.nt;
             if (!mine || co0 >= Cout) continue;
-            if (none) {
 #pragma unroll
-                for (int k = 0; k < 16; k++) v[k] = 0.f;
-            }
+            for (int k = 0; k < 16; k++) v[k] = !good ? __int_as_float(0x7fc00000) : (none ? 0.f : v[k]);
             float* dst = part + (((size_t)blockIdx.x * 27 + dz * 9 + t) * Cin + ci) * Cout + co0;
             if (Cout % 4 == 0) {
 #pragma unroll
                 for (int k = 0; k < 16; k += 4)
-                    if (co0 + k < Cout)
-                        *reinterpret_cast<float4*>(dst + k) =
-                            good ? make_float4(v[k], v[k + 1], v[k + 2], v[k + 3])
-                                 : make_float4(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000),
-                                               __int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
+                    if (co0 + k < Cout) *reinterpret_cast<float4*>(dst + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
             } else {
 #pragma unroll
                 for (int k = 0; k < 16; k++)
-                    if (co0 + k < Cout) dst[k] = good ? v[k] : __int_as_float(0x7fc00000);
+                    if (co0 + k < Cout) dst[k] = v[k];
             }
         }
     }
@@ -1034,6 +1227,29 @@ static int sm_count() {
         }
     }
     return sms;
+}
+
+// The convolution of two or four input channels (x aligned to a voxel).
+template <int CI>
+static int conv3d_few(const void* x, int n, int d, int h, int w, const void* wgt, const float* bias, int cout, int relu,
+                      int wrap, void* y, float* y32, bool vy, bool vy32, cudaStream_t s) {
+    const int want = (cout + 15) / 16 * 16, nt = want < 64 ? want : 64, gy = (cout + nt - 1) / nt;
+    const long long tiles = (long long)n * ((d + FEW_Z - 1) / FEW_Z) * ((h + 15) / 16) * ((w + 7) / 8);
+    const uint32_t smem = few_smem(CI, nt);
+    uint32_t cols = 32;
+    while (cols < (uint32_t)nt) cols <<= 1;
+    long long per_sm = (224 << 10) / (smem + 2048);  // by shared memory, TMEM columns and threads
+    if (per_sm > 512 / cols) per_sm = 512 / cols;
+    if (per_sm > 8) per_sm = 8;
+    const long long most = per_sm * sm_count(), gx = tiles < most ? tiles : most;
+    if (gy > 65535) return fail(LBM_ERR_ARG, "convolution: %d output channels exceed the grid", cout);
+    int rc = tc_launch_ok((const void*)k_conv_few<CI>, smem, "cudaFuncSetAttribute(k_conv_few)");
+    if (rc) return rc;
+    k_conv_few<CI><<<dim3((unsigned)gx, (unsigned)gy), TC_M, smem, s>>>(
+        static_cast<const bf16*>(x), n, d, h, w, static_cast<const bf16*>(wgt), bias, cout, nt, relu, wrap, vy, vy32,
+        static_cast<bf16*>(y), y32);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_conv_few launch");
 }
 
 // The convolution as an implicit GEMM, any channel counts and alignment.
@@ -1090,12 +1306,17 @@ static CvShape cv_pick(int n, int d, int h, int w, int cin, int cout, int* grid_
     return best;
 }
 
-// The convolution: halo planes for cin % 16 == 0, else the implicit GEMM.  Any
+// The convolution: halo planes for cin % 16 == 0, rows put together from a halo
+// for two or four input channels, else the gathering implicit GEMM.  Any
 // channel counts and alignment (16-byte copies and stores where a tensor's
 // channels and address allow, else narrower ones).
 int conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt, const float* bias, int cout, int relu,
            int wrap, void* y, float* y32, cudaStream_t s) {
     const bool vy = cout % 8 == 0 && (uintptr_t)y % 16 == 0, vy32 = cout % 4 == 0 && (uintptr_t)y32 % 16 == 0;
+    if (cin == 2 && (uintptr_t)x % 4 == 0)
+        return conv3d_few<2>(x, n, d, h, w, wgt, bias, cout, relu, wrap, y, y32, vy, vy32, s);
+    if (cin == 4 && (uintptr_t)x % 8 == 0)
+        return conv3d_few<4>(x, n, d, h, w, wgt, bias, cout, relu, wrap, y, y32, vy, vy32, s);
     if (cin % 16) return conv3d_im2col(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, vy, vy32, s);
     int gx = 1;
     const CvShape sh = cv_pick(n, d, h, w, cin, cout, &gx);
@@ -1156,42 +1377,61 @@ float* chunk_scratch(size_t floats) {
     return g_part_buf;
 }
 
-// dst[e] += sum over the chunks c of part[c][e], in a fixed order: NC threads
-// share an element (thread j takes chunks j, j + NC, ..), their sums are added
-// in thread order.  A thread's chain of loads over
-// its chunks is what it costs, so few elements (biases: up to 304 chunks of a
-// handful of channels) take more threads each.
-template <int NC>
-__global__ void __launch_bounds__(256) k_sum_chunks(const float* __restrict__ part, long long chunks, long long E,
-                                                    float* __restrict__ dst) {
-    constexpr int NE = 256 / NC;  // elements per block
-    __shared__ float sm[NC][NE];
-    const int i = threadIdx.x % NE, j = threadIdx.x / NE;
-    for (long long e0 = (long long)blockIdx.x * NE; e0 < E; e0 += (long long)gridDim.x * NE) {
-        const long long e = e0 + i;
+// dst[e] += sum over c = 0 .. chunks-1 of part[c][e], in that order, one thread
+// per element.  Bound by the chain of loads where there are few elements: 16 are
+// in flight at a time.
+__global__ void __launch_bounds__(64) k_sum_chunks(const float* __restrict__ part, long long chunks, long long E,
+                                                   float* __restrict__ dst) {
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (long long)gridDim.x * blockDim.x) {
         float s = 0.f;
-        if (e < E) {
-#pragma unroll 4
-            for (long long c = j; c < chunks; c += NC) s += part[c * E + e];
-        }
-        sm[j][i] = s;
-        __syncthreads();
-        if (j == 0 && e < E) {
-            float t = 0.f;
+        long long c = 0;
+        for (; c + 16 <= chunks; c += 16) {
+            float v[16];
 #pragma unroll
-            for (int k = 0; k < NC; k++) t += sm[k][i];
-            dst[e] += t;
+            for (int k = 0; k < 16; k++) v[k] = __ldg(part + (c + k) * E + e);
+#pragma unroll
+            for (int k = 0; k < 16; k++) s += v[k];
         }
-        __syncthreads();
+        for (; c < chunks; c++) s += __ldg(part + c * E + e);
+        dst[e] += s;
     }
 }
 
+// The same for few elements (bias gradients: 512 chunks of a handful of
+// channels), whose chain of loads is what it costs: a block's threads bring 256
+// chunks of eight elements to shared memory at once, eight of them add.
+__global__ void __launch_bounds__(256) k_sum_few(const float* __restrict__ part, long long chunks, long long E,
+                                                 float* __restrict__ dst) {
+    __shared__ float sm[256][8];
+    const int i = threadIdx.x % 8, j = threadIdx.x / 8;
+    for (long long e0 = (long long)blockIdx.x * 8; e0 < E; e0 += (long long)gridDim.x * 8) {
+        const long long e = e0 + i;
+        float s = 0.f;
+        for (long long c0 = 0; c0 < chunks; c0 += 256) {
+            const int n = (int)(chunks - c0 < 256 ? chunks - c0 : 256);
+#pragma unroll
+            for (int c = j; c < 256; c += 32) sm[c][i] = e < E && c < n ? __ldg(part + (c0 + c) * E + e) : 0.f;
+            __syncthreads();
+            if (j == 0) {
+#pragma unroll 16
+                for (int c = 0; c < n; c++) s += sm[c][i];
+            }
+            __syncthreads();
+        }
+        if (j == 0 && e < E) dst[e] += s;
+    }
+}
+
+int sum_few(const float* part, long long chunks, long long E, float* dst, cudaStream_t s) {
+    const long long blocks = (E + 7) / 8;
+    k_sum_few<<<(unsigned)(blocks < 8192 ? blocks : 8192), 256, 0, s>>>(part, chunks, E, dst);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_sum_few launch");
+}
+
 int sum_chunks(const float* part, long long chunks, long long E, float* dst, cudaStream_t s) {
-    const bool few = E < 4096;
-    const long long ne = few ? 8 : 32, blocks = (E + ne - 1) / ne;
-    const unsigned grid = (unsigned)(blocks < 8192 ? blocks : 8192);
-    if (few) k_sum_chunks<32><<<grid, 256, 0, s>>>(part, chunks, E, dst);
-    else k_sum_chunks<8><<<grid, 256, 0, s>>>(part, chunks, E, dst);
+    const long long blocks = (E + 63) / 64;
+    k_sum_chunks<<<(unsigned)(blocks < 16384 ? blocks : 16384), 64, 0, s>>>(part, chunks, E, dst);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_sum_chunks launch");
 }
@@ -1200,29 +1440,27 @@ int sum_chunks(const float* part, long long chunks, long long E, float* dst, cud
 // where a tensor's channels and address allow, else value by value).
 int wgrad_tc(const void* x, const void* dy, int n, int d, int h, int w, int cin, int cout, int wrap, float* dw,
              cudaStream_t s) {
-    // Voxel chunks: a block's FP32 accumulators in TMEM truncate, about 2e-8 of a sum per K = 16 step, so the
-    // chunks (their number here, their bounds in wg_chunk_begin) are part of the result's rounding.  A chunk is
-    // one of SMs / q of the voxels, q the 448-column accumulators that 27 taps of the input channels would fill
-    // (and the 128-channel output tiles), or 8192 voxels outside 8 .. 256 input channels; shorter chunks would be
-    // more exact, but up to 1e-4 from the results of that split, more than FP32 results may move.  For the same
-    // reason long sums run in bricks of few planes, closer to the order of memory: on random operands of 884,736
-    // voxels by 96 and 192 channels 1.8e-5 and 3.2e-5 from it with four planes, 1.3e-5 and 2.6e-5 with two, 7e-6
-    // and 1.1e-5 with one, which costs up to 1.4 times the time.
-    const long long M = (long long)n * d * h * w;
-    long long chunks = (M + 8191) / 8192;
+    const int Wp = (w + 2 + 7) / 8 * 8;
+    const WgShape sh = wg_shape(cin, cout, Wp);
+    const long long nsteps = ((long long)n * (d + 2) * (h + 2) * Wp + 63) / 64;
+    const long long groups = (cin + sh.cc - 1) / sh.cc, mt = (cout + sh.nt - 1) / sh.nt;
+    if (!sh.nt || groups > 65535 || mt > 65535)
+        return fail(LBM_ERR_ARG, "weight gradient: %d x %d channels exceed the grid", cin, cout);
+    // Chunks of positions: the FP32 accumulators in TMEM truncate, about 2e-8 of a sum per K = 16 step, so the
+    // chunks, their order and the order within them are part of the result's rounding: a different split moved the
+    // gradients of long sums by up to 1e-4, and a network trained on them drifts away from one trained before.  A
+    // chunk is one of SMs / q of the positions, q the 448-column accumulators that 27 taps of the input channels
+    // would fill (and the 128-channel output tiles), or 8192 voxels outside 8 .. 256 input channels.
+    long long chunks = ((long long)n * d * h * w + 8191) / 8192;
     const int cp = (cin + 15) / 16 * 16;
     if (cin >= 8 && cp <= 256) {
         const int per = 448 / cp < 27 ? 448 / cp : 27;
-        chunks = sm_count() / ((27 + per - 1) / per * ((cout + 127) / 128));
+        chunks = sm_count() / ((27 + per - 1) / per * ((cout + TC_M - 1) / TC_M));
     }
     if (chunks < 1) chunks = 1;
-    const long long steps = M / 16 / chunks;
-    const WgShape sh = wg_shape(cin, cout, steps > 2700 ? 1 : (steps > 1600 ? 2 : 4));
-    const long long tiles = (long long)n * ((d + sh.mb - 1) / sh.mb) * ((h + 15) / 16) * ((w + 7) / 8);
-    const long long groups = (cin + sh.cc - 1) / sh.cc, mt = (cout + sh.nt - 1) / sh.nt;
-    if (groups > 65535 || mt > 65535)
-        return fail(LBM_ERR_ARG, "weight gradient: %d x %d channels exceed the grid", cin, cout);
-    if (chunks > tiles) chunks = tiles;
+    if (chunks > nsteps) chunks = nsteps;
+    const long long spc = (nsteps + chunks - 1) / chunks;
+    chunks = (nsteps + spc - 1) / spc;
     const long long E = 27LL * cin * cout;
     float* part = chunk_scratch((size_t)(chunks * E));
     if (!part) return fail(LBM_ERR_OOM, "weight-gradient partial sums: %lld floats", chunks * E);
@@ -1230,7 +1468,7 @@ int wgrad_tc(const void* x, const void* dy, int n, int d, int h, int w, int cin,
         int rc = tc_launch_ok((const void*)kern, sh.smem, "cudaFuncSetAttribute(k_wgrad_tc)");
         if (rc) return rc;
         kern<<<dim3((unsigned)chunks, (unsigned)groups, (unsigned)mt), WG_THREADS, sh.smem, s>>>(
-            static_cast<const bf16*>(x), static_cast<const bf16*>(dy), n, d, h, w, cin, cout, wrap, sh, part);
+            static_cast<const bf16*>(x), static_cast<const bf16*>(dy), n, d, h, w, cin, cout, wrap, Wp, nsteps, spc, sh, part);
         const cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_wgrad_tc launch");
     };
