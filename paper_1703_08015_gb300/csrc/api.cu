@@ -83,6 +83,8 @@ struct lbm_ctx {
     StepLaunch publish_fn = nullptr;
     std::vector<SampleRange> samples;     // one entry per geometry of a batch
     std::vector<int> part_begin, part_blocks;  // their slices of the partial sums
+    int4* d_parts = nullptr;  // batch: the samples' blocks and tiles for one moments launch over all (NodeArgs::parts)
+    int batch_blocks = 0;     // its blocks
     StepArgs sa{};
     NodeArgs na{};
     StepLaunch step_fn = nullptr;
@@ -171,6 +173,7 @@ static void release(lbm_ctx* c) {
     cudaFree(c->d_ntab);
     cudaFree(c->d_partials);
     cudaFree(c->d_result);
+    cudaFree(c->d_parts);
     cudaFree(c->d_u_saved);
     cudaFree(c->d_stage);
     delete c;
@@ -248,7 +251,7 @@ static int init_ctx(lbm_ctx** out, const lbm_params* p, HostTiling& T, const std
         c->part_blocks.push_back(node_blocks(p->lattice, p->tile_a, r.n_tiles));
         acc += c->part_blocks.back();
     }
-    const int n_partials = std::max(std::max(c->nblocks, acc), 1);
+    const int n_partials = std::max(std::max(node_blocks_most(p->lattice, p->tile_a, nf), acc), 1);
 #define TRY(x)                \
     do {                      \
         int r_ = (x);         \
@@ -332,6 +335,14 @@ static int init_ctx(lbm_ctx** out, const lbm_params* p, HostTiling& T, const std
     }
     CTRY(cudaMalloc(&c->d_partials, (size_t)n_partials * 8 * sizeof(double)));
     CTRY(cudaMalloc(&c->d_result, 8 * sizeof(double) * samples.size()));
+    std::vector<int4> parts;
+    if (samples.size() > 1) {
+        for (size_t k = 0; k < samples.size(); k++)
+            parts.push_back(make_int4(c->part_begin[k], samples[k].tile_begin, samples[k].n_tiles,
+                                      node_groups_per_block(p->lattice, p->tile_a, samples[k].n_tiles)));
+        TRY(upload(&c->d_parts, parts, s));
+        c->batch_blocks = acc;
+    }
     CTRY(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking));
 
     StepArgs& sa = c->sa;
@@ -557,21 +568,29 @@ static NodeArgs sample_args(const lbm_ctx* c, size_t k) {
     return a;
 }
 
-// Moments of every sample (fields only for a single sample), each reduced in
-// a fixed order into d_result[8k .. 8k+7].
-static int launch_sample_moments(lbm_ctx* c, double* d_rho, double* d_u, bool residual, cudaStream_t s) {
+// Moments of every sample (fields only for a single sample) and, for `sums`,
+// each reduced in a fixed order into d_result[8k .. 8k+7].  A batch takes one
+// launch over all samples: 64 launches in turn, most of them too small for the
+// chip, took 4.1 ms for 64 samples of 32^3 to 160^3.
+static int launch_sample_moments(lbm_ctx* c, double* d_rho, double* d_u, bool residual, bool sums, cudaStream_t s) {
     if (residual && !c->d_u_saved)
         LBM_CUDA_TRY(cudaMalloc(&c->d_u_saved, (size_t)c->na.n_slots * 3 * sizeof(float2) + 8));
-    for (size_t k = 0; k < c->samples.size(); k++) {
-        NodeArgs a = sample_args(c, k);
-        a.rho_out = d_rho;
-        a.u_out = d_u;
-        a.residual = residual ? 1 : 0;
-        a.u_saved = residual ? c->d_u_saved : nullptr;
-        a.partials = c->d_partials + (size_t)8 * c->part_begin[k];
-        LBM_CUDA_TRY(c->moments_fn(a, s));
-        LBM_CUDA_TRY(launch_reduce(a.partials, c->part_blocks[k], c->d_result + 8 * k, s));
+    const int n = (int)c->samples.size();
+    NodeArgs a = sample_args(c, 0);
+    a.rho_out = d_rho;
+    a.u_out = d_u;
+    a.residual = residual ? 1 : 0;
+    a.u_saved = residual ? c->d_u_saved : nullptr;
+    a.partials = c->d_partials;
+    if (n > 1) {
+        a.parts = c->d_parts;
+        a.n_parts = n;
+        a.part_blocks = c->batch_blocks;
     }
+    LBM_CUDA_TRY(c->moments_fn(a, s));
+    if (!sums) return LBM_OK;
+    LBM_CUDA_TRY(n > 1 ? launch_reduce_parts(c->d_partials, c->batch_blocks, c->d_parts, n, c->d_result, s)
+                       : launch_reduce(c->d_partials, c->part_blocks[0], c->d_result, s));
     return LBM_OK;
 }
 
@@ -616,7 +635,7 @@ extern "C" int lbm_moments(lbm_ctx* c, double* rho, double* u, lbm_stats* stats,
         if (d_rho) LBM_CUDA_TRY(launch_fill_nan(d_rho, N, s));
         if (d_u) LBM_CUDA_TRY(launch_fill_nan(d_u, d * N, s));
     }
-    int rc = launch_sample_moments(c, d_rho, d_u, residual, s);
+    int rc = launch_sample_moments(c, d_rho, d_u, residual, stats != nullptr, s);
     if (rc) return rc;
     if (!dev && rho) LBM_CUDA_TRY(cudaMemcpyAsync(rho, d_rho, N * sizeof(double), cudaMemcpyDeviceToHost, s));
     if (!dev && u) LBM_CUDA_TRY(cudaMemcpyAsync(u, d_u, d * N * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -672,7 +691,7 @@ extern "C" int lbm_moments_batch(lbm_ctx* c, lbm_stats* stats, int flags, void* 
     if (!c || !stats) return fail(LBM_ERR_ARG, "NULL argument");
     cudaStream_t s = S(stream);
     const bool residual = flags & LBM_STATS_RESIDUAL;
-    int rc = launch_sample_moments(c, nullptr, nullptr, residual, s);
+    int rc = launch_sample_moments(c, nullptr, nullptr, residual, true, s);
     if (rc) return rc;
     std::vector<double> r(8 * c->samples.size());
     LBM_CUDA_TRY(cudaMemcpyAsync(r.data(), c->d_result, r.size() * sizeof(double), cudaMemcpyDeviceToHost, s));

@@ -219,6 +219,11 @@ struct NodeArgs {         // kernels that visit every node of every tile
     float2* u_saved;          // [3][n_slots] velocity of the last residual check (float-float) or NULL
     int residual;             // compare and save velocity
     double* partials;         // [blocks][8]
+    int groups_per_block;     // moments: tile groups of a block (set by the launch)
+    // moments without fields over every sample of a batch in one launch of part_blocks blocks: per sample {first
+    // block, first tile, tiles, tile groups per block}; n_parts 0: the tiles above
+    const int4* parts;
+    int n_parts, part_blocks;
 };
 
 using StepLaunch = cudaError_t (*)(const StepArgs&, cudaStream_t);
@@ -265,4 +270,9 @@ cudaError_t launch_reduce(const double* partials, int nblocks, double* result, c
 void fixed_consts(const lbm_params* p, FixedConsts* k);
 void ff_consts(const lbm_params* p, FFConsts* k);
 
+int node_blocks_most(int lattice, int a, int n_tiles);  // the largest over all numbers of tiles up to n_tiles
+int node_groups_per_block(int lattice, int a, int n_tiles);
 }  // namespace lbm
+// the same for each sample of a batch (parts as in NodeArgs, nblocks of all): result[8 k ..] of sample k
+cudaError_t launch_reduce_parts(const double* partials, int nblocks, const int4* parts, int n_parts, double* result,
+                                cudaStream_t s);

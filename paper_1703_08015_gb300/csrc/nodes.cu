@@ -8,7 +8,15 @@
 namespace lbm {
 
 constexpr int kStats = 8;  // mass, momentum x/y/z, |u|^2, |u - u_saved|^2, fluid count, spare
-constexpr int kMomentGroups = 8;  // tile groups per block of the moments kernel
+
+// Tile groups per block of the moments kernel: up to eight, whose staging
+// overlaps, but no fewer than two blocks per SM while there are groups to
+// spare: a block works through a group in about 3 us, so eight groups on a
+// quarter of the SMs took 25 us for a 64^3 sample.
+static int moment_groups(int groups) {
+    const int g = groups / 304;
+    return g < 1 ? 1 : (g > 8 ? 8 : g);
+}
 
 template <class L, int A>
 __device__ __forceinline__ bool dense_index(const NodeArgs& a, int tile, const NodePos<A>& p, size_t& n) {
@@ -169,8 +177,23 @@ __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256
     __shared__ double red[NTH / 32][kStats];
     const int lt = threadIdx.x / TL::NT;
     const int node = threadIdx.x - lt * TL::NT;
-    const int tile_end = a.tile_begin + a.n_tiles;
-    const int n_groups = (a.n_tiles + TPB - 1) / TPB;
+    // the tiles of this launch, or of this block's sample in a launch over a batch
+    int tile_begin = a.tile_begin, n_tiles = a.n_tiles, per_block = a.groups_per_block, block = blockIdx.x;
+    if (a.n_parts) {
+        int lo = 0, hi = a.n_parts - 1;  // the last sample that begins at or before this block
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) / 2;
+            if (__ldg(&a.parts[mid].x) <= block) lo = mid;
+            else hi = mid - 1;
+        }
+        const int4 part = __ldg(a.parts + lo);
+        block -= part.x;
+        tile_begin = part.y;
+        n_tiles = part.z;
+        per_block = part.w;
+    }
+    const int tile_end = tile_begin + n_tiles;
+    const int n_groups = (n_tiles + TPB - 1) / TPB;
     const NodePos<A> p = node_pos<TL>(node);
     const bool want_fields = a.rho_out || a.u_out;
     const size_t N = (size_t)a.nx * a.ny * a.nz;  // fields only for a single-sample launch
@@ -188,7 +211,7 @@ __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256
     const int e_lt = e / PER_TILE, e_rem = e - e_lt * PER_TILE;
     const int e_slot = e_rem / TL::W, e_w = e_rem - e_slot * TL::W;
     auto load_nb = [&](int g) {
-        const int t = a.tile_begin + g * TPB + e_lt;
+        const int t = tile_begin + g * TPB + e_lt;
         return has_entry && t < tile_end ? __ldg(a.nbr + (size_t)t * TL::NN + e_slot) : -1;
     };
     auto load_rec = [&](int nb) {
@@ -204,9 +227,9 @@ __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256
             s.loc[e_lt][e_slot] = r.y ? make_int2((int)((long long)(r.y >> 24) - origin), (int)(r.y & 0xFFFFFFull))
                                       : make_int2(0, 0);
     };
-    const int g0 = blockIdx.x * kMomentGroups;
-    const int g_end = min(n_groups, g0 + kMomentGroups);
-    if (g0 < g_end) store(sh[0], load_rec(load_nb(g0)), __ldg(a.tile_off + a.tile_begin + g0 * TPB));
+    const int g0 = block * per_block;
+    const int g_end = min(n_groups, g0 + per_block);
+    if (g0 < g_end) store(sh[0], load_rec(load_nb(g0)), __ldg(a.tile_off + tile_begin + g0 * TPB));
     int nb_next = g0 + 1 < g_end ? load_nb(g0 + 1) : -1;
     __syncthreads();
     for (int g = g0; g < g_end; g++) {
@@ -216,10 +239,10 @@ __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256
         long long origin_next = 0;
         if (more) {
             rec_next = load_rec(nb_next);
-            origin_next = __ldg(a.tile_off + a.tile_begin + (g + 1) * TPB);
+            origin_next = __ldg(a.tile_off + tile_begin + (g + 1) * TPB);
         }
         const int nb_after = g + 2 < g_end ? load_nb(g + 2) : -1;
-        const int tile = a.tile_begin + g * TPB + lt;
+        const int tile = tile_begin + g * TPB + lt;
         size_t n = 0;
         if (tile < tile_end && mask_bit(cur, lt, TL::CENTER, node) && (!want_fields || dense_index<L, A>(a, tile, p, n))) {
             T raw[L::Q];
@@ -325,9 +348,16 @@ __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256
     }
 }
 
-// One block sums the per-block partials in a fixed order.
+// One block per sample sums its per-block partials in a fixed order (parts: the
+// samples' first blocks; NULL: one sample of nblocks).
 __global__ void __launch_bounds__(256) k_reduce(const double* __restrict__ partials, int nblocks,
-                                               double* __restrict__ result) {
+                                               const int4* __restrict__ parts, double* __restrict__ result) {
+    if (parts) {
+        const int begin = parts[blockIdx.x].x;
+        nblocks = (blockIdx.x + 1 < gridDim.x ? parts[blockIdx.x + 1].x : nblocks) - begin;
+        partials += (size_t)begin * kStats;
+        result += (size_t)blockIdx.x * kStats;
+    }
     __shared__ double sm[256][kStats];
     double acc[kStats];
 #pragma unroll
@@ -547,9 +577,11 @@ template <class L, int A, int MODEL, class S>
 cudaError_t launch_moments(const NodeArgs& a, cudaStream_t s) {
     constexpr int TPB = tiles_per_block<L, A>();
     const int groups = (a.n_tiles + TPB - 1) / TPB;
-    const int blocks = (groups + kMomentGroups - 1) / kMomentGroups;
+    NodeArgs b = a;
+    b.groups_per_block = moment_groups(groups);
+    const int blocks = a.n_parts ? a.part_blocks : (groups + b.groups_per_block - 1) / b.groups_per_block;
     if (blocks == 0) return cudaSuccess;
-    k_moments<L, A, TPB, MODEL, S><<<blocks, TPB * Tile<L, A>::NT, 0, s>>>(a);
+    k_moments<L, A, TPB, MODEL, S><<<blocks, TPB * Tile<L, A>::NT, 0, s>>>(b);
     return cudaGetLastError();
 }
 
@@ -590,17 +622,36 @@ cudaError_t launch_average(void* cur, const void* prev, size_t bytes, int storag
 }
 
 cudaError_t launch_reduce(const double* partials, int nblocks, double* result, cudaStream_t s) {
-    k_reduce<<<1, 256, 0, s>>>(partials, nblocks, result);
+    k_reduce<<<1, 256, 0, s>>>(partials, nblocks, nullptr, result);
     return cudaGetLastError();
 }
 
-int node_blocks(int lattice, int a, int n_tiles) {
+cudaError_t launch_reduce_parts(const double* partials, int nblocks, const int4* parts, int n_parts, double* result,
+                                cudaStream_t s) {
+    k_reduce<<<n_parts, 256, 0, s>>>(partials, nblocks, parts, result);
+    return cudaGetLastError();
+}
+
+static int tile_groups(int lattice, int a, int n_tiles) {
     int nt = 1;
     const int d = lattice == LBM_D2Q9 ? 2 : 3;
     for (int k = 0; k < d; k++) nt *= a;
     const int tpb = nt >= 256 ? 1 : 256 / nt;
-    const int groups = (n_tiles + tpb - 1) / tpb;
-    return (groups + kMomentGroups - 1) / kMomentGroups;
+    return (n_tiles + tpb - 1) / tpb;
+}
+
+int node_groups_per_block(int lattice, int a, int n_tiles) { return moment_groups(tile_groups(lattice, a, n_tiles)); }
+
+int node_blocks(int lattice, int a, int n_tiles) {
+    const int per = node_groups_per_block(lattice, a, n_tiles);
+    return (tile_groups(lattice, a, n_tiles) + per - 1) / per;
+}
+
+// fewer tiles can take more blocks, of fewer groups each: at most 607 of one or two
+int node_blocks_most(int lattice, int a, int n_tiles) {
+    const int groups = tile_groups(lattice, a, n_tiles), now = node_blocks(lattice, a, n_tiles);
+    const int small = groups < 608 ? groups : 608;
+    return now > small ? now : small;
 }
 
 // ---- selection ------------------------------------------------------------------------
