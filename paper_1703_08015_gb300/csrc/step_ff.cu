@@ -46,10 +46,10 @@ __global__ void __launch_bounds__(BT, MINB) k_step_ff(const StepArgs a) {
         T b[L::Q];
         int stride;
         T* out = gather_rec<L, A, work_tiles(), T>(sh, a.src, a.dst, wn.lt, wn.node, p, b, stride);
-        // out of range: the same update in native FP64 (a call, so that its
-        // registers do not weigh on the float-float path)
+        // out of range: the wider rounding, then native FP64 (a call, so that
+        // its registers do not weigh on the float-float path)
         if (!collide_ff<L, MODEL, FAX>(b, a.fx, a.ffc, out, stride))
-            update_fp64_rec<L, A, MODEL, work_tiles()>(sh, a, wn, p);
+            update_wide_rec<L, A, MODEL, work_tiles()>(sh, a, wn, p);
     } else {
         __shared__ NeighShared<TL, work_tiles()> sh;
         WorkNode wn;
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(BT, MINB) k_step_ff(const StepArgs a) {
         const int stride = sh.loc[wn.lt][TL::CENTER].y;
         T* out = own_slot<TL, work_tiles(), T>(sh, a.dst, wn.lt, rank);
         if (!collide_ff<L, MODEL, FAX>(b, a.fx, a.ffc, out, stride))
-            update_fp64<L, A, MODEL, work_tiles()>(sh, a, wn, p, out, stride);
+            update_wide<L, A, MODEL, work_tiles()>(sh, a, wn, p, out, stride);
     }
 }
 

@@ -150,6 +150,19 @@ __device__ __noinline__ Words<L::Q> tgb_update_fp64(const NeighShared<Tile<L, A>
     return w;
 }
 
+// The same with the float-float arithmetic's wider rounding first (update_wide).
+template <class L, int A, int MODEL, int KMAX>
+__device__ __noinline__ Words<L::Q> tgb_update_wide(const NeighShared<Tile<L, A>, KMAX>& sh,
+                                                    const int (&nbt)[KMAX][Tile<L, A>::NN], const StepArgs& a, int lt,
+                                                    int node, const NodePos<A>& p) {
+    unsigned long long raw[L::Q];
+    gather_tgb<L, A, KMAX, unsigned long long>(sh, nbt, static_cast<const unsigned long long*>(a.dst),
+                                               static_cast<const unsigned long long*>(a.ghost_in), lt, node, p, raw);
+    Words<L::Q> w;
+    if (!collide_ff<L, MODEL, -1, true>(raw, a.fx, a.ffc, w.v, 1)) w = tgb_update_fp64<L, A, MODEL, KMAX>(sh, nbt, a, lt, node, p);
+    return w;
+}
+
 // Resident blocks per SM requested (register cap) for each arithmetic.
 template <class L, int A, int ARITH>
 constexpr int tgb_min_blocks() {
@@ -190,7 +203,7 @@ __global__ void __launch_bounds__(work_threads<L, A>(), tgb_min_blocks<L, A, ARI
         } else {
             if constexpr (ARITH == 1) {
                 if (!collide_ff<L, MODEL>(raw, a.fx, a.ffc, vals, 1)) {
-                    const Words<L::Q> w = tgb_update_fp64<L, A, MODEL, work_tiles()>(sh, nbt, a, lt, node, p);
+                    const Words<L::Q> w = tgb_update_wide<L, A, MODEL, work_tiles()>(sh, nbt, a, lt, node, p);
                     static_for<0, L::Q>([&](auto I) { vals[decltype(I)::value] = w.v[decltype(I)::value]; });
                 }
             } else {
