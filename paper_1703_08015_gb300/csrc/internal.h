@@ -234,6 +234,23 @@ using NodeListLaunch = cudaError_t (*)(const uint64_t* tmask, const long long* t
 NodeListLaunch select_node_list(int lattice, int a);
 using NodeLaunch = cudaError_t (*)(const NodeArgs&, cudaStream_t);
 
+// Launch of a step kernel that may start while its predecessor in the stream
+// still runs (programmatic dependent launch; kept by graph capture): up to
+// chain_wait() (tile.cuh) it reads only tables that no step writes.
+template <class... P, class... Args>
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t s, Args&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // Kernel selection (nullptr when a combination is not compiled).
 StepLaunch select_step(const lbm_params* p);
 void f32_consts(const lbm_params* p, double omega, const double* force, F32Consts* k);
@@ -253,6 +270,8 @@ NodeLaunch select_moments(int lattice, int a, int model, int storage);
 NodeLaunch select_export(int lattice, int a, int storage);
 NodeLaunch select_import(int lattice, int a, int storage);
 int node_blocks(int lattice, int a, int n_tiles);  // grid (= partial sums) of the moments kernel
+int node_blocks_most(int lattice, int a, int n_tiles);  // the largest over all numbers of tiles up to n_tiles
+int node_groups_per_block(int lattice, int a, int n_tiles);
 cudaError_t launch_fill_nan(double* p, size_t n, cudaStream_t s);
 // the neighbour records of the compact tiles from their coordinates and the
 // dense tile map (build_tiling's rule); a check that no neighbour lies more
@@ -266,13 +285,11 @@ cudaError_t launch_build_ntab(const int32_t* nbr, const uint64_t* tmask, const l
                               const int32_t* tile_stride, int n_tiles, int nn, NRec* ntab, cudaStream_t s);
 cudaError_t launch_average(void* cur, const void* prev, size_t bytes, int storage, cudaStream_t s);
 cudaError_t launch_reduce(const double* partials, int nblocks, double* result, cudaStream_t s);
+// the same for each sample of a batch (parts as in NodeArgs, nblocks of all): result[8 k ..] of sample k
+cudaError_t launch_reduce_parts(const double* partials, int nblocks, const int4* parts, int n_parts, double* result,
+                                cudaStream_t s);
 
 void fixed_consts(const lbm_params* p, FixedConsts* k);
 void ff_consts(const lbm_params* p, FFConsts* k);
 
-int node_blocks_most(int lattice, int a, int n_tiles);  // the largest over all numbers of tiles up to n_tiles
-int node_groups_per_block(int lattice, int a, int n_tiles);
 }  // namespace lbm
-// the same for each sample of a batch (parts as in NodeArgs, nblocks of all): result[8 k ..] of sample k
-cudaError_t launch_reduce_parts(const double* partials, int nblocks, const int4* parts, int n_parts, double* result,
-                                cudaStream_t s);

@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256
         size_t n = 0;
         if (tile < tile_end && mask_bit(cur, lt, TL::CENTER, node) && (!want_fields || dense_index<L, A>(a, tile, p, n))) {
             T raw[L::Q];
-            const int rank = gather<L, A, TPB, T>(cur, a.pdf, lt, node, p, raw);
+            const int rank = gather<L, A, TPB, T, true>(cur, a.pdf, lt, node, p, raw);
             const long long slot = (cur.origin + cur.loc[lt][TL::CENTER].x) / L::Q + rank;
             float2 prev[3];
             float2* us = a.residual && a.u_saved ? a.u_saved + slot : nullptr;

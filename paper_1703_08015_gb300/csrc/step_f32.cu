@@ -15,7 +15,11 @@
 
 namespace lbm {
 
-template <class L, int A, int MODEL, class S, int BT, bool PERSIST>
+// CHAIN: launched while the step before still runs (chain_wait).  That hides a
+// small grid's launch and staging (64^3 sample, FP32 deviations: 4.24 to 3.6 us
+// per step); a large one gains less from it than it loses by the ordinary loads
+// (192 x 177 x 203: 71.1 to 71.7 us, 256^3 in FP16: 139.9 to 144.1).
+template <class L, int A, int MODEL, class S, int BT, bool PERSIST, bool CHAIN>
 __global__ void __launch_bounds__(BT, (!PERSIST && BT <= 256) ? 1536 / BT : 1) k_step_f32(const StepArgs a) {
     using TL = Tile<L, A>;
     using T = typename S::T;
@@ -29,12 +33,12 @@ __global__ void __launch_bounds__(BT, (!PERSIST && BT <= 256) ? 1536 / BT : 1) k
         WorkBlock pw{};
         if (pf) pw = a.blocks[wbi + a.pf_ahead];
         WorkNode wn;
-        const bool active = stage_work_at<TL, work_tiles(), BT>(sh, a, wbi, wn);
+        const bool active = stage_work_at<TL, work_tiles(), BT, CHAIN>(sh, a, wbi, wn);
         if (pf) prefetch_work_block<TL::NN>(a, pw);
         if (active) {
             const NodePos<A> p = node_pos<TL>(wn.node);
             T raw[L::Q];
-            const int rank = gather<L, A, work_tiles(), T>(sh, a.src, wn.lt, wn.node, p, raw);
+            const int rank = gather<L, A, work_tiles(), T, !CHAIN>(sh, a.src, wn.lt, wn.node, p, raw);
             const int stride = sh.loc[wn.lt][TL::CENTER].y;
             float g[L::Q];
             static_for<0, L::Q>([&](auto I) {
@@ -62,12 +66,15 @@ cudaError_t launch_step_f32(const StepArgs& a, cudaStream_t s) {
             int dev = 0, sms = 0, per_sm = 0;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_f32<L, A, MODEL, S, BT, PERSIST>, BT, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_f32<L, A, MODEL, S, BT, PERSIST, false>, BT, 0);
             resident = sms * (per_sm > 0 ? per_sm : 1);
         }
         grid = a.n_work_blocks < resident ? a.n_work_blocks : resident;
     }
-    k_step_f32<L, A, MODEL, S, BT, PERSIST><<<grid, BT, 0, s>>>(a);
+    // two waves of six blocks per SM
+    if constexpr (!PERSIST)
+        if (grid <= 1824) return launch_chained(k_step_f32<L, A, MODEL, S, BT, false, true>, (unsigned)grid, BT, s, a);
+    k_step_f32<L, A, MODEL, S, BT, PERSIST, false><<<grid, BT, 0, s>>>(a);
     return cudaGetLastError();
 }
 

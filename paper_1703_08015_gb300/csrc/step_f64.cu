@@ -33,8 +33,7 @@ __global__ void __launch_bounds__(work_threads<L, A>()) k_step_f64(const StepArg
 template <class L, int A, int MODEL, class S>
 cudaError_t launch_step_f64(const StepArgs& a, cudaStream_t s) {
     if (a.n_work_blocks == 0) return cudaSuccess;
-    k_step_f64<L, A, MODEL, S><<<a.n_work_blocks, work_threads<L, A>(), 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_step_f64<L, A, MODEL, S>, (unsigned)a.n_work_blocks, work_threads<L, A>(), s, a);
 }
 
 template <class L, int A, class S>

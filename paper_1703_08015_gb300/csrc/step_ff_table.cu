@@ -76,10 +76,11 @@ __global__ void __launch_bounds__(kTableThreads, 7) k_step_ff_table(const StepAr
     const T* src = static_cast<const T*>(a.src);
     const int own = __ldg(t);
     T b[L::Q];
-    b[0] = __ldg(src + own);
+    chain_wait();
+    b[0] = src[own];
     static_for<1, L::Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
-        b[i] = __ldg(src + __ldg(t + i * P));
+        b[i] = src[__ldg(t + i * P)];
     });
     const int stride = __ldg(t + L::Q * P);
     T* out = static_cast<T*>(a.dst) + own;
@@ -92,8 +93,7 @@ __global__ void __launch_bounds__(kTableThreads, 7) k_step_ff_table(const StepAr
 template <class L, int MODEL>
 cudaError_t launch_step_ff_table(const StepArgs& a, cudaStream_t s) {
     if (a.n_nodes == 0) return cudaSuccess;
-    k_step_ff_table<L, MODEL><<<(unsigned)((a.n_nodes + kTableThreads - 1) / kTableThreads), kTableThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_step_ff_table<L, MODEL>, (unsigned)((a.n_nodes + kTableThreads - 1) / kTableThreads), kTableThreads, s, a);
 }
 
 template <class L, int A>

@@ -191,8 +191,7 @@ __global__ void __launch_bounds__(work_threads<L, A>(), MINB) k_step_fixed(const
 template <class L, int A, int MODEL, int MINB>
 cudaError_t launch_step_fixed(const StepArgs& a, cudaStream_t s) {
     if (a.n_work_blocks == 0) return cudaSuccess;
-    k_step_fixed<L, A, MODEL, MINB><<<a.n_work_blocks, work_threads<L, A>(), 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_step_fixed<L, A, MODEL, MINB>, (unsigned)a.n_work_blocks, work_threads<L, A>(), s, a);
 }
 
 // ---- host: constants -------------------------------------------------------

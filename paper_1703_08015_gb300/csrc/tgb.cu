@@ -99,7 +99,7 @@ constexpr int ghost_per_tile() {
 // when it is outside, bounce-back when the source is not a fluid node.
 template <class L, int A, int KMAX, class T>
 __device__ __forceinline__ int gather_tgb(const NeighShared<Tile<L, A>, KMAX>& sh, const int (&nbt)[KMAX][Tile<L, A>::NN],
-                                          const T* copy, const T* __restrict__ ghost_in, int lt, int node,
+                                          const T* copy, const T* ghost_in, int lt, int node,
                                           const NodePos<A>& p, T (&f)[L::Q]) {
     using TL = Tile<L, A>;
     constexpr int E = ghost_per_tile<L, A>();
@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(work_threads<L, A>(), tgb_min_blocks<L, A, ARI
     const uint32_t e = active ? __ldg(a.nodes + wb.node_begin + threadIdx.x) : 0u;  // in flight during the staging
     stage_tables<TL, work_tiles(), work_threads<L, A>()>(sh, a, wb, nbt);
     __syncthreads();
+    chain_wait();
     T vals[L::Q];
     int tile = 0, lt = 0, node = 0, rank = 0;
     NodePos<A> p{0, 0, 0};
@@ -255,8 +256,7 @@ __global__ void k_tgb_publish(const StepArgs a) {
 template <class L, int A, int MODEL, class S, int ARITH>
 cudaError_t launch_step_tgb(const StepArgs& a, cudaStream_t s) {
     if (a.n_work_blocks == 0) return cudaSuccess;
-    k_step_tgb<L, A, MODEL, S, ARITH><<<a.n_work_blocks, work_threads<L, A>(), 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_step_tgb<L, A, MODEL, S, ARITH>, (unsigned)a.n_work_blocks, work_threads<L, A>(), s, a);
 }
 
 template <class L, int A, class S>
