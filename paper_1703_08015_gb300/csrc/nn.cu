@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 #include "lbm_nn.h"
@@ -81,122 +82,140 @@ __global__ void k_weight_flip(const bf16* __restrict__ w, int Cin, int Cout, bf1
     }
 }
 
-__global__ void k_relu_mask(bf16* __restrict__ g, const bf16* __restrict__ act, size_t n) {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-        if (!(__bfloat162float(act[e]) > 0.f)) g[e] = __float2bfloat16(0.f);
+// ---- elementwise passes over activations ------------------------------------
+// All are bound by memory.  A thread takes V consecutive channels of a voxel, 8
+// (16 bytes) where the channel counts and addresses allow, and finds its voxel
+// with indices of type I, 32 bits where the tensors allow: one channel per
+// thread with 64-bit divisions these passes took 1.9 ms of a training step on 8
+// x 64^3 voxels, several times their memory time.
+template <int V>
+struct alignas(2 * V) Pack {
+    bf16 v[V];
+};
+
+template <int V>
+__device__ __forceinline__ Pack<V> load_pack(const bf16* p) {
+    return *reinterpret_cast<const Pack<V>*>(p);
+}
+template <int V>
+__device__ __forceinline__ void store_pack(bf16* p, const Pack<V>& x) {
+    *reinterpret_cast<Pack<V>*>(p) = x;
 }
 
-__global__ void k_pool2(const bf16* __restrict__ x, int N, int D, int H, int W, int C, bf16* __restrict__ y) {
-    const int d = D / 2, h = H / 2, w = W / 2;
-    const long long n = (long long)N * d * h * w * C;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        long long t = e / C;
-        const int xx = (int)(t % w);
-        t /= w;
-        const int yy = (int)(t % h);
-        t /= h;
-        const int zz = (int)(t % d);
-        const int nn = (int)(t / d);
-        float s = 0.f;
+template <int V, class I>
+__global__ void k_relu_mask(bf16* __restrict__ g, const bf16* __restrict__ act, I n) {
+    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < n; e += (I)gridDim.x * blockDim.x) {
+        const Pack<V> a = load_pack<V>(act + (size_t)e * V);
+        Pack<V> x = load_pack<V>(g + (size_t)e * V);
+#pragma unroll
+        for (int k = 0; k < V; k++)
+            if (!(__bfloat162float(a.v[k]) > 0.f)) x.v[k] = __float2bfloat16(0.f);
+        store_pack(g + (size_t)e * V, x);
+    }
+}
+
+// The group of channels e of a tensor [.][D][H][W][G groups]: its sample, voxel
+// and group.
+template <class I>
+struct Cell {
+    I n;
+    int z, y, x, g;
+    __device__ __forceinline__ Cell(I e, int D, int H, int W, int G) {
+        I t = e / G;
+        g = (int)(e - t * G);
+        I u = t / W;
+        x = (int)(t - u * W);
+        t = u / H;
+        y = (int)(u - t * H);
+        n = t / D;
+        z = (int)(t - n * D);
+    }
+};
+
+// y[n][z][y][x] = the mean (MEAN) or sum of the eight voxels of a D x H x W box of
+// twice the size.
+template <int V, class I, bool MEAN>
+__global__ void k_down2(const bf16* __restrict__ x, I total, int D, int H, int W, int G, bf16* __restrict__ y) {
+    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < total; e += (I)gridDim.x * blockDim.x) {
+        const Cell<I> c(e, D, H, W, G);
+        float s[V];
+#pragma unroll
+        for (int j = 0; j < V; j++) s[j] = 0.f;
+#pragma unroll
         for (int k = 0; k < 8; k++) {
-            const int z = 2 * zz + (k >> 2), y_ = 2 * yy + ((k >> 1) & 1), x_ = 2 * xx + (k & 1);
-            s += __bfloat162float(x[((((long long)nn * D + z) * H + y_) * W + x_) * C + c]);
+            const size_t at = ((((size_t)c.n * 2 * D + 2 * c.z + (k >> 2)) * 2 * H + 2 * c.y + ((k >> 1) & 1)) * 2 * W + 2 * c.x + (k & 1)) * G + c.g;
+            const Pack<V> v = load_pack<V>(x + at * V);
+#pragma unroll
+            for (int j = 0; j < V; j++) s[j] += __bfloat162float(v.v[j]);
         }
-        y[e] = __float2bfloat16(0.125f * s);
+        Pack<V> o;
+#pragma unroll
+        for (int j = 0; j < V; j++) o.v[j] = __float2bfloat16(MEAN ? 0.125f * s[j] : s[j]);
+        store_pack(y + (size_t)e * V, o);
     }
 }
 
-__global__ void k_pool2_bwd(const bf16* __restrict__ dy, int N, int D, int H, int W, int C, bf16* __restrict__ dx) {
-    const long long n = (long long)N * D * H * W * C;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        long long t = e / C;
-        const int x_ = (int)(t % W);
-        t /= W;
-        const int y_ = (int)(t % H);
-        t /= H;
-        const int z = (int)(t % D);
-        const int nn = (int)(t / D);
-        const long long src = ((((long long)nn * (D / 2) + z / 2) * (H / 2) + y_ / 2) * (W / 2) + x_ / 2) * C + c;
-        dx[e] = __float2bfloat16(0.125f * __bfloat162float(dy[src]));
-    }
-}
-
-__global__ void k_up2(const bf16* __restrict__ x, int N, int D, int H, int W, int C, bf16* __restrict__ y) {
-    const long long n = (long long)N * 8 * D * H * W * C;
-    const int D2 = 2 * D, H2 = 2 * H, W2 = 2 * W;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        long long t = e / C;
-        const int x_ = (int)(t % W2);
-        t /= W2;
-        const int y_ = (int)(t % H2);
-        t /= H2;
-        const int z = (int)(t % D2);
-        const int nn = (int)(t / D2);
-        y[e] = x[((((long long)nn * D + z / 2) * H + y_ / 2) * W + x_ / 2) * C + c];
-    }
-}
-
-__global__ void k_up2_bwd(const bf16* __restrict__ dy, int N, int D, int H, int W, int C, bf16* __restrict__ dx) {
-    const long long n = (long long)N * D * H * W * C;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        long long t = e / C;
-        const int x_ = (int)(t % W);
-        t /= W;
-        const int y_ = (int)(t % H);
-        t /= H;
-        const int z = (int)(t % D);
-        const int nn = (int)(t / D);
-        float s = 0.f;
-        for (int k = 0; k < 8; k++) {
-            const int zz = 2 * z + (k >> 2), yy = 2 * y_ + ((k >> 1) & 1), xx = 2 * x_ + (k & 1);
-            s += __bfloat162float(dy[((((long long)nn * 2 * D + zz) * 2 * H + yy) * 2 * W + xx) * C + c]);
+// y (D x H x W) from a box of half the size: each voxel's parent, an eighth of it (SCALE).
+template <int V, class I, bool SCALE>
+__global__ void k_up2(const bf16* __restrict__ x, I total, int D, int H, int W, int G, bf16* __restrict__ y) {
+    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < total; e += (I)gridDim.x * blockDim.x) {
+        const Cell<I> c(e, D, H, W, G);
+        const size_t at = ((((size_t)c.n * (D / 2) + c.z / 2) * (H / 2) + c.y / 2) * (W / 2) + c.x / 2) * G + c.g;
+        Pack<V> v = load_pack<V>(x + at * V);
+        if constexpr (SCALE) {
+#pragma unroll
+            for (int j = 0; j < V; j++) v.v[j] = __float2bfloat16(0.125f * __bfloat162float(v.v[j]));
         }
-        dx[e] = __float2bfloat16(s);
+        store_pack(y + (size_t)e * V, v);
     }
 }
 
-__global__ void k_concat(const bf16* __restrict__ a, int ca, const bf16* __restrict__ b, int cb, size_t vox,
+// ga and gb groups of channels per voxel
+template <int V, class I>
+__global__ void k_concat(const bf16* __restrict__ a, int ga, const bf16* __restrict__ b, int gb, I total,
                          bf16* __restrict__ y) {
-    const int c = ca + cb;
-    const size_t n = vox * c;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const size_t v = e / c;
-        const int k = (int)(e - v * c);
-        y[e] = k < ca ? a[v * ca + k] : b[v * cb + (k - ca)];
+    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < total; e += (I)gridDim.x * blockDim.x) {
+        const I v = e / (ga + gb);
+        const int k = (int)(e - v * (ga + gb));
+        store_pack(y + (size_t)e * V, k < ga ? load_pack<V>(a + ((size_t)v * ga + k) * V)
+                                             : load_pack<V>(b + ((size_t)v * gb + (k - ga)) * V));
     }
 }
 
-__global__ void k_split(const bf16* __restrict__ y, int ca, int cb, size_t vox, bf16* __restrict__ a,
-                        bf16* __restrict__ b) {
-    const int c = ca + cb;
-    const size_t n = vox * c;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const size_t v = e / c;
-        const int k = (int)(e - v * c);
-        if (k < ca) {
-            if (a) a[v * ca + k] = y[e];
+template <int V, class I>
+__global__ void k_split(const bf16* __restrict__ y, int ga, int gb, I total, bf16* __restrict__ a, bf16* __restrict__ b) {
+    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < total; e += (I)gridDim.x * blockDim.x) {
+        const I v = e / (ga + gb);
+        const int k = (int)(e - v * (ga + gb));
+        if (k < ga) {
+            if (a) store_pack(a + ((size_t)v * ga + k) * V, load_pack<V>(y + (size_t)e * V));
         } else if (b) {
-            b[v * cb + (k - ca)] = y[e];
+            store_pack(b + ((size_t)v * gb + (k - ga)) * V, load_pack<V>(y + (size_t)e * V));
         }
     }
 }
 
-__global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ tgt, const uint8_t* __restrict__ mask,
-                      size_t vox, int c, float inv_count, double* __restrict__ loss, bf16* __restrict__ dpred) {
+// The block's squared errors are added up before its one atomic addition (one
+// per warp made 32,768 additions to one address).
+template <class I>
+__global__ void __launch_bounds__(256) k_mse(const float* __restrict__ pred, const float* __restrict__ tgt,
+                                             const uint8_t* __restrict__ mask, I total, int c, float inv_count,
+                                             double* __restrict__ loss, bf16* __restrict__ dpred) {
+    __shared__ double sm[8];
     double s = 0.0;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < vox * c; e += (size_t)gridDim.x * blockDim.x) {
-        const size_t v = e / c;
+    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < total; e += (I)gridDim.x * blockDim.x) {
         float d = 0.f;
-        if (mask[v]) d = pred[e] - tgt[e];
+        if (mask[e / c]) d = pred[e] - tgt[e];
         s += (double)d * d;
         dpred[e] = __float2bfloat16(2.f * d * inv_count);
     }
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, s * inv_count);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; w++) s += sm[w];
+        atomicAdd(loss, s * inv_count);
+    }
 }
 
 __global__ void k_adam(float* __restrict__ p, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
@@ -214,9 +233,15 @@ __global__ void k_adam(float* __restrict__ p, float* __restrict__ g, float* __re
     }
 }
 
-__global__ void k_add(const bf16* __restrict__ a, const bf16* __restrict__ b, size_t n, bf16* __restrict__ y) {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-        y[e] = __float2bfloat16(__bfloat162float(a[e]) + __bfloat162float(b[e]));
+template <int V, class I>
+__global__ void k_add(const bf16* a, const bf16* b, I n, bf16* y) {  // y may be a or b
+    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < n; e += (I)gridDim.x * blockDim.x) {
+        const Pack<V> p = load_pack<V>(a + (size_t)e * V), q = load_pack<V>(b + (size_t)e * V);
+        Pack<V> o;
+#pragma unroll
+        for (int k = 0; k < V; k++) o.v[k] = __float2bfloat16(__bfloat162float(p.v[k]) + __bfloat162float(q.v[k]));
+        store_pack(y + (size_t)e * V, o);
+    }
 }
 
 __global__ void k_mask_input(const uint8_t* __restrict__ mask, size_t vox, float value, bf16* __restrict__ x) {
@@ -319,52 +344,98 @@ extern "C" int lbm_nn_conv3d_wgrad(const void* x, const void* dy, int n, int d, 
     return rc ? rc : sum_few(part, nb, cout, dbias, S(stream));
 }
 
+// Runs go(V, I) with the widest pack that the channel counts (or total) `c` and
+// the addresses `at` (ORed) allow, and indices wide enough for `total` values
+// plus a grid's stride.
+template <class F>
+static void by_width(unsigned long long c, uintptr_t at, size_t total, F go) {
+    const bool wide = c % 8 == 0 && at % 16 == 0, small = total < (1ull << 31);
+    using W8 = std::integral_constant<int, 8>;
+    using W1 = std::integral_constant<int, 1>;
+    if (wide && small) go(W8{}, unsigned{});
+    else if (wide) go(W8{}, (unsigned long long)0);
+    else if (small) go(W1{}, unsigned{});
+    else go(W1{}, (unsigned long long)0);
+}
+static uintptr_t adr(const void* p) { return reinterpret_cast<uintptr_t>(p); }
+
 extern "C" int lbm_nn_relu_mask(void* g, const void* act, size_t count, void* stream) {
     if (!g || !act) return fail(LBM_ERR_ARG, "lbm_nn_relu_mask: NULL");
-    k_relu_mask<<<grid_for(count), 256, 0, S(stream)>>>(static_cast<bf16*>(g), static_cast<const bf16*>(act), count);
+    by_width(count, adr(g) | adr(act), count, [&](auto V, auto I) {
+        constexpr int v = decltype(V)::value;
+        k_relu_mask<v, decltype(I)><<<grid_for(count / v), 256, 0, S(stream)>>>(
+            static_cast<bf16*>(g), static_cast<const bf16*>(act), (decltype(I))(count / v));
+    });
     return check(cudaGetLastError(), "k_relu_mask launch");
+}
+
+// One thread per pack of the result, of voxels n x d x h x w and c channels.
+template <class K>
+static void over_cells(const void* x, int n, int d, int h, int w, int c, void* y, K launch) {
+    const size_t total = (size_t)n * d * h * w * c;
+    by_width((unsigned)c, adr(x) | adr(y), total, [&](auto V, auto I) {
+        constexpr int v = decltype(V)::value;
+        launch(V, I, (decltype(I))(total / v), c / v, grid_for(total / v));
+    });
 }
 
 extern "C" int lbm_nn_pool2(const void* x, int n, int d, int h, int w, int c, void* y, void* stream) {
     if (!x || !y || (d | h | w) & 1) return fail(LBM_ERR_ARG, "lbm_nn_pool2: bad arguments");
-    k_pool2<<<grid_for((size_t)n * d * h * w * c / 8), 256, 0, S(stream)>>>(static_cast<const bf16*>(x), n, d, h, w,
-                                                                            c, static_cast<bf16*>(y));
-    return check(cudaGetLastError(), "k_pool2 launch");
+    over_cells(x, n, d / 2, h / 2, w / 2, c, y, [&](auto V, auto I, auto total, int groups, unsigned grid) {
+        k_down2<decltype(V)::value, decltype(I), true><<<grid, 256, 0, S(stream)>>>(
+            static_cast<const bf16*>(x), total, d / 2, h / 2, w / 2, groups, static_cast<bf16*>(y));
+    });
+    return check(cudaGetLastError(), "k_down2 launch");
 }
 
 extern "C" int lbm_nn_pool2_bwd(const void* dy, int n, int d, int h, int w, int c, void* dx, void* stream) {
     if (!dy || !dx || (d | h | w) & 1) return fail(LBM_ERR_ARG, "lbm_nn_pool2_bwd: bad arguments");
-    k_pool2_bwd<<<grid_for((size_t)n * d * h * w * c), 256, 0, S(stream)>>>(static_cast<const bf16*>(dy), n, d, h, w,
-                                                                            c, static_cast<bf16*>(dx));
-    return check(cudaGetLastError(), "k_pool2_bwd launch");
+    over_cells(dy, n, d, h, w, c, dx, [&](auto V, auto I, auto total, int groups, unsigned grid) {
+        k_up2<decltype(V)::value, decltype(I), true><<<grid, 256, 0, S(stream)>>>(
+            static_cast<const bf16*>(dy), total, d, h, w, groups, static_cast<bf16*>(dx));
+    });
+    return check(cudaGetLastError(), "k_up2 launch");
 }
 
 extern "C" int lbm_nn_up2(const void* x, int n, int d, int h, int w, int c, void* y, void* stream) {
     if (!x || !y) return fail(LBM_ERR_ARG, "lbm_nn_up2: NULL");
-    k_up2<<<grid_for((size_t)n * 8 * d * h * w * c), 256, 0, S(stream)>>>(static_cast<const bf16*>(x), n, d, h, w, c,
-                                                                           static_cast<bf16*>(y));
+    over_cells(x, n, 2 * d, 2 * h, 2 * w, c, y, [&](auto V, auto I, auto total, int groups, unsigned grid) {
+        k_up2<decltype(V)::value, decltype(I), false><<<grid, 256, 0, S(stream)>>>(
+            static_cast<const bf16*>(x), total, 2 * d, 2 * h, 2 * w, groups, static_cast<bf16*>(y));
+    });
     return check(cudaGetLastError(), "k_up2 launch");
 }
 
 extern "C" int lbm_nn_up2_bwd(const void* dy, int n, int d, int h, int w, int c, void* dx, void* stream) {
     if (!dy || !dx) return fail(LBM_ERR_ARG, "lbm_nn_up2_bwd: NULL");
-    k_up2_bwd<<<grid_for((size_t)n * d * h * w * c), 256, 0, S(stream)>>>(static_cast<const bf16*>(dy), n, d, h, w, c,
-                                                                           static_cast<bf16*>(dx));
-    return check(cudaGetLastError(), "k_up2_bwd launch");
+    over_cells(dy, n, d, h, w, c, dx, [&](auto V, auto I, auto total, int groups, unsigned grid) {
+        k_down2<decltype(V)::value, decltype(I), false><<<grid, 256, 0, S(stream)>>>(
+            static_cast<const bf16*>(dy), total, d, h, w, groups, static_cast<bf16*>(dx));
+    });
+    return check(cudaGetLastError(), "k_down2 launch");
 }
 
 extern "C" int lbm_nn_concat(const void* a, int ca, const void* b, int cb, size_t voxels, void* y, void* stream) {
     if (!a || !b || !y) return fail(LBM_ERR_ARG, "lbm_nn_concat: NULL");
-    k_concat<<<grid_for(voxels * (ca + cb)), 256, 0, S(stream)>>>(static_cast<const bf16*>(a), ca,
-                                                                 static_cast<const bf16*>(b), cb, voxels,
-                                                                 static_cast<bf16*>(y));
+    const size_t total = voxels * (ca + cb);
+    by_width((unsigned)(ca | cb), adr(a) | adr(b) | adr(y), total, [&](auto V, auto I) {
+        constexpr int v = decltype(V)::value;
+        k_concat<v, decltype(I)><<<grid_for(total / v), 256, 0, S(stream)>>>(
+            static_cast<const bf16*>(a), ca / v, static_cast<const bf16*>(b), cb / v, (decltype(I))(total / v),
+            static_cast<bf16*>(y));
+    });
     return check(cudaGetLastError(), "k_concat launch");
 }
 
 extern "C" int lbm_nn_split(const void* y, int ca, int cb, size_t voxels, void* a, void* b, void* stream) {
     if (!y) return fail(LBM_ERR_ARG, "lbm_nn_split: NULL");
-    k_split<<<grid_for(voxels * (ca + cb)), 256, 0, S(stream)>>>(static_cast<const bf16*>(y), ca, cb, voxels,
-                                                                static_cast<bf16*>(a), static_cast<bf16*>(b));
+    const size_t total = voxels * (ca + cb);
+    by_width((unsigned)(ca | cb), adr(a) | adr(b) | adr(y), total, [&](auto V, auto I) {
+        constexpr int v = decltype(V)::value;
+        k_split<v, decltype(I)><<<grid_for(total / v), 256, 0, S(stream)>>>(
+            static_cast<const bf16*>(y), ca / v, cb / v, (decltype(I))(total / v), static_cast<bf16*>(a),
+            static_cast<bf16*>(b));
+    });
     return check(cudaGetLastError(), "k_split launch");
 }
 
@@ -373,8 +444,13 @@ extern "C" int lbm_nn_mse(const float* pred, const float* target, const uint8_t*
     if (!pred || !target || !mask || !loss || !dpred || c < 1) return fail(LBM_ERR_ARG, "lbm_nn_mse: bad arguments");
     const float inv = count ? 1.f / ((float)count * c) : 0.f;
     LBM_CUDA_TRY(cudaMemsetAsync(loss, 0, sizeof(double), S(stream)));
-    k_mse<<<grid_for(voxels * c), 256, 0, S(stream)>>>(pred, target, mask, voxels, c, inv, loss,
-                                                       static_cast<bf16*>(dpred));
+    const size_t total = voxels * c;
+    if (total < (1ull << 31))
+        k_mse<unsigned><<<grid_for(total), 256, 0, S(stream)>>>(pred, target, mask, (unsigned)total, c, inv, loss,
+                                                                static_cast<bf16*>(dpred));
+    else
+        k_mse<unsigned long long><<<grid_for(total), 256, 0, S(stream)>>>(pred, target, mask, total, c, inv, loss,
+                                                                          static_cast<bf16*>(dpred));
     return check(cudaGetLastError(), "k_mse launch");
 }
 
@@ -389,8 +465,11 @@ extern "C" int lbm_nn_adam(float* p, float* g, float* m, float* v, void* pb, siz
 
 extern "C" int lbm_nn_add(const void* a, const void* b, size_t count, void* y, void* stream) {
     if (!a || !b || !y) return fail(LBM_ERR_ARG, "lbm_nn_add: NULL");
-    k_add<<<grid_for(count), 256, 0, S(stream)>>>(static_cast<const bf16*>(a), static_cast<const bf16*>(b), count,
-                                                  static_cast<bf16*>(y));
+    by_width(count, adr(a) | adr(b) | adr(y), count, [&](auto V, auto I) {
+        constexpr int v = decltype(V)::value;
+        k_add<v, decltype(I)><<<grid_for(count / v), 256, 0, S(stream)>>>(
+            static_cast<const bf16*>(a), static_cast<const bf16*>(b), (decltype(I))(count / v), static_cast<bf16*>(y));
+    });
     return check(cudaGetLastError(), "k_add launch");
 }
 

@@ -454,3 +454,77 @@ def test_conv_weight_gradient_tile_edges(nn, case, offset):
     err = np.abs(f64(dw).reshape(27, cin, cout) - 0.25 - ref_w)
     assert np.all(err <= tol_w), float(np.max(err / tol_w))
     assert np.allclose(f64(db) + 0.5, ref_b, rtol=1e-5, atol=1e-4)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("c", [8, 24, 12])
+def test_elementwise_passes_wide_and_narrow(nn, c, offset):
+    """The elementwise passes on 16-byte packs (channel counts of 8, aligned tensors) and value by value: pure
+    moves and sums of eight BF16 values in [0.5, 2), exact in FP32."""
+    rng = np.random.default_rng(19 + c + offset)
+    n, d, h, w = 2, 4, 2, 6
+
+    def dev(a):
+        t = torch.empty(a.size + offset, dtype=torch.bfloat16, device="cuda")
+        t[offset:] = bf16_dev(a).reshape(-1)
+        return t[offset:]
+
+    def new(*shape):
+        return torch.zeros(int(np.prod(shape)) + offset, dtype=torch.bfloat16, device="cuda")[offset:]
+
+    x = R.bf16_round(rng.uniform(0.5, 2.0, (n, d, h, w, c)) * rng.choice([-1, 1], (n, d, h, w, c)))
+    xs = R.bf16_round(rng.uniform(0.5, 2.0, (n, d // 2, h // 2, w // 2, c)))
+    b = R.bf16_round(rng.normal(size=(n, d, h, w, 8)))
+    small, large, large2, cat = new(*xs.shape), new(*x.shape), new(*x.shape), new(n, d, h, w, c + 8)
+    b2 = new(*b.shape)
+    vox = n * d * h * w
+    nn.lbm_nn_pool2(dev(x), n, d, h, w, c, small)
+    assert np.array_equal(f64(small).reshape(xs.shape), R.bf16_round(R.pool2(x)))
+    nn.lbm_nn_up2_bwd(dev(x), n, d // 2, h // 2, w // 2, c, small)
+    assert np.array_equal(f64(small).reshape(xs.shape), R.bf16_round(R.up2_bwd(x)))
+    nn.lbm_nn_up2(dev(xs), n, d // 2, h // 2, w // 2, c, large)
+    assert np.array_equal(f64(large).reshape(x.shape), R.up2(xs))
+    nn.lbm_nn_pool2_bwd(dev(xs), n, d, h, w, c, large)
+    assert np.array_equal(f64(large).reshape(x.shape), R.bf16_round(R.pool2_bwd(xs)))
+    nn.lbm_nn_concat(dev(x), c, dev(b), 8, vox, cat)
+    assert np.array_equal(f64(cat).reshape(n, d, h, w, c + 8), np.concatenate([x, b], axis=4))
+    nn.lbm_nn_split(cat, c, 8, vox, large, b2)
+    assert np.array_equal(f64(large).reshape(x.shape), x) and np.array_equal(f64(b2).reshape(b.shape), b)
+    nn.lbm_nn_split(cat, c, 8, vox, None, b2)
+    nn.lbm_nn_add(large, large, x.size, large2)
+    assert np.array_equal(f64(large2).reshape(x.shape), 2 * x)
+    g = dev(np.ones_like(x))
+    nn.lbm_nn_relu_mask(g, dev(x), x.size)
+    assert np.array_equal(f64(g).reshape(x.shape), (x > 0).astype(np.float64))
+
+
+@pytest.mark.parametrize("case", [
+    # n, d, h, w, cin, cout, relu, wrap: an input of two or four channels (rows put together from a halo) at a
+    # brick's edges and several output tiles, chunks of 64 input channels with a shorter last one, output channels
+    # that are no multiple of 16, of 8 or of 4
+    (1, 9, 17, 9, 2, 16, 1, 1),
+    (2, 8, 16, 8, 4, 70, 0, 6),
+    (1, 1, 1, 1, 4, 3, 0, 7),
+    (1, 17, 18, 7, 16, 4, 0, 1),
+    (1, 3, 16, 8, 80, 36, 1, 2),
+    (2, 2, 5, 17, 128, 10, 0, 4),
+    (1, 5, 4, 6, 144, 130, 1, 3),
+])
+def test_conv_tile_edges(nn, case):
+    """The convolution where its bricks, channel chunks and output tiles end; the tolerance is that of the cases
+    above."""
+    n, d, h, w, cin, cout, relu, wrap = case
+    rng = np.random.default_rng(23 + hash(case) % 2**31)
+    x = rand_bf16(rng, (n, d, h, w, cin))
+    wt = rand_bf16(rng, (27, cin, cout), 1.0 / np.sqrt(27 * cin))
+    b = rng.normal(0, 0.1, cout).astype(np.float32)
+    y = torch.empty((n, d, h, w, cout), dtype=torch.bfloat16, device="cuda")
+    y32 = torch.empty((n, d, h, w, cout), dtype=torch.float32, device="cuda")
+    nn.lbm_nn_conv3d(bf16_dev(x), n, d, h, w, cin, bf16_dev(wt), torch.from_numpy(b).cuda(), cout, relu, wrap, y, y32)
+    torch.cuda.synchronize()
+    assert nn.lbm_nn_tc_timeouts() == 0
+    ref = R.conv3d(x, wt, b.astype(np.float64), bool(relu), wrap)
+    tol = 2.0 ** -16 * R.conv3d(np.abs(x), np.abs(wt), np.abs(b.astype(np.float64)), False, wrap) + 1e-30
+    got = f64(y32)
+    assert np.all(np.abs(got - ref) <= tol), np.max(np.abs(got - ref) / tol)
+    assert np.array_equal(f64(y), R.bf16_round(got))
