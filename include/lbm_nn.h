@@ -5,9 +5,8 @@
  * field from a geometry mask so that the lattice Boltzmann solve reaches its
  * steady state in fewer steps; the LBM residual alone still decides
  * convergence.  These entry points are the network's GPU kernels: 3x3x3
- * convolutions on tensor cores (BF16 operands, FP32 accumulation; tcgen05 or
- * mma.sync by shape) for the
- * forward pass and both backward passes, plus the pooling, upsampling,
+ * convolutions on the tcgen05 tensor cores (BF16 operands, FP32 accumulation)
+ * for the forward pass and both backward passes, plus the pooling, upsampling,
  * concatenation, loss and optimiser steps of training.
  *
  * Conventions
@@ -79,9 +78,9 @@ int lbm_nn_weight_flip(const void* wgt, int cin, int cout, void* wt, void* strea
  * tcgen05 tensor cores for every shape, reading both operands from
  * channels-last tiles in shared memory (zero-padded to 8 input and 16 output
  * channels); the partial sums live in a library-owned device buffer (grown on
- * demand, kept for the process; calls
- * must not overlap on different streams).  Errors: LBM_ERR_ARG, LBM_ERR_OOM
- * (no room for the partial sums), LBM_ERR_CUDA. */
+ * demand, kept for the process; calls must not overlap on different streams).
+ * Errors: LBM_ERR_ARG, LBM_ERR_OOM (no room for the partial sums),
+ * LBM_ERR_CUDA. */
 int lbm_nn_conv3d_wgrad(const void* x, const void* dy, int n, int d, int h, int w, int cin, int cout,
                         int wrap, float* dw, float* dbias, void* stream);
 
