@@ -13,9 +13,10 @@ constexpr int kStats = 8;  // mass, momentum x/y/z, |u|^2, |u - u_saved|^2, flui
 // overlaps, but no fewer than two blocks per SM while there are groups to
 // spare: a block works through a group in about 3 us, so eight groups on a
 // quarter of the SMs took 25 us for a 64^3 sample.
+constexpr int kMomentGroups = 8;
 static int moment_groups(int groups) {
     const int g = groups / 304;
-    return g < 1 ? 1 : (g > 8 ? 8 : g);
+    return g < 1 ? 1 : (g > kMomentGroups ? kMomentGroups : g);
 }
 
 template <class L, int A>
@@ -78,7 +79,7 @@ __global__ void k_init(const NodeArgs a) {
 // form sums its deviations f_i - w_i in float-float; u = (j + F/2) / rho
 // follows in float-float.  A node whose FP64 words fall outside that range
 // (or are not finite) takes the FP64 formulas.  Each thread accumulates its
-// nodes of kMomentGroups tile groups in float-float, and the block sums its
+// nodes of its tile groups in float-float, and the block sums its
 // threads in a fixed order; the per-block partials are FP64.
 
 __device__ __forceinline__ ff ff_of(double v) {
@@ -165,7 +166,11 @@ __device__ __forceinline__ void moments_words(const typename S::T (&raw)[L::Q], 
     jz = ff_norm(z);
 }
 
-template <class L, int A, int TPB, int MODEL, class S>
+// GROUPS: tile groups per block of a launch over one sample, 0: as the launch
+// says; -1: every sample of a batch in one launch, without fields
+// (NodeArgs::parts).  Apart, because the search for the block's sample and a
+// group count in a register spill the large launches that need neither.
+template <class L, int A, int TPB, int MODEL, class S, int GROUPS>
 __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256 ? 1 : (S::id == LBM_STORE_F64 ? 2 : 3))
     k_moments(const NodeArgs a) {
     using TL = Tile<L, A>;
@@ -178,8 +183,10 @@ __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256
     const int lt = threadIdx.x / TL::NT;
     const int node = threadIdx.x - lt * TL::NT;
     // the tiles of this launch, or of this block's sample in a launch over a batch
-    int tile_begin = a.tile_begin, n_tiles = a.n_tiles, per_block = a.groups_per_block, block = blockIdx.x;
-    if (a.n_parts) {
+    constexpr bool BATCH = GROUPS < 0;
+    int tile_begin = a.tile_begin, n_tiles = a.n_tiles, per_block = GROUPS > 0 ? GROUPS : a.groups_per_block,
+        block = blockIdx.x;
+    if constexpr (BATCH) {
         int lo = 0, hi = a.n_parts - 1;  // the last sample that begins at or before this block
         while (lo < hi) {
             const int mid = (lo + hi + 1) / 2;
@@ -195,7 +202,7 @@ __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256
     const int tile_end = tile_begin + n_tiles;
     const int n_groups = (n_tiles + TPB - 1) / TPB;
     const NodePos<A> p = node_pos<TL>(node);
-    const bool want_fields = a.rho_out || a.u_out;
+    const bool want_fields = !BATCH && (a.rho_out || a.u_out);
     const size_t N = (size_t)a.nx * a.ny * a.nz;  // fields only for a single-sample launch
     const ff half_f[3] = {ff_of(0.5 * a.force[0]), ff_of(0.5 * a.force[1]), ff_of(L::D == 3 ? 0.5 * a.force[2] : 0.0)};
     ff acc_dr{0.f, 0.f}, acc_m[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, acc_u2{0.f, 0.f}, acc_du2{0.f, 0.f};
@@ -295,8 +302,8 @@ __global__ void __launch_bounds__(TPB* Tile<L, A>::NT, TPB* Tile<L, A>::NT > 256
                 u[1] = ff_of(uy);
                 u[2] = ff_of(uz);
             }
-            if (a.rho_out) a.rho_out[n] = 1.0 + dbl_of(dr);
-            if (a.u_out) {
+            if (!BATCH && a.rho_out) a.rho_out[n] = 1.0 + dbl_of(dr);
+            if (!BATCH && a.u_out) {
                 a.u_out[n] = dbl_of(u[0]);
                 a.u_out[N + n] = dbl_of(u[1]);
                 if (L::D == 3) a.u_out[2 * N + n] = dbl_of(u[2]);
@@ -581,7 +588,12 @@ cudaError_t launch_moments(const NodeArgs& a, cudaStream_t s) {
     b.groups_per_block = moment_groups(groups);
     const int blocks = a.n_parts ? a.part_blocks : (groups + b.groups_per_block - 1) / b.groups_per_block;
     if (blocks == 0) return cudaSuccess;
-    k_moments<L, A, TPB, MODEL, S><<<blocks, TPB * Tile<L, A>::NT, 0, s>>>(b);
+    if (a.n_parts)
+        k_moments<L, A, TPB, MODEL, S, -1><<<blocks, TPB * Tile<L, A>::NT, 0, s>>>(b);
+    else if (b.groups_per_block == kMomentGroups)
+        k_moments<L, A, TPB, MODEL, S, kMomentGroups><<<blocks, TPB * Tile<L, A>::NT, 0, s>>>(b);
+    else
+        k_moments<L, A, TPB, MODEL, S, 0><<<blocks, TPB * Tile<L, A>::NT, 0, s>>>(b);
     return cudaGetLastError();
 }
 
