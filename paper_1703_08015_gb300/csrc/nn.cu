@@ -1,6 +1,7 @@
 // nn.cu -- the learned warm start (not in the paper): the entry points of the
-// 3x3x3 convolutions, whose tensor-core kernels are in nn_tc.cu, the bias
-// gradient and the elementwise steps of training.  See include/lbm_nn.h.
+// 3x3x3 convolutions, whose tcgen05 kernels are in nn_tc.cu, their mma.sync form
+// for odd numbers of input channels, the bias gradient and the elementwise steps
+// of training.  See include/lbm_nn.h.
 #include <cuda_bf16.h>
 
 #include <cstdint>
@@ -14,6 +15,123 @@ namespace lbm {
 namespace nn {
 
 using bf16 = __nv_bfloat16;
+
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], const unsigned (&b)[2]) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+__device__ __forceinline__ unsigned lds32(const bf16* p) { return *reinterpret_cast<const unsigned*>(p); }
+
+constexpr int BM = 64;  // GEMM rows per block
+constexpr int BK = 32;  // reduction depth per shared-memory stage
+constexpr int LD = BK + 8;
+
+// Neighbour coordinate along one axis with zero padding (returns -1 outside)
+// or periodic wrap.
+__device__ __forceinline__ int nb_coord(int c, int d, int n, bool wrap) {
+    c += d;
+    if (wrap) return c < 0 ? c + n : (c >= n ? c - n : c);
+    return (c < 0 || c >= n) ? -1 : c;
+}
+
+// C[p][co] = sum_k A[p][k] B[k][co], A[p][(tap,ci)] = x[p + off(tap)][ci] (0 outside,
+// or wrapped on the axes set in `wrap`), B[(tap,ci)][co] = wgt[tap][ci][co]; one
+// block computes 64 voxels x NF*8 outputs starting at channel blockIdx.y * NF*8.
+// For an odd number of input channels, whose values lie at odd addresses: gathered
+// one by one either way, the warp-level MMAs cost less here than the tcgen05
+// pipeline's start per block (1 -> 16 channels on 4 x 32^3 voxels 21 and 47 us,
+// 7 -> 9 84 and 171).
+template <int NF>
+__global__ void __launch_bounds__(128) k_conv(const bf16* __restrict__ x, int N, int D, int H, int W, int Cin,
+                                              const bf16* __restrict__ wgt, const float* __restrict__ bias,
+                                              int Cout, int relu, int wrap, bf16* __restrict__ y,
+                                              float* __restrict__ y32) {
+    constexpr int BN = NF * 8;
+    __shared__ __align__(16) bf16 As[BM][LD];
+    __shared__ __align__(16) bf16 Bs[BN][LD];
+    const long long M = (long long)N * D * H * W;
+    const int K = 27 * Cin;
+    const long long m0 = (long long)blockIdx.x * BM;
+    const int n0 = blockIdx.y * BN;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    float acc[NF][4];
+#pragma unroll
+    for (int f = 0; f < NF; f++) acc[f][0] = acc[f][1] = acc[f][2] = acc[f][3] = 0.f;
+
+    // this thread gathers row ar, columns ak .. ak+15 of every A stage
+    const int ar = tid >> 1, ak = (tid & 1) * 16;
+    const long long am = m0 + ar;
+    const bool arow = am < M;
+    int an = 0, az = 0, ay = 0, ax = 0;
+    if (arow) {
+        long long t = am;
+        ax = (int)(t % W);
+        t /= W;
+        ay = (int)(t % H);
+        t /= H;
+        az = (int)(t % D);
+        an = (int)(t / D);
+    }
+    const bool wx = wrap & 1, wy = wrap & 2, wz = wrap & 4;
+    const bf16 zero = __float2bfloat16(0.f);
+    for (int k0 = 0; k0 < K; k0 += BK) {
+        int k = k0 + ak;
+        int tap = k / Cin, ci = k - tap * Cin;
+#pragma unroll
+        for (int j = 0; j < 16; j++) {
+            bf16 v = zero;
+            if (arow && k < K) {
+                const int zz = nb_coord(az, tap / 9 - 1, D, wz), yy = nb_coord(ay, (tap / 3) % 3 - 1, H, wy),
+                          xx = nb_coord(ax, tap % 3 - 1, W, wx);
+                if ((zz | yy | xx) >= 0) v = x[((((long long)an * D + zz) * H + yy) * W + xx) * Cin + ci];
+            }
+            As[ar][ak + j] = v;
+            k++;
+            if (++ci == Cin) {
+                ci = 0;
+                tap++;
+            }
+        }
+        for (int e = tid; e < BN * BK; e += 128) {
+            const int kk = e / BN, nn = e - kk * BN;
+            const int kg = k0 + kk;
+            Bs[nn][kk] = (kg < K && n0 + nn < Cout) ? wgt[(long long)kg * Cout + n0 + nn] : zero;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int ks = 0; ks < BK; ks += 16) {
+            const int r = warp * 16 + (lane >> 2), c = ks + (lane & 3) * 2;
+            const unsigned a[4] = {lds32(&As[r][c]), lds32(&As[r + 8][c]), lds32(&As[r][c + 8]),
+                                   lds32(&As[r + 8][c + 8])};
+#pragma unroll
+            for (int f = 0; f < NF; f++) {
+                const int nn = f * 8 + (lane >> 2);
+                const unsigned b[2] = {lds32(&Bs[nn][c]), lds32(&Bs[nn][c + 8])};
+                mma_bf16(acc[f], a, b);
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int f = 0; f < NF; f++)
+#pragma unroll
+        for (int h2 = 0; h2 < 2; h2++)
+#pragma unroll
+            for (int j = 0; j < 2; j++) {
+                const long long row = m0 + warp * 16 + (lane >> 2) + h2 * 8;
+                const int co = n0 + f * 8 + (lane & 3) * 2 + j;
+                if (row < M && co < Cout) {
+                    float v = acc[f][h2 * 2 + j] + (bias ? bias[co] : 0.f);
+                    if (relu) v = fmaxf(v, 0.f);
+                    if (y) y[row * Cout + co] = __float2bfloat16(v);
+                    if (y32) y32[row * Cout + co] = v;
+                }
+            }
+}
 
 // Partial bias gradients of blocks of kBiasRows rows: part[blockIdx.x][c] = sum
 // of dy over the block's rows, in row order (one FP32 chain per channel: the
@@ -297,6 +415,22 @@ static int check(cudaError_t e, const char* what) { return e == cudaSuccess ? LB
 using namespace lbm;
 using namespace lbm::nn;
 
+// Output-channel tiling of k_conv: the channels are split into equal tiles of at most 128, each a multiple of 8.
+static int pick_nf(int cout, int* n_tiles) {
+    const int tiles = (cout + 127) / 128;
+    const int per = (cout + tiles - 1) / tiles;
+    const int need = (per + 7) / 8;
+    static const int sizes[] = {1, 2, 4, 6, 8, 12, 16};
+    int nf = 16;
+    for (int s : sizes)
+        if (s >= need) {
+            nf = s;
+            break;
+        }
+    *n_tiles = (cout + nf * 8 - 1) / (nf * 8);
+    return nf;
+}
+
 namespace lbm {
 namespace nn {
 int conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt, const float* bias, int cout, int relu,
@@ -312,7 +446,25 @@ extern "C" int lbm_nn_conv3d(const void* x, int n, int d, int h, int w, int cin,
                              const float* bias, int cout, int relu, int wrap, void* y, float* y32, void* stream) {
     if (!x || !wgt || n < 1 || d < 1 || h < 1 || w < 1 || cin < 1 || cout < 1 || (!y && !y32) || (wrap & ~7))
         return fail(LBM_ERR_ARG, "lbm_nn_conv3d: bad arguments");
-    return conv3d(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, S(stream));
+    if (cin % 2 == 0) return conv3d(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, S(stream));
+    const long long M = (long long)n * d * h * w;
+    int ny = 0;
+    const int nf = pick_nf(cout, &ny);
+    const dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)ny);
+    auto go = [&](auto kern) {
+        kern<<<grid, 128, 0, S(stream)>>>(static_cast<const bf16*>(x), n, d, h, w, cin, static_cast<const bf16*>(wgt),
+                                          bias, cout, relu, wrap, static_cast<bf16*>(y), y32);
+    };
+    switch (nf) {
+        case 1: go(k_conv<1>); break;
+        case 2: go(k_conv<2>); break;
+        case 4: go(k_conv<4>); break;
+        case 6: go(k_conv<6>); break;
+        case 8: go(k_conv<8>); break;
+        case 12: go(k_conv<12>); break;
+        default: go(k_conv<16>); break;
+    }
+    return check(cudaGetLastError(), "k_conv launch");
 }
 
 extern "C" int lbm_nn_weight_flip(const void* wgt, int cin, int cout, void* wt, void* stream) {
