@@ -6,8 +6,9 @@
  * steady state in fewer steps; the LBM residual alone still decides
  * convergence.  These entry points are the network's GPU kernels: 3x3x3
  * convolutions on tensor cores (BF16 operands, FP32 accumulation; tcgen05, or
- * mma.sync for odd numbers of input channels) for the forward pass and both backward passes, plus the pooling, upsampling,
- * concatenation, loss and optimiser steps of training.
+ * mma.sync for odd numbers of input channels) for the forward pass and both
+ * backward passes, plus the pooling, upsampling, concatenation, loss and
+ * optimiser steps of training.
  *
  * Conventions
  *   - Activations are channels-last BF16 (or FP32 where stated) tensors
