@@ -625,6 +625,10 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
                     if (inside && co0 < Cout) conv_out(v, ok, sbias + q, relu, co0, Cout, at + co0, vy, vy32, y, y32);
                 }
             }
+            // Every warp's arrival has to belong to this brick: a warp without a plane of it (half 1 of a brick of
+            // one plane) waits for the brick's sums as well.  Arriving at once, it ran ahead of the others, and its
+            // arrivals for later bricks handed over accumulators that were still being read.
+            if (half >= nz && ok) ok = __all_sync(0xffffffffu, tc::mbar_wait(&accf[buf][0], (it >> 1) & 1, TC_WAIT));
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&acce[buf]);

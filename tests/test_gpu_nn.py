@@ -528,3 +528,41 @@ def test_conv_tile_edges(nn, case):
     got = f64(y32)
     assert np.all(np.abs(got - ref) <= tol), np.max(np.abs(got - ref) / tol)
     assert np.array_equal(f64(y), R.bf16_round(got))
+
+
+@pytest.mark.parametrize("case", [
+    # n, d, h, w, cin, cout, relu, wrap, planes per brick (0: as chosen).  The blocks share 152 SMs with the output
+    # tiles, so that many output channels leave each block five bricks and more of a box the reference can do.
+    (3, 1, 17, 84, 16, 448, 0, 1, 0),   # boxes and bricks of one plane, one chunk of input channels
+    (3, 1, 17, 57, 80, 448, 1, 6, 0),   # and two
+    (2, 9, 4, 89, 16, 448, 0, 0, 0),    # bricks of 4 planes, the last of one
+    (2, 9, 4, 59, 80, 448, 0, 4, 0),    # and two chunks
+    (2, 33, 4, 71, 16, 256, 1, 0, 0),   # bricks of 8 planes, the last of one
+    (1, 9, 33, 33, 16, 256, 0, 2, 1),   # every brick one plane
+    (3, 32, 4, 27, 16, 448, 0, 5, 0),   # whole bricks of 8 planes
+    (3, 10, 7, 52, 80, 448, 0, 0, 0),   # two chunks through a ring of two stages
+    (3, 9, 50, 81, 32, 128, 0, 3, 0),   # bricks of up to 16 planes
+])
+def test_conv_several_bricks_per_block(nn, case):
+    """The convolution where each block works through several bricks: both accumulator sets in turn, weights kept or
+    loaded anew, stages used again, bricks of one plane among them.  The tolerance is that of the cases above."""
+    n, d, h, w, cin, cout, relu, wrap, planes = case
+    rng = np.random.default_rng(29 + hash(case) % 2**31)
+    x = rand_bf16(rng, (n, d, h, w, cin))
+    wt = rand_bf16(rng, (27, cin, cout), 1.0 / np.sqrt(27 * cin))
+    b = rng.normal(0, 0.1, cout).astype(np.float32)
+    y = torch.empty((n, d, h, w, cout), dtype=torch.bfloat16, device="cuda")
+    y32 = torch.full((n, d, h, w, cout), float("nan"), dtype=torch.float32, device="cuda")
+    try:
+        nn.lbm_nn_conv_tune(planes, 0)
+        nn.lbm_nn_conv3d(bf16_dev(x), n, d, h, w, cin, bf16_dev(wt), torch.from_numpy(b).cuda(), cout, relu, wrap, y,
+                         y32)
+        torch.cuda.synchronize()
+    finally:
+        nn.lbm_nn_conv_tune(0, 0)
+    assert nn.lbm_nn_tc_timeouts() == 0
+    ref = R.conv3d(x, wt, b.astype(np.float64), bool(relu), wrap)
+    tol = 2.0 ** -16 * R.conv3d(np.abs(x), np.abs(wt), np.abs(b.astype(np.float64)), False, wrap) + 1e-30
+    got = f64(y32)
+    assert np.all(np.abs(got - ref) <= tol), np.max(np.abs(got - ref) / tol)
+    assert np.array_equal(f64(y), R.bf16_round(got))
