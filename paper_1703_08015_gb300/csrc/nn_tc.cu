@@ -136,14 +136,15 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const bf16* __restrict__ A, con
 
 // 16 output channels from co0 of one voxel: their bias (in shared memory), ReLU,
 // and the stores that the tensors allow (vy: 16 bytes of y, vy32: 16 bytes of y32, else value by value);
-// `at`: offset of (voxel, co0).  NaN where the sums are not there.
+// `at`: offset of (voxel, co0).  NaN where the sums are not there, with or without ReLU.
 __device__ __forceinline__ void conv_out(float (&v)[16], bool ok, const float* bias, int relu, int co0,
                                          int Cout, size_t at, bool vy, bool vy32, bf16* __restrict__ y,
                                          float* __restrict__ y32) {
 #pragma unroll
     for (int k = 0; k < 16; k++) {
-        v[k] = ok ? v[k] + bias[k] : __int_as_float(0x7fc00000);
+        v[k] += bias[k];
         if (relu) v[k] = fmaxf(v[k], 0.f);
+        if (!ok) v[k] = __int_as_float(0x7fc00000);
     }
     if (y && vy) {
 #pragma unroll
@@ -511,7 +512,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
                                                              float* __restrict__ y32) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ HaloAxes axes[2];
-    __shared__ uint64_t full[CV_STAGES], empty[CV_STAGES], wfull[9], wempty[9], accf[2][HMB_MAX], acce[2];
+    __shared__ uint64_t full[CV_STAGES], empty[CV_STAGES], wfull[9], wempty[9], accf[2][HMB_MAX], acce[2], done;
     __shared__ float sbias[64];
     __shared__ uint32_t tmem_slot;
     __shared__ int stop[2];
@@ -537,6 +538,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
             for (int m = 0; m < sh.mb; m++) tc::mbar_init(&accf[s][m], 1);
             tc::mbar_init(&acce[s], CV_EPI / 32);
         }
+        tc::mbar_init(&done, 1);
         stop[0] = stop[1] = 0;
     }
     tc::fence_before_sync();
@@ -604,6 +606,10 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
                 if (fresh) wph ^= 1;
             }
         }
+        // whatever ran out, the MMAs issued are over before the block gives up its TMEM and shared memory
+        if (tc::elect_one()) tc::mma_commit(&done);
+        __syncwarp();
+        ok = (wait(&done, 0) || wait(&done, 0)) && ok;
     } else if (warp <= CV_EPI / 32) {
         const int quad = warp & 3, half = (warp - 1) >> 2, r = quad * 32 + lane;
         int it = 0;
@@ -682,7 +688,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
         hand_over_all();
         ok &= !stopped;
     } else {
-        uint32_t ph = 0;
+        uint32_t ph = 0, copies = 0;  // to the slots, in turn
         bool again = false;
         const uint4* tile = wpack ? wpack + (size_t)blockIdx.y * 27 * sh.nt * (Cin / 8) : nullptr;
         for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
@@ -690,7 +696,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
             for (int c = 0; c < sh.chunks && ok; c++) {
                 const int c0 = c * CV_CC, cc = Cin - c0 < CV_CC ? Cin - c0 : CV_CC;
                 const int units = 3 * sh.nt * (cc / 8);  // of a slot
-                for (int t9 = 0; t9 < 9; t9++) {
+                for (int t9 = 0; t9 < 9; t9++, copies++) {
                     if (again && !(ok = __all_sync(0xffffffffu, tc::mbar_wait(&wempty[t9], ph, TC_WAIT)))) break;
                     unsigned char* slot = smem + t9 * sh.slot_bytes;
                     if (wpack) {
@@ -711,7 +717,9 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
                 again = true;
             }
         }
-        // bulk copies in flight land before the block ends: the MMAs that wait for them are waited for below
+        // bulk copies in flight land before the block ends, also when no MMA waits for them any more
+        for (uint32_t c = copies < 9 ? 0 : copies - 9; c < copies; c++)
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&wfull[c % 9], (c / 9) & 1, TC_WAIT)) && ok;
     }
     if (!ok && lane == 0) atomicAdd(&g_tc_timeouts, 1u);
     tc::fence_before_sync();
@@ -806,7 +814,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_few(const bf16* __restrict__ x, i
             }
             tc::fence_smem_to_async();
             __syncthreads();
-            if (tid == 0) {
+            if (tid == 0 && ok) {
                 tc::fence_after_sync();
                 const uint32_t a0 = tc::smem_u32(smem), b0 = tc::smem_u32(sb);
 #pragma unroll
@@ -815,8 +823,8 @@ __global__ void __launch_bounds__(TC_M) k_conv_few(const bf16* __restrict__ x, i
                                  tc::smem_desc(b0 + 2 * j * TC_KGAP, TC_KGAP, RGAP), idesc, j > 0);
                 tc::mma_commit(&mbar);
             }
-            if (ok) ok = __all_sync(0xffffffffu, tc::mbar_wait(&mbar, ph, TC_WAIT));
-            ph ^= 1;
+            bool landed = ok;
+            if (ok) landed = __all_sync(0xffffffffu, tc::mbar_wait(&mbar, ph, TC_WAIT));
             tc::fence_after_sync();
             const size_t at = ((((size_t)b.n * D + b.z0 + z) * H + vy_) * W + vx) * Cout;
             for (int q = 0; q < nt; q += 16) {
@@ -824,14 +832,20 @@ __global__ void __launch_bounds__(TC_M) k_conv_few(const bf16* __restrict__ x, i
                 __syncwarp();
                 tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)q, v);
                 if (vx < W && vy_ < H && n0 + q < Cout)
-                    conv_out(v, ok, sbias + q, relu, n0 + q, Cout, at + n0 + q, vy, vy32, y, y32);
+                    conv_out(v, landed, sbias + q, relu, n0 + q, Cout, at + n0 + q, vy, vy32, y, y32);
             }
             tc::fence_before_sync();
-            __syncthreads();  // the rows and the accumulator are free
+            // the rows and the accumulator are free; a wait that ran out in any warp stops the MMAs
+            ok = __syncthreads_and(landed);
+            if (ok) ph ^= 1;
             tc::fence_after_sync();
         }
     }
-    if (!ok && lane == 0) atomicAdd(&g_tc_timeouts, 1u);
+    if (!ok) {  // the last MMAs issued may still run
+        (void)tc::mbar_wait(&mbar, ph, TC_WAIT);
+        if (lane == 0) atomicAdd(&g_tc_timeouts, 1u);
+        __syncthreads();
+    }
     if (warp == 0) tc::tmem_dealloc(tmem, ncols);
 }
 
