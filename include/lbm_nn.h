@@ -35,7 +35,10 @@ extern "C" {
  * which are periodic.  Output BF16 (y) and/or FP32 (y32); either may be NULL.
  * Any cout (output channels are tiled over the grid).  The backward-data pass
  * is this same call on dy with the weights from lbm_nn_weight_flip and the
- * same `wrap`. */
+ * same `wrap`.  For cin % 16 == 0 the weights are repacked into device memory
+ * that the call takes and gives back in the order of its stream, so calls may
+ * overlap on different streams, host threads and devices, and may be captured
+ * into a graph (whose memory nodes then hold them). */
 int lbm_nn_conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt,
                   const float* bias, int cout, int relu, int wrap, void* y, float* y32, void* stream);
 

@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 
 #include <cstdint>
+#include <mutex>
 #include <type_traits>
 
 #include "internal.h"
@@ -1230,10 +1231,65 @@ extern "C" int lbm_nn_gemm_bf16(const void* a, const void* b, float* c, int m, i
 namespace lbm {
 namespace nn {
 static int g_halo_mb = 0, g_halo_nt = 0;  // fixed by lbm_nn_conv_tune; 0 = chosen per shape
-// The convolution's weights packed as its slots (k_pack_weights): kept for
-// the process, grown on demand; calls on one stream reuse it in order.
-static uint4* g_wpack = nullptr;
-static size_t g_wpack_bytes = 0;
+
+// Device memory of one call, in the order of its stream: taken before the kernel
+// that writes it, given back behind the one that reads it.  Calls on other
+// streams, threads and devices have memory of their own, and a call under capture
+// leaves the two as nodes of its graph.  It comes from a pool per device that
+// keeps up to kPoolKeep bytes between calls and gives back what is beyond them
+// when the device is next synchronised.  NULL where there is no room.
+class StreamBuffer {
+public:
+    StreamBuffer(size_t bytes, cudaStream_t s) : stream_(s) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(s, &cap);
+        cudaMemPool_t pool = nullptr;
+        if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone)
+            e = cudaMallocAsync(&p_, bytes, s);  // the graph's own memory, whatever the pool
+        else if (e == cudaSuccess && (e = pool_of_device(&pool)) == cudaSuccess)
+            e = cudaMallocFromPoolAsync(&p_, bytes, pool, s);
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();
+            p_ = nullptr;
+        }
+    }
+    ~StreamBuffer() {
+        if (p_) (void)cudaFreeAsync(p_, stream_);
+    }
+    StreamBuffer(const StreamBuffer&) = delete;
+    StreamBuffer& operator=(const StreamBuffer&) = delete;
+    void* get() const { return p_; }
+
+private:
+    static constexpr uint64_t kPoolKeep = 64ull << 20;
+    static cudaError_t pool_of_device(cudaMemPool_t* pool) {
+        static std::mutex lock;
+        static cudaMemPool_t pools[64] = {};
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev >= 64) return cudaErrorInvalidDevice;
+        std::lock_guard<std::mutex> hold(lock);
+        if (!pools[dev]) {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t made = nullptr;
+            e = cudaMemPoolCreate(&made, &props);
+            if (e != cudaSuccess) return e;
+            uint64_t keep = kPoolKeep;
+            int no = 0;  // memory of another stream is taken once that stream is past it, never by waiting for it
+            (void)cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+            (void)cudaMemPoolSetAttribute(made, cudaMemPoolReuseAllowInternalDependencies, &no);
+            pools[dev] = made;
+        }
+        *pool = pools[dev];
+        return cudaSuccess;
+    }
+    void* p_ = nullptr;
+    cudaStream_t stream_;
+};
 
 static int sm_count() {
     static int sms = 0;
@@ -1340,21 +1396,13 @@ int conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt, 
     const CvShape sh = cv_pick(n, d, h, w, cin, cout, &gx);
     const long long gy = sh.nt ? (cout + sh.nt - 1) / sh.nt : 0;
     if (gy < 1 || gy > 65535) return fail(LBM_ERR_ARG, "convolution: %d output channels exceed the grid", cout);
+    // the weights packed as the blocks' slots; no room for them: the blocks gather them
     const size_t units = (size_t)gy * 27 * sh.nt * (cin / 8);
-    if (units * 16 > g_wpack_bytes) {
-        if (g_wpack) cudaFree(g_wpack);
-        g_wpack = nullptr;
-        g_wpack_bytes = 0;
-        if (cudaMalloc(&g_wpack, units * 16) == cudaSuccess) {
-            g_wpack_bytes = units * 16;
-        } else {  // no room: the blocks gather the weights
-            (void)cudaGetLastError();
-            g_wpack = nullptr;
-        }
-    }
-    if (g_wpack) {
+    const StreamBuffer packed(units * 16, s);
+    uint4* const wpack = static_cast<uint4*>(packed.get());
+    if (wpack) {
         k_pack_weights<<<(unsigned)((units + 127) / 128 < 1216 ? (units + 127) / 128 : 1216), 128, 0, s>>>(
-            static_cast<const bf16*>(wgt), cin, cout, sh.nt, (int)gy, g_wpack);
+            static_cast<const bf16*>(wgt), cin, cout, sh.nt, (int)gy, wpack);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "k_pack_weights launch");
     }
@@ -1362,7 +1410,7 @@ int conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt, 
         int rc = tc_launch_ok((const void*)kern, sh.smem, "cudaFuncSetAttribute(k_conv_halo)");
         if (rc) return rc;
         kern<<<dim3((unsigned)gx, (unsigned)gy), CV_THREADS, sh.smem, s>>>(
-            static_cast<const bf16*>(x), n, d, h, w, cin, static_cast<const bf16*>(wgt), g_wpack, bias, cout, relu, wrap, sh,
+            static_cast<const bf16*>(x), n, d, h, w, cin, static_cast<const bf16*>(wgt), wpack, bias, cout, relu, wrap, sh,
             vy, vy32, static_cast<bf16*>(y), y32);
         const cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_conv_halo launch");

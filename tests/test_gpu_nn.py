@@ -566,3 +566,64 @@ def test_conv_several_bricks_per_block(nn, case):
     got = f64(y32)
     assert np.all(np.abs(got - ref) <= tol), np.max(np.abs(got - ref) / tol)
     assert np.array_equal(f64(y), R.bf16_round(got))
+
+
+def _conv_inputs(rng, n, side, cin, cout):
+    x = torch.randn(n, side, side, side, cin, device="cuda", generator=rng).bfloat16()
+    w = (torch.randn(27, cin, cout, device="cuda", generator=rng) / np.sqrt(27 * cin)).bfloat16()
+    return x, w, torch.full((n, side, side, side, cout), float("nan"), device="cuda")
+
+
+@pytest.mark.parametrize("cin,cout", [(16, 4), (16, 16), (32, 64), (80, 36)])
+def test_conv_on_two_streams_at_once(nn, cin, cout):
+    """Convolutions with different weights that wait on two streams and then run at once: each the bits of its call
+    alone."""
+    rng = torch.Generator(device="cuda").manual_seed(31 + cin + cout)
+    n, side = 2, 24
+    calls = [_conv_inputs(rng, n, side, cin, cout) for _ in range(8)]
+
+    def conv(x, w, y, stream):
+        nn.lbm_nn_conv3d(x, n, side, side, side, cin, w, None, cout, 0, 1, None, y, stream.cuda_stream)
+
+    main = torch.cuda.current_stream()
+    alone = []
+    for x, w, y in calls:
+        conv(x, w, y, main)
+        torch.cuda.synchronize()
+        alone.append(y.clone())
+        y.fill_(float("nan"))
+    gate, streams = torch.cuda.Event(), (torch.cuda.Stream(), torch.cuda.Stream())
+    torch.cuda._sleep(20_000_000)  # both queues fill behind it
+    gate.record(main)
+    for s in streams:
+        s.wait_event(gate)
+    for k, (x, w, y) in enumerate(calls):
+        conv(x, w, y, streams[k % 2])
+    torch.cuda.synchronize()
+    assert nn.lbm_nn_tc_timeouts() == 0
+    for (x, w, y), want in zip(calls, alone):
+        assert torch.equal(y, want)
+
+
+def test_conv_captured_into_a_graph(nn):
+    """A first call of its size under capture, and the graph's replay after calls with other and larger weights: the
+    bits of the plain call."""
+    rng = torch.Generator(device="cuda").manual_seed(37)
+    n, side = 1, 12
+    x, w, y = _conv_inputs(rng, n, side, 208, 240)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        nn.lbm_nn_conv3d(x, n, side, side, side, 208, w, None, 240, 0, 1, None, y,
+                         torch.cuda.current_stream().cuda_stream)
+    x2, w2, y2 = _conv_inputs(rng, n, side, 256, 320)
+    nn.lbm_nn_conv3d(x2, n, side, side, side, 256, w2, None, 320, 0, 1, None, y2)
+    for _ in range(2):
+        y.fill_(float("nan"))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        got = y.clone()
+        nn.lbm_nn_conv3d(x, n, side, side, side, 208, w, None, 240, 0, 1, None, y)
+        torch.cuda.synchronize()
+        assert torch.equal(got, y)
+    assert nn.lbm_nn_tc_timeouts() == 0
