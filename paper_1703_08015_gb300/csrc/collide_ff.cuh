@@ -178,16 +178,11 @@ constexpr int ff_first_of_class() {
     return i;
 }
 
-// The node's update in native FP64 (the range fallback of the float-float and
-// fixed-point steps): the words are gathered again, collided and stored.  Not
-// inlined: as a call its registers stay off the step's hot path (inline, the
-// FP64 update held enough registers to spill the whole D3Q19 step).
-template <class L, int A, int MODEL, int KMAX>
-__device__ __noinline__ void update_fp64(const NeighShared<Tile<L, A>, KMAX>& sh, const StepArgs& a,
-                                            const WorkNode& wn, const NodePos<A>& p, unsigned long long* out,
-                                            int stride) {
-    unsigned long long b[L::Q];
-    gather<L, A, KMAX, unsigned long long>(sh, a.src, wn.lt, wn.node, p, b);
+// The update in native FP64 from the gathered words (the range fallback of the
+// float-float and fixed-point steps).
+template <class L, int MODEL>
+__device__ __forceinline__ void store_fp64(const unsigned long long (&b)[L::Q], const StepArgs& a,
+                                           unsigned long long* out, int stride) {
     double f[L::Q];
     static_for<0, L::Q>([&](auto I) { f[decltype(I)::value] = __longlong_as_double((long long)b[decltype(I)::value]); });
     collide_f64<L, MODEL>(f, a.omega, a.force);
@@ -197,20 +192,16 @@ __device__ __noinline__ void update_fp64(const NeighShared<Tile<L, A>, KMAX>& sh
     });
 }
 
-// update_fp64 for the steps that stage neighbour records (gather_rec).
+// The node's update in native FP64: the words are gathered again, collided and
+// stored.  Not inlined: as a call its registers stay off the step's hot path
+// (inline, the FP64 update held enough registers to spill the whole D3Q19 step).
 template <class L, int A, int MODEL, int KMAX>
-__device__ __noinline__ void update_fp64_rec(const RecShared<Tile<L, A>, KMAX>& sh, const StepArgs& a,
-                                             const WorkNode& wn, const NodePos<A>& p) {
+__device__ __noinline__ void update_fp64(const NeighShared<Tile<L, A>, KMAX>& sh, const StepArgs& a,
+                                            const WorkNode& wn, const NodePos<A>& p, unsigned long long* out,
+                                            int stride) {
     unsigned long long b[L::Q];
-    int stride;
-    unsigned long long* out = gather_rec<L, A, KMAX, unsigned long long>(sh, a.src, a.dst, wn.lt, wn.node, p, b, stride);
-    double f[L::Q];
-    static_for<0, L::Q>([&](auto I) { f[decltype(I)::value] = __longlong_as_double((long long)b[decltype(I)::value]); });
-    collide_f64<L, MODEL>(f, a.omega, a.force);
-    static_for<0, L::Q>([&](auto I) {
-        constexpr int i = decltype(I)::value;
-        out[i * stride] = (unsigned long long)__double_as_longlong(f[i]);
-    });
+    gather<L, A, KMAX, unsigned long long>(sh, a.src, wn.lt, wn.node, p, b);
+    store_fp64<L, MODEL>(b, a, out, stride);
 }
 
 // ---- two float-float numbers at once (f32x2) ------------------------------------
@@ -398,8 +389,12 @@ constexpr int link_comp() {
     return X == 0 ? Link<L, I>::cx : (X == 1 ? Link<L, I>::cy : (X == 2 ? Link<L, I>::cz : 0));
 }
 
+// What collide_ff made of a node: its results stored, or the words that arrived
+// out of range (nothing stored), or a result (some may be stored).
+enum class FFRange { ok, input, result };
+
 template <class L, int MODEL, int FAX = -1, bool WIDE = false>
-__device__ __forceinline__ bool collide_ff(const unsigned long long (&b)[L::Q], const FixedConsts& k,
+__device__ __forceinline__ FFRange collide_ff(const unsigned long long (&b)[L::Q], const FixedConsts& k,
                                            const FFConsts& c, unsigned long long* out, int stride) {
     constexpr int Q = L::Q;
     static_assert(ulps_to_binade_edge(L::wc_[0]) >= 281474976710656.0 &&
@@ -438,7 +433,7 @@ __device__ __forceinline__ bool collide_ff(const unsigned long long (&b)[L::Q], 
     const long long jy = k.half_f[1] + (sy[1] << S1) + (sy[2] << S2);
     const long long jz = k.half_f[2] + (sz[1] << S1) + (sz[2] << S2);
     ok &= small_ll(dr, 55) & small_ll(jx, 56) & small_ll(jy, 56) & small_ll(jz, 56);
-    if (!ok) return false;
+    if (!ok) return FFRange::input;
 
     // (j_x, j_y) side by side: the first group's c_i . p of its two pairs
     const ff2 JXY = q60_to_ff_2(jx, jy);
@@ -564,32 +559,64 @@ __device__ __forceinline__ bool collide_ff(const unsigned long long (&b)[L::Q], 
         class_consts(c.w22, c.rho22, VV, CC);
         static_for<1, GR::n>([&](auto G) { group(G, VV, CC); });
     }
-    return ok;
+    return ok ? FFRange::ok : FFRange::result;
 }
 
-// The update of a node whose float-float results reach 2^46 ulps, which
-// collide_ff's rounding does not take: the same arithmetic with the wider
-// rounding, and native FP64 only beyond that (or where an input is out of
-// range).  Nodes of closed pores that keep the momentum of the starting field
-// stay there for the whole run, and one of them held its block for 600 FP64
-// instructions: 128^2 nodes in 2D 10.6 to 5.9 us per step, a 64^3 sample 18.6 to
-// 11.8, 128^3 in place 91.3 to 81.1.
+// The update of a node out of collide_ff's range (r).  A result of 2^46 ulps or
+// more: the same arithmetic with the wider rounding, native FP64 beyond that; an
+// input out of range, which the wider rounding does not take either: native FP64
+// at once.  Nodes of closed pores that keep the momentum of the starting field
+// stay in the wider range for the whole run, and one of them held its block for
+// 600 FP64 instructions: 128^2 nodes in 2D 10.6 to 5.9 us per step, a 64^3 sample
+// 18.6 to 11.8, 128^3 in place 91.3 to 81.1.  With the wider rounding tried on
+// inputs out of range as well, flows of |u| = 0.02 took 1 to 2.4 % longer (64^3
+// nodes 190.7 us per step, now 188.5; in 8^3 tiles 231 and 225).
+//
+// As calls, so that their registers do not weigh on the step, and as one call site:
+// the nodes of a warp that need either FP64 or the wider rounding then go through
+// one FP64 update together (one site for each took 70 us where this takes 53).
 template <class L, int A, int MODEL, int KMAX>
-__device__ __noinline__ void update_wide(const NeighShared<Tile<L, A>, KMAX>& sh, const StepArgs& a, const WorkNode& wn,
-                                         const NodePos<A>& p, unsigned long long* out, int stride) {
+__device__ __forceinline__ bool wide_result(const NeighShared<Tile<L, A>, KMAX>& sh, const StepArgs& a,
+                                            const WorkNode& wn, const NodePos<A>& p, unsigned long long* out, int stride) {
     unsigned long long b[L::Q];
     gather<L, A, KMAX, unsigned long long>(sh, a.src, wn.lt, wn.node, p, b);
-    if (!collide_ff<L, MODEL, -1, true>(b, a.fx, a.ffc, out, stride))
-        update_fp64<L, A, MODEL, KMAX>(sh, a, wn, p, out, stride);
+    return collide_ff<L, MODEL, -1, true>(b, a.fx, a.ffc, out, stride) == FFRange::ok;
 }
 
 template <class L, int A, int MODEL, int KMAX>
-__device__ __noinline__ void update_wide_rec(const RecShared<Tile<L, A>, KMAX>& sh, const StepArgs& a, const WorkNode& wn,
-                                             const NodePos<A>& p) {
+__device__ __noinline__ bool update_wide(const NeighShared<Tile<L, A>, KMAX>& sh, const StepArgs& a, const WorkNode& wn,
+                                         const NodePos<A>& p, unsigned long long* out, int stride) {
+    return wide_result<L, A, MODEL, KMAX>(sh, a, wn, p, out, stride);
+}
+
+template <class L, int A, int MODEL, int KMAX>
+__device__ __noinline__ void update_out_of_range(const NeighShared<Tile<L, A>, KMAX>& sh, const StepArgs& a,
+                                                 const WorkNode& wn, const NodePos<A>& p, unsigned long long* out,
+                                                 int stride, FFRange r) {
+    if (r == FFRange::result && wide_result<L, A, MODEL, KMAX>(sh, a, wn, p, out, stride)) return;
+    update_fp64<L, A, MODEL, KMAX>(sh, a, wn, p, out, stride);
+}
+
+// The same for the steps that stage neighbour records (gather_rec).
+template <class L, int A, int MODEL, int KMAX>
+__device__ __noinline__ void update_fp64_rec(const RecShared<Tile<L, A>, KMAX>& sh, const StepArgs& a,
+                                             const WorkNode& wn, const NodePos<A>& p) {
     unsigned long long b[L::Q];
     int stride;
     unsigned long long* out = gather_rec<L, A, KMAX, unsigned long long>(sh, a.src, a.dst, wn.lt, wn.node, p, b, stride);
-    if (!collide_ff<L, MODEL, -1, true>(b, a.fx, a.ffc, out, stride)) update_fp64_rec<L, A, MODEL, KMAX>(sh, a, wn, p);
+    store_fp64<L, MODEL>(b, a, out, stride);
+}
+
+template <class L, int A, int MODEL, int KMAX>
+__device__ __noinline__ void update_out_of_range_rec(const RecShared<Tile<L, A>, KMAX>& sh, const StepArgs& a,
+                                                     const WorkNode& wn, const NodePos<A>& p, FFRange r) {
+    if (r == FFRange::result) {
+        unsigned long long b[L::Q];
+        int stride;
+        unsigned long long* out = gather_rec<L, A, KMAX, unsigned long long>(sh, a.src, a.dst, wn.lt, wn.node, p, b, stride);
+        if (collide_ff<L, MODEL, -1, true>(b, a.fx, a.ffc, out, stride) == FFRange::ok) return;
+    }
+    update_fp64_rec<L, A, MODEL, KMAX>(sh, a, wn, p);
 }
 
 }  // namespace lbm

@@ -127,9 +127,9 @@ __device__ __forceinline__ int gather_tgb(const NeighShared<Tile<L, A>, KMAX>& s
     return own_rank;
 }
 
-// The q FP64 words of a node's update in native FP64, for the nodes outside
-// the range of the float-float arithmetic: a call rather than inline code, so
-// that its registers do not weigh on the step.
+// The q FP64 words of the update of a node outside the range of the
+// float-float arithmetic (update_out_of_range): a call rather than inline code,
+// so that its registers do not weigh on the step.
 template <int Q>
 struct Words {
     unsigned long long v[Q];
@@ -142,25 +142,23 @@ __device__ __noinline__ Words<L::Q> tgb_update_fp64(const NeighShared<Tile<L, A>
     unsigned long long raw[L::Q];
     gather_tgb<L, A, KMAX, unsigned long long>(sh, nbt, static_cast<const unsigned long long*>(a.dst),
                                                static_cast<const unsigned long long*>(a.ghost_in), lt, node, p, raw);
-    double f[L::Q];
-    static_for<0, L::Q>([&](auto I) { f[decltype(I)::value] = __longlong_as_double((long long)raw[decltype(I)::value]); });
-    collide_f64<L, MODEL>(f, a.omega, a.force);
     Words<L::Q> w;
-    static_for<0, L::Q>([&](auto I) { w.v[decltype(I)::value] = (unsigned long long)__double_as_longlong(f[decltype(I)::value]); });
+    store_fp64<L, MODEL>(raw, a, w.v, 1);
     return w;
 }
 
-// The same with the float-float arithmetic's wider rounding first (update_wide).
 template <class L, int A, int MODEL, int KMAX>
-__device__ __noinline__ Words<L::Q> tgb_update_wide(const NeighShared<Tile<L, A>, KMAX>& sh,
-                                                    const int (&nbt)[KMAX][Tile<L, A>::NN], const StepArgs& a, int lt,
-                                                    int node, const NodePos<A>& p) {
-    unsigned long long raw[L::Q];
-    gather_tgb<L, A, KMAX, unsigned long long>(sh, nbt, static_cast<const unsigned long long*>(a.dst),
-                                               static_cast<const unsigned long long*>(a.ghost_in), lt, node, p, raw);
-    Words<L::Q> w;
-    if (!collide_ff<L, MODEL, -1, true>(raw, a.fx, a.ffc, w.v, 1)) w = tgb_update_fp64<L, A, MODEL, KMAX>(sh, nbt, a, lt, node, p);
-    return w;
+__device__ __noinline__ Words<L::Q> tgb_update_out_of_range(const NeighShared<Tile<L, A>, KMAX>& sh,
+                                                            const int (&nbt)[KMAX][Tile<L, A>::NN], const StepArgs& a,
+                                                            int lt, int node, const NodePos<A>& p, FFRange r) {
+    if (r == FFRange::result) {
+        unsigned long long raw[L::Q];
+        gather_tgb<L, A, KMAX, unsigned long long>(sh, nbt, static_cast<const unsigned long long*>(a.dst),
+                                                   static_cast<const unsigned long long*>(a.ghost_in), lt, node, p, raw);
+        Words<L::Q> w;
+        if (collide_ff<L, MODEL, -1, true>(raw, a.fx, a.ffc, w.v, 1) == FFRange::ok) return w;
+    }
+    return tgb_update_fp64<L, A, MODEL, KMAX>(sh, nbt, a, lt, node, p);
 }
 
 // Resident blocks per SM requested (register cap) for each arithmetic.
@@ -203,8 +201,9 @@ __global__ void __launch_bounds__(work_threads<L, A>(), tgb_min_blocks<L, A, ARI
             static_for<0, L::Q>([&](auto I) { vals[decltype(I)::value] = IO::template raw<decltype(I)::value>(g[decltype(I)::value], a); });
         } else {
             if constexpr (ARITH == 1) {
-                if (!collide_ff<L, MODEL>(raw, a.fx, a.ffc, vals, 1)) {
-                    const Words<L::Q> w = tgb_update_wide<L, A, MODEL, work_tiles()>(sh, nbt, a, lt, node, p);
+                const FFRange r = collide_ff<L, MODEL>(raw, a.fx, a.ffc, vals, 1);
+                if (r != FFRange::ok) {
+                    const Words<L::Q> w = tgb_update_out_of_range<L, A, MODEL, work_tiles()>(sh, nbt, a, lt, node, p, r);
                     static_for<0, L::Q>([&](auto I) { vals[decltype(I)::value] = w.v[decltype(I)::value]; });
                 }
             } else {

@@ -454,3 +454,35 @@ def test_fp64_fallback_far_from_equilibrium(oracle, arith):
         s.close()
     ref = oracle.run(19, mask, per, tau, F, oracle.init(19, mask, rho=rho, u=u), steps)
     assert max_rel(gpu, ref, mask) <= TOL
+
+
+@pytest.mark.parametrize("lattice,a,model", [(19, 4, 0), (19, 8, 1), (9, 8, 0), (9, 16, 1)])
+def test_fp64_ranges_in_every_float_float_form(oracle, lattice, a, model):
+    """Velocities from 0 to 0.02 bring nodes to each branch of the float-float update (the fast rounding, the wider
+    one for results of 2^46 ulps and more, native FP64): the staged step, the gather table and the in-place form take
+    the same one at every node, bit for bit, and stay within the bar of the oracle."""
+    _cuda()
+    if lattice == 19:
+        mask, _ = geo.sphere_pack_3d(shape=(24, 22, 18), seed=12, r_min=2, r_max=4, target_fluid=0.55)
+    else:
+        mask, _ = geo.circles_2d(80, 50, seed=5, max_attempts=400)
+    shape = mask.shape
+    ny = shape[1]
+    u = np.zeros((3 if lattice == 19 else 2,) + shape)
+    u[0] = (0.02 * np.arange(ny) / (ny - 1))[None, :, None]
+    rho = 1.0 + 0.0005 * np.cos(2 * np.pi * np.arange(shape[2]) / shape[2])[None, None, :] * np.ones(shape)
+    per, tau, F, steps = (1, 0, 0), 0.7, (1e-5, 0, 0), 25
+    got = []
+    for kw in (dict(arith=lbm.LBM_ARITH_FF), dict(arith=lbm.LBM_ARITH_FF_TABLE),
+               dict(arith=lbm.LBM_ARITH_FF, layout=lbm.LBM_LAYOUT_TGB)):
+        s = lbm.Solver(mask, lattice, a, per, tau, F, model=model, rho_init=rho, u_init=u, **kw)
+        try:
+            s.step(steps)
+            got.append(s.export_pdfs())
+        finally:
+            s.close()
+    ref = oracle.run(lattice, mask, per, tau, F, oracle.init(lattice, mask, model=model, rho=rho, u=u), steps, model=model)
+    assert max_rel(got[0], ref, mask) <= TOL
+    fl = np.asarray(mask).astype(bool)
+    for other in got[1:]:
+        assert np.array_equal(got[0][:, fl], other[:, fl])
