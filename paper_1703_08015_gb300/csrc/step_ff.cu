@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(BT, MINB) k_step_ff(const StepArgs a) {
     } else {
         __shared__ NeighShared<TL, work_tiles()> sh;
         WorkNode wn;
-        if (!stage_work<TL, work_tiles(), BT>(sh, a, wn)) return;
+        if (!stage_work<TL, work_tiles(), BT, true>(sh, a, wn)) return;
         const NodePos<A> p = node_pos<TL>(wn.node);
         T b[L::Q];
         const int rank = gather<L, A, work_tiles(), T>(sh, a.src, wn.lt, wn.node, p, b);

@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(work_threads<L, A>()) k_gather_table(const Ste
     using TL = Tile<L, A>;
     __shared__ NeighShared<TL, work_tiles()> sh;
     WorkNode wn;
-    if (!stage_work<TL, work_tiles(), work_threads<L, A>()>(sh, a, wn)) return;
+    if (!stage_work<TL, work_tiles(), work_threads<L, A>(), false>(sh, a, wn)) return;
     const long long pos = (long long)a.blocks[blockIdx.x].node_begin + threadIdx.x;
     const long long P = a.gtab_pitch;
     const NodePos<A> p = node_pos<TL>(wn.node);

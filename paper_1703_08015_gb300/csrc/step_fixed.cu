@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(work_threads<L, A>(), MINB) k_step_fixed(const
     using T = unsigned long long;
     __shared__ NeighShared<TL, work_tiles()> sh;
     WorkNode wn;
-    if (!stage_work<TL, work_tiles(), work_threads<L, A>()>(sh, a, wn)) return;
+    if (!stage_work<TL, work_tiles(), work_threads<L, A>(), true>(sh, a, wn)) return;
     const NodePos<A> p = node_pos<TL>(wn.node);
     T b[L::Q];
     const int rank = gather<L, A, work_tiles(), T>(sh, a.src, wn.lt, wn.node, p, b);

@@ -319,8 +319,10 @@ __device__ __forceinline__ void stage_tables(NeighShared<TL, KMAX>& sh, const St
 
 // Stage the neighbourhoods of the block's tiles, then decode this thread's
 // fluid node.  Every thread of the block must call it (it holds the barrier);
-// returns false for threads beyond the block's node count.
-template <class TL, int KMAX, int BT, bool CHAIN = true>
+// returns false for threads beyond the block's node count.  CHAIN: a step kernel
+// launched while its predecessor runs; any other kernel passes false, so that a
+// chained step behind it cannot start before what it writes is there.
+template <class TL, int KMAX, int BT, bool CHAIN>
 __device__ __forceinline__ bool stage_work_at(NeighShared<TL, KMAX>& sh, const StepArgs& a, int wbi,
                                               WorkNode& wn) {
     const WorkBlock wb = a.blocks[wbi];
@@ -336,9 +338,9 @@ __device__ __forceinline__ bool stage_work_at(NeighShared<TL, KMAX>& sh, const S
     return true;
 }
 
-template <class TL, int KMAX, int BT>
+template <class TL, int KMAX, int BT, bool CHAIN>
 __device__ __forceinline__ bool stage_work(NeighShared<TL, KMAX>& sh, const StepArgs& a, WorkNode& wn) {
-    return stage_work_at<TL, KMAX, BT>(sh, a, blockIdx.x, wn);
+    return stage_work_at<TL, KMAX, BT, CHAIN>(sh, a, blockIdx.x, wn);
 }
 
 // ---- staging from the per-tile neighbour table (tiles of one mask word) ---------
