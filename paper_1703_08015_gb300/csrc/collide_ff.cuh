@@ -592,9 +592,8 @@ __device__ __noinline__ bool update_wide(const NeighShared<Tile<L, A>, KMAX>& sh
 template <class L, int A, int MODEL, int KMAX>
 __device__ __noinline__ void update_out_of_range(const NeighShared<Tile<L, A>, KMAX>& sh, const StepArgs& a,
                                                  const WorkNode& wn, const NodePos<A>& p, unsigned long long* out,
-                                                 int stride, FFRange r) {
-    if (r == FFRange::result && wide_result<L, A, MODEL, KMAX>(sh, a, wn, p, out, stride)) return;
-    update_fp64<L, A, MODEL, KMAX>(sh, a, wn, p, out, stride);
+                                                 int stride) {
+    if (!wide_result<L, A, MODEL, KMAX>(sh, a, wn, p, out, stride)) update_fp64<L, A, MODEL, KMAX>(sh, a, wn, p, out, stride);
 }
 
 // The same for the steps that stage neighbour records (gather_rec).

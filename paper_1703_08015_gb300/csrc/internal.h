@@ -251,6 +251,30 @@ cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, 
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// Blocks of a kernel that an SM and the device hold at once.
+struct Room {
+    int per_sm, blocks;
+};
+template <class... P>
+Room room_for(void (*kernel)(P...), int threads) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
+    if (per_sm < 1) per_sm = 1;
+    return Room{per_sm, sms * per_sm};
+}
+
+// Whether a step of `blocks` blocks gains from launch_chained.  Not where it leaves a
+// little less room than the next step needs (half of the device to `from` of it): the
+// part that starts early fills some SMs and the rest then crowds on those that fall
+// free first (at 0.56, three blocks per SM: fixed point 12.5 us per step, 15.7
+// chained; in place 10.2 and 11.4).  Below, both steps fit; above, and with one
+// block per SM, chained steps measured faster.
+inline bool chain_pays(long long blocks, const Room& room, double from = 0.65) {
+    return room.per_sm == 1 || 2 * blocks <= room.blocks || blocks >= from * room.blocks;
+}
+
 // Kernel selection (nullptr when a combination is not compiled).
 StepLaunch select_step(const lbm_params* p);
 void f32_consts(const lbm_params* p, double omega, const double* force, F32Consts* k);

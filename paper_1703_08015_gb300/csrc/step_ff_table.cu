@@ -74,7 +74,9 @@ __device__ __noinline__ void update_out_of_range_table(const StepArgs& a, const 
 // 256^3 step for three blocks of 256 at 80 registers.
 constexpr int kTableThreads = 128;
 
-template <class L, int MODEL>
+// CHAIN: launched while the step before still runs, its values read with ordinary
+// loads (chain_wait).
+template <class L, int MODEL, bool CHAIN>
 __global__ void __launch_bounds__(kTableThreads, 7) k_step_ff_table(const StepArgs a) {
     using T = unsigned long long;
     const long long pos = (long long)blockIdx.x * kTableThreads + threadIdx.x;
@@ -84,11 +86,12 @@ __global__ void __launch_bounds__(kTableThreads, 7) k_step_ff_table(const StepAr
     const T* src = static_cast<const T*>(a.src);
     const int own = __ldg(t);
     T b[L::Q];
-    chain_wait();
-    b[0] = src[own];
+    if constexpr (CHAIN) chain_wait();
+    auto value = [&](int at) { return CHAIN ? src[at] : __ldg(src + at); };
+    b[0] = value(own);
     static_for<1, L::Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
-        b[i] = src[__ldg(t + i * P)];
+        b[i] = value(__ldg(t + i * P));
     });
     const int stride = __ldg(t + L::Q * P);
     T* out = static_cast<T*>(a.dst) + own;
@@ -99,7 +102,13 @@ __global__ void __launch_bounds__(kTableThreads, 7) k_step_ff_table(const StepAr
 template <class L, int MODEL>
 cudaError_t launch_step_ff_table(const StepArgs& a, cudaStream_t s) {
     if (a.n_nodes == 0) return cudaSuccess;
-    return launch_chained(k_step_ff_table<L, MODEL>, (unsigned)((a.n_nodes + kTableThreads - 1) / kTableThreads), kTableThreads, s, a);
+    const long long grid = (a.n_nodes + kTableThreads - 1) / kTableThreads;
+    // chained where two steps fit the device (24^3 to 60^3 samples 4 to 12 % faster): the step is bound by its
+    // loads, and beyond that the ordinary ones cost more (64^3: 6.8 us per step, 8.6 chained; 256^3: 337 and 347)
+    static const Room room = room_for(k_step_ff_table<L, MODEL, true>, kTableThreads);
+    if (2 * grid <= room.blocks) return launch_chained(k_step_ff_table<L, MODEL, true>, (unsigned)grid, kTableThreads, s, a);
+    k_step_ff_table<L, MODEL, false><<<(unsigned)grid, kTableThreads, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 template <class L, int A>

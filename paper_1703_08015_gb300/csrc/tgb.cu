@@ -255,7 +255,11 @@ __global__ void k_tgb_publish(const StepArgs a) {
 template <class L, int A, int MODEL, class S, int ARITH>
 cudaError_t launch_step_tgb(const StepArgs& a, cudaStream_t s) {
     if (a.n_work_blocks == 0) return cudaSuccess;
-    return launch_chained(k_step_tgb<L, A, MODEL, S, ARITH>, (unsigned)a.n_work_blocks, work_threads<L, A>(), s, a);
+    static const Room room = room_for(k_step_tgb<L, A, MODEL, S, ARITH>, work_threads<L, A>());
+    if (chain_pays(a.n_work_blocks, room))
+        return launch_chained(k_step_tgb<L, A, MODEL, S, ARITH>, (unsigned)a.n_work_blocks, work_threads<L, A>(), s, a);
+    k_step_tgb<L, A, MODEL, S, ARITH><<<a.n_work_blocks, work_threads<L, A>(), 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 template <class L, int A, class S>
