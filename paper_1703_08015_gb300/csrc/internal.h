@@ -248,7 +248,8 @@ cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, 
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    return cudaGetLastError();  // as after <<<>>>: a failed launch leaves no error behind for the next call
 }
 
 // Blocks of a kernel that an SM and the device hold at once.
