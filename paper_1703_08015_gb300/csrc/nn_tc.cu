@@ -504,7 +504,8 @@ __device__ __forceinline__ void cv_issue(uint32_t acc, uint64_t a, uint64_t b, i
 }
 
 // Grid: x = bricks (blockIdx.x, + gridDim.x, ..), y = output-channel tiles.
-// wpack NULL (no room for it): the weights' warp gathers them from wgt.
+// wpack NULL (few weights, or no room for it): weights of one chunk are gathered by
+// the whole block before it starts, those of several by the weights' warp.
 template <bool VX>
 __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restrict__ x, int N, int D, int H, int W, int Cin,
                                                              const bf16* __restrict__ wgt, const uint4* __restrict__ wpack,
@@ -542,6 +543,14 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
         tc::mbar_init(&done, 1);
         stop[0] = stop[1] = 0;
     }
+    const bool held = !wpack && sh.chunks == 1;  // the weights are in their slots when the block starts
+    if (held) {
+        const int units = 27 * sh.nt * (Cin / 8);
+#pragma unroll 2
+        for (int u = tid; u < units; u += CV_THREADS)
+            reinterpret_cast<uint4*>(smem)[u] = cv_weights(wgt, Cin, Cout, sh.nt, 0, Cin, blockIdx.y, u);
+        tc::fence_smem_to_async();
+    }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -564,7 +573,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
             if (it >= 2) ok = wait(&acce[buf], ((it >> 1) - 1) & 1);
             for (int c = 0; c < sh.chunks && ok; c++) {
                 const int cc = Cin - c * CV_CC < CV_CC ? Cin - c * CV_CC : CV_CC, ks = cc / 16;
-                const bool fresh = sh.chunks > 1 || it == 0;  // the weights' slots are filled anew
+                const bool fresh = !held && (sh.chunks > 1 || it == 0);  // the weights' slots are filled anew
                 for (int h0 = 0; h0 < nz + 2 && ok; h0 += sh.planes) {
                     if (!(ok = wait(&full[s], ph))) break;
                     tc::fence_after_sync();
@@ -692,7 +701,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
         uint32_t ph = 0, copies = 0;  // to the slots, in turn
         bool again = false;
         const uint4* tile = wpack ? wpack + (size_t)blockIdx.y * 27 * sh.nt * (Cin / 8) : nullptr;
-        for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+        for (long long t = blockIdx.x; t < tiles && ok && !held; t += gridDim.x) {
             if (again && sh.chunks == 1) break;  // the weights stay
             for (int c = 0; c < sh.chunks && ok; c++) {
                 const int c0 = c * CV_CC, cc = Cin - c0 < CV_CC ? Cin - c0 : CV_CC;
@@ -1241,6 +1250,7 @@ static int g_halo_mb = 0, g_halo_nt = 0;  // fixed by lbm_nn_conv_tune; 0 = chos
 class StreamBuffer {
 public:
     StreamBuffer(size_t bytes, cudaStream_t s) : stream_(s) {
+        if (!bytes) return;
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         cudaError_t e = cudaStreamIsCapturing(s, &cap);
         cudaMemPool_t pool = nullptr;
@@ -1380,6 +1390,13 @@ static CvShape cv_pick(int n, int d, int h, int w, int cin, int cout, int* grid_
     return best;
 }
 
+// Up to so many 16-byte units of an output tile's weights (of one chunk of input
+// channels) each block gathers them itself, eight rounds of its threads, instead of a
+// packing launch before it: 16 -> 4 channels on 8^3 voxels 17.2 and 10.9 us, 48 -> 16
+// 19.2 and 15.1, on 8 x 64^3 222 and 218; with 6912 units, 64 -> 32 on 32^3, 21.3 and
+// 23.1.
+constexpr size_t kGatherUnits = 4096;
+
 // The convolution: halo planes for cin % 16 == 0, rows put together from a halo
 // for two or four input channels, else the gathering implicit GEMM.  Any
 // channel counts and alignment (16-byte copies and stores where a tensor's
@@ -1396,9 +1413,10 @@ int conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt, 
     const CvShape sh = cv_pick(n, d, h, w, cin, cout, &gx);
     const long long gy = sh.nt ? (cout + sh.nt - 1) / sh.nt : 0;
     if (gy < 1 || gy > 65535) return fail(LBM_ERR_ARG, "convolution: %d output channels exceed the grid", cout);
-    // the weights packed as the blocks' slots; no room for them: the blocks gather them
-    const size_t units = (size_t)gy * 27 * sh.nt * (cin / 8);
-    const StreamBuffer packed(units * 16, s);
+    // The weights packed as the blocks' slots, except where a block gathers them as fast (or where there is no room).
+    const size_t per_tile = (size_t)27 * sh.nt * (cin / 8), units = gy * per_tile;
+    const bool gather = sh.chunks == 1 && per_tile <= kGatherUnits;
+    const StreamBuffer packed(gather ? 0 : units * 16, s);
     uint4* const wpack = static_cast<uint4*>(packed.get());
     if (wpack) {
         k_pack_weights<<<(unsigned)((units + 127) / 128 < 1216 ? (units + 127) / 128 : 1216), 128, 0, s>>>(

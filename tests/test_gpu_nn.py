@@ -627,3 +627,44 @@ def test_conv_captured_into_a_graph(nn):
         torch.cuda.synchronize()
         assert torch.equal(got, y)
     assert nn.lbm_nn_tc_timeouts() == 0
+
+
+def _check_conv(nn, case, offset=0):
+    """lbm_nn_conv3d against the FP64 reference on tensors that start `offset` values past a 16-byte boundary; the
+    tolerance is that of the cases above.  Returns the FP32 output."""
+    n, d, h, w, cin, cout, relu, wrap = case
+    rng = np.random.default_rng(41 + hash(case) % 2**31)
+    x = rand_bf16(rng, (n, d, h, w, cin))
+    wt = rand_bf16(rng, (27, cin, cout), 1.0 / np.sqrt(27 * cin))
+    b = rng.normal(0, 0.1, cout).astype(np.float32)
+
+    def dev(a):
+        t = torch.empty(a.size + offset, dtype=torch.bfloat16, device="cuda")
+        t[offset:] = bf16_dev(a).reshape(-1)
+        return t[offset:]
+
+    y = torch.empty(n * d * h * w * cout + offset, dtype=torch.bfloat16, device="cuda")[offset:]
+    y32 = torch.full((n * d * h * w * cout + offset,), float("nan"), dtype=torch.float32, device="cuda")[offset:]
+    nn.lbm_nn_conv3d(dev(x), n, d, h, w, cin, dev(wt), torch.from_numpy(b).cuda(), cout, relu, wrap, y, y32)
+    torch.cuda.synchronize()
+    assert nn.lbm_nn_tc_timeouts() == 0
+    ref = R.conv3d(x, wt, b.astype(np.float64), bool(relu), wrap)
+    tol = 2.0 ** -16 * R.conv3d(np.abs(x), np.abs(wt), np.abs(b.astype(np.float64)), False, wrap) + 1e-30
+    got = f64(y32).reshape(ref.shape)
+    assert np.all(np.abs(got - ref) <= tol), np.max(np.abs(got - ref) / tol)
+    assert np.array_equal(f64(y).reshape(ref.shape), R.bf16_round(got))
+    return y32
+
+
+@pytest.mark.parametrize("case", [(3, 17, 33, 41, 32, 128, 0, 1), (2, 33, 40, 70, 48, 64, 1, 0)])
+def test_conv_weights_gathered_or_packed(nn, case):
+    """Output tiles of 16 channels, whose weights each block gathers itself, and of 64, packed by a launch before:
+    the same sums, bit for bit, over several bricks per block."""
+    out = []
+    try:
+        for tile in (16, 64):
+            nn.lbm_nn_conv_tune(0, tile)
+            out.append(_check_conv(nn, case))
+    finally:
+        nn.lbm_nn_conv_tune(0, 0)
+    assert torch.equal(out[0], out[1])
