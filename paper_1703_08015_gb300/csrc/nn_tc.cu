@@ -748,18 +748,19 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv_halo(const bf16* __restr
 // the chain of a plane (rows, MMAs, outputs), which as many blocks as an SM
 // holds overlap; k_conv_tc spent it on the addresses of 27 CI separate loads per
 // voxel: 2 -> 16 channels on 8 x 64^3 voxels 334 and 53 us, 4 -> 16
-// 615 and 86.
-constexpr int FEW_Z = 8;
+// 615 and 86.  Small boxes take shallower columns, one plane each at the least (2 -> 16
+// on 8^3 voxels 14.7 us with eight planes to a block, now 7.4; on 24^3 16.6 and 8.5).
+constexpr int FEW_Z = 8;  // planes of a brick, at most
 __host__ __device__ constexpr int few_groups(int ci) { return (27 * ci + 15) / 16 * 2; }  // 8-value groups of a row
-__host__ __device__ constexpr uint32_t few_smem(int ci, int nt) {
-    return (uint32_t)((TC_M + nt) * few_groups(ci) * 16 + (FEW_Z + 2) * HPLANE * 2 * ci);
+__host__ __device__ constexpr uint32_t few_smem(int ci, int nt, int mb) {
+    return (uint32_t)((TC_M + nt) * few_groups(ci) * 16 + (mb + 2) * HPLANE * 2 * ci);
 }
 
 template <int CI>
 __global__ void __launch_bounds__(TC_M) k_conv_few(const bf16* __restrict__ x, int N, int D, int H, int W,
                                                    const bf16* __restrict__ wgt, const float* __restrict__ bias, int Cout,
-                                                   int nt, int relu, int wrap, bool vy, bool vy32, bf16* __restrict__ y,
-                                                   float* __restrict__ y32) {
+                                                   int nt, int mb, int relu, int wrap, bool vy, bool vy32,
+                                                   bf16* __restrict__ y, float* __restrict__ y32) {
     static_assert(CI == 2 || CI == 4, "a cell of 4 or 8 bytes");
     using Cell = typename std::conditional<CI == 2, uint32_t, uint2>::type;
     constexpr int KG = few_groups(CI), K = 27 * CI;
@@ -790,14 +791,14 @@ __global__ void __launch_bounds__(TC_M) k_conv_few(const bf16* __restrict__ x, i
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = tmem_slot, idesc = tc::idesc_bf16_f32(TC_M, nt);
-    const int BX = (W + 7) / 8, BY = (H + 15) / 16, BZ = (D + FEW_Z - 1) / FEW_Z;
+    const int BX = (W + 7) / 8, BY = (H + 15) / 16, BZ = (D + mb - 1) / mb;
     const long long tiles = (long long)N * BZ * BY * BX;
     const int lx = tid & 7, ly = tid >> 3;
     bool ok = true;
     uint32_t ph = 0;
     for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        const Brick b = brick_at(t, BX, BY, BZ, FEW_Z);
-        const int nz = D - b.z0 < FEW_Z ? D - b.z0 : FEW_Z;
+        const Brick b = brick_at(t, BX, BY, BZ, mb);
+        const int nz = D - b.z0 < mb ? D - b.z0 : mb;
 #pragma unroll 4
         for (int e = tid; e < (nz + 2) * HPLANE; e += TC_M) {
             const int hx = e % HX, hy = e / HX % HY, hz = e / HPLANE;
@@ -1318,8 +1319,12 @@ template <int CI>
 static int conv3d_few(const void* x, int n, int d, int h, int w, const void* wgt, const float* bias, int cout, int relu,
                       int wrap, void* y, float* y32, bool vy, bool vy32, cudaStream_t s) {
     const int want = (cout + 15) / 16 * 16, nt = want < 64 ? want : 64, gy = (cout + nt - 1) / nt;
-    const long long tiles = (long long)n * ((d + FEW_Z - 1) / FEW_Z) * ((h + 15) / 16) * ((w + 7) / 8);
-    const uint32_t smem = few_smem(CI, nt);
+    // shallower bricks while they are fewer than the SMs: a block works through its planes in turn
+    const long long columns = (long long)n * ((h + 15) / 16) * ((w + 7) / 8);
+    int mb = FEW_Z;
+    while (mb > 1 && columns * ((d + mb - 1) / mb) * gy < sm_count()) mb /= 2;
+    const long long tiles = columns * ((d + mb - 1) / mb);
+    const uint32_t smem = few_smem(CI, nt, mb);
     uint32_t cols = 32;
     while (cols < (uint32_t)nt) cols <<= 1;
     long long per_sm = (224 << 10) / (smem + 2048);  // by shared memory, TMEM columns and threads
@@ -1330,7 +1335,7 @@ static int conv3d_few(const void* x, int n, int d, int h, int w, const void* wgt
     int rc = tc_launch_ok((const void*)k_conv_few<CI>, smem, "cudaFuncSetAttribute(k_conv_few)");
     if (rc) return rc;
     k_conv_few<CI><<<dim3((unsigned)gx, (unsigned)gy), TC_M, smem, s>>>(
-        static_cast<const bf16*>(x), n, d, h, w, static_cast<const bf16*>(wgt), bias, cout, nt, relu, wrap, vy, vy32,
+        static_cast<const bf16*>(x), n, d, h, w, static_cast<const bf16*>(wgt), bias, cout, nt, mb, relu, wrap, vy, vy32,
         static_cast<bf16*>(y), y32);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_conv_few launch");

@@ -668,3 +668,13 @@ def test_conv_weights_gathered_or_packed(nn, case):
     finally:
         nn.lbm_nn_conv_tune(0, 0)
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("case", [
+    # two and four input channels: columns of one, two, four and eight planes, with a ragged last one, and more
+    # columns than blocks run at once
+    (1, 24, 24, 24, 2, 16, 1, 5), (1, 23, 40, 44, 4, 20, 0, 0), (2, 21, 40, 40, 2, 4, 0, 2), (4, 19, 40, 40, 4, 36, 1, 7),
+    (2, 41, 128, 128, 2, 16, 0, 0),
+])
+def test_conv_few_channels_column_depths(nn, case):
+    _check_conv(nn, case)
