@@ -1,6 +1,6 @@
 // nn.cu -- the learned warm start (not in the paper): the entry points of the
 // 3x3x3 convolutions, whose tcgen05 kernels are in nn_tc.cu, their mma.sync form
-// for odd numbers of input channels, the bias gradient and the elementwise steps
+// for few channels and thin boxes, the bias gradient and the elementwise steps
 // of training.  See include/lbm_nn.h.
 #include <cuda_bf16.h>
 
@@ -41,11 +41,9 @@ __device__ __forceinline__ int nb_coord(int c, int d, int n, bool wrap) {
 // C[p][co] = sum_k A[p][k] B[k][co], A[p][(tap,ci)] = x[p + off(tap)][ci] (0 outside,
 // or wrapped on the axes set in `wrap`), B[(tap,ci)][co] = wgt[tap][ci][co]; one
 // block computes 64 voxels x NF*8 outputs starting at channel blockIdx.y * NF*8.
-// For an odd number of input channels, whose values lie at odd addresses: gathered
-// one by one either way, the warp-level MMAs cost less here than the tcgen05
-// pipeline's start per block (1 -> 16 channels on 4 x 32^3 voxels 21 and 47 us,
-// 7 -> 9 84 and 171).
-template <int NF>
+// VEC: Cin % 16 == 0, so that a thread's 16 consecutive k share one tap and are
+// read as two 16-byte vectors.  For the shapes of by_warps().
+template <int NF, bool VEC>
 __global__ void __launch_bounds__(128) k_conv(const bf16* __restrict__ x, int N, int D, int H, int W, int Cin,
                                               const bf16* __restrict__ wgt, const float* __restrict__ bias,
                                               int Cout, int relu, int wrap, bf16* __restrict__ y,
@@ -81,19 +79,35 @@ __global__ void __launch_bounds__(128) k_conv(const bf16* __restrict__ x, int N,
     for (int k0 = 0; k0 < K; k0 += BK) {
         int k = k0 + ak;
         int tap = k / Cin, ci = k - tap * Cin;
-#pragma unroll
-        for (int j = 0; j < 16; j++) {
-            bf16 v = zero;
+        if constexpr (VEC) {
+            uint4 v0 = make_uint4(0, 0, 0, 0), v1 = v0;
             if (arow && k < K) {
                 const int zz = nb_coord(az, tap / 9 - 1, D, wz), yy = nb_coord(ay, (tap / 3) % 3 - 1, H, wy),
                           xx = nb_coord(ax, tap % 3 - 1, W, wx);
-                if ((zz | yy | xx) >= 0) v = x[((((long long)an * D + zz) * H + yy) * W + xx) * Cin + ci];
+                if ((zz | yy | xx) >= 0) {
+                    const uint4* src =
+                        reinterpret_cast<const uint4*>(x + ((((long long)an * D + zz) * H + yy) * W + xx) * Cin + ci);
+                    v0 = src[0];
+                    v1 = src[1];
+                }
             }
-            As[ar][ak + j] = v;
-            k++;
-            if (++ci == Cin) {
-                ci = 0;
-                tap++;
+            *reinterpret_cast<uint4*>(&As[ar][ak]) = v0;
+            *reinterpret_cast<uint4*>(&As[ar][ak + 8]) = v1;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 16; j++) {
+                bf16 v = zero;
+                if (arow && k < K) {
+                    const int zz = nb_coord(az, tap / 9 - 1, D, wz), yy = nb_coord(ay, (tap / 3) % 3 - 1, H, wy),
+                              xx = nb_coord(ax, tap % 3 - 1, W, wx);
+                    if ((zz | yy | xx) >= 0) v = x[((((long long)an * D + zz) * H + yy) * W + xx) * Cin + ci];
+                }
+                As[ar][ak + j] = v;
+                k++;
+                if (++ci == Cin) {
+                    ci = 0;
+                    tap++;
+                }
             }
         }
         for (int e = tid; e < BN * BK; e += 128) {
@@ -442,11 +456,37 @@ int wgrad_tc(const void* x, const void* dy, int n, int d, int h, int w, int cin,
 }  // namespace nn
 }  // namespace lbm
 
+// The convolutions that k_conv does faster than the tcgen05 kernels (on both, us):
+// - an odd number of input channels, whose values lie at odd addresses: gathered one
+//   by one either way, the warp-level MMAs cost less than the tcgen05 pipeline's
+//   start per block (1 -> 16 channels on 4 x 32^3 voxels 21 and 47, 7 -> 9 84 and
+//   171); and an even one that allows no 8-channel loads, where both are few (6 -> 4
+//   on 16^3 23 and 27, 10 -> 32 36 and 41, 20 -> 4 61 and 66; but 26 -> 16 89 and 80,
+//   10 -> 64 52 and 46);
+// - boxes so thin along x or y that most of the 8 x 16 columns of the halo kernels is
+//   padding, once that is what they spend their time on (2 -> 16 on 512 x 1 x 512 49
+//   and 76, on 512 x 512 x 1, half as empty, 56 and 50; 16 -> 16 on 256 x 1 x 256 23
+//   and 77, 64 -> 64 154 and 256), and boxes of one plane of 16 channels, each plane
+//   with its two neighbours in z (16 -> 4 on 1 x 256 x 256 19 and 25).
+static bool by_warps(const void* x, int n, int d, int h, int w, int cin, int cout) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(x);
+    if (cin % 2) return true;
+    const double voxels = (double)n * d * h * w;
+    const double column = (double)n * ((h + 15) / 16) * ((w + 7) / 8) * 128;  // positions of one plane
+    if ((cin == 2 || cin == 4) && at % (2 * cin) == 0) return column * d > 8 * voxels && column * d >= 1 << 18;
+    if (cin % 8) return cin < 24 && cout <= 32;
+    if (cin % 16 || at % 16) return false;
+    const double read = column * (d + 2 * ((d + 15) / 16));  // positions that the halo planes hold
+    if (cin == 16 && cout <= 16) return read > 2.75 * voxels && read >= 1 << 17;
+    return read > (cin == 16 ? 9 : 16) * voxels && read >= 400e3;
+}
+
 extern "C" int lbm_nn_conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt,
                              const float* bias, int cout, int relu, int wrap, void* y, float* y32, void* stream) {
     if (!x || !wgt || n < 1 || d < 1 || h < 1 || w < 1 || cin < 1 || cout < 1 || (!y && !y32) || (wrap & ~7))
         return fail(LBM_ERR_ARG, "lbm_nn_conv3d: bad arguments");
-    if (cin % 2 == 0) return conv3d(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, S(stream));
+    if (!by_warps(x, n, d, h, w, cin, cout))
+        return conv3d(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, S(stream));
     const long long M = (long long)n * d * h * w;
     int ny = 0;
     const int nf = pick_nf(cout, &ny);
@@ -455,14 +495,15 @@ extern "C" int lbm_nn_conv3d(const void* x, int n, int d, int h, int w, int cin,
         kern<<<grid, 128, 0, S(stream)>>>(static_cast<const bf16*>(x), n, d, h, w, cin, static_cast<const bf16*>(wgt),
                                           bias, cout, relu, wrap, static_cast<bf16*>(y), y32);
     };
+    const bool vec = cin % 16 == 0;
     switch (nf) {
-        case 1: go(k_conv<1>); break;
-        case 2: go(k_conv<2>); break;
-        case 4: go(k_conv<4>); break;
-        case 6: go(k_conv<6>); break;
-        case 8: go(k_conv<8>); break;
-        case 12: go(k_conv<12>); break;
-        default: go(k_conv<16>); break;
+        case 1: vec ? go(k_conv<1, true>) : go(k_conv<1, false>); break;
+        case 2: vec ? go(k_conv<2, true>) : go(k_conv<2, false>); break;
+        case 4: vec ? go(k_conv<4, true>) : go(k_conv<4, false>); break;
+        case 6: vec ? go(k_conv<6, true>) : go(k_conv<6, false>); break;
+        case 8: vec ? go(k_conv<8, true>) : go(k_conv<8, false>); break;
+        case 12: vec ? go(k_conv<12, true>) : go(k_conv<12, false>); break;
+        default: vec ? go(k_conv<16, true>) : go(k_conv<16, false>); break;
     }
     return check(cudaGetLastError(), "k_conv launch");
 }

@@ -678,3 +678,16 @@ def test_conv_weights_gathered_or_packed(nn, case):
 ])
 def test_conv_few_channels_column_depths(nn, case):
     _check_conv(nn, case)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("case", [
+    # thin boxes on either side of the lines between the two tensor-core paths (one voxel along x, y or z), for few
+    # channels, 16 and more; even channel counts that allow no 16-byte loads
+    (1, 256, 1, 512, 2, 16, 0, 1), (1, 512, 128, 1, 4, 20, 1, 2), (1, 1, 256, 256, 16, 4, 0, 0),
+    (1, 128, 2, 128, 16, 16, 1, 7), (1, 256, 1, 256, 16, 40, 0, 4), (1, 4096, 1, 1, 32, 24, 0, 0),
+    (1, 2, 128, 130, 16, 4, 0, 3), (1, 7, 8, 300, 16, 12, 1, 0),
+    (2, 9, 7, 11, 6, 4, 1, 0), (1, 8, 9, 10, 20, 32, 0, 5), (1, 8, 9, 10, 22, 33, 0, 2), (1, 5, 6, 7, 26, 16, 1, 0),
+])
+def test_conv_routes(nn, case, offset):
+    _check_conv(nn, case, offset)
