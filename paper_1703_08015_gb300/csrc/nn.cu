@@ -234,9 +234,11 @@ __device__ __forceinline__ void store_pack(bf16* p, const Pack<V>& x) {
     *reinterpret_cast<Pack<V>*>(p) = x;
 }
 
+// (n packs and, behind them, `rest` < V values, the first threads' own)
 template <int V, class I>
-__global__ void k_relu_mask(bf16* __restrict__ g, const bf16* __restrict__ act, I n) {
-    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < n; e += (I)gridDim.x * blockDim.x) {
+__global__ void k_relu_mask(bf16* __restrict__ g, const bf16* __restrict__ act, I n, int rest) {
+    const I t = blockIdx.x * (I)blockDim.x + threadIdx.x;
+    for (I e = t; e < n; e += (I)gridDim.x * blockDim.x) {
         const Pack<V> a = load_pack<V>(act + (size_t)e * V);
         Pack<V> x = load_pack<V>(g + (size_t)e * V);
 #pragma unroll
@@ -244,6 +246,8 @@ __global__ void k_relu_mask(bf16* __restrict__ g, const bf16* __restrict__ act, 
             if (!(__bfloat162float(a.v[k]) > 0.f)) x.v[k] = __float2bfloat16(0.f);
         store_pack(g + (size_t)e * V, x);
     }
+    const size_t at = (size_t)n * V + t;
+    if (t < (I)rest && !(__bfloat162float(act[at]) > 0.f)) g[at] = __float2bfloat16(0.f);
 }
 
 // The group of channels e of a tensor [.][D][H][W][G groups]: its sample, voxel
@@ -366,14 +370,17 @@ __global__ void k_adam(float* __restrict__ p, float* __restrict__ g, float* __re
 }
 
 template <int V, class I>
-__global__ void k_add(const bf16* a, const bf16* b, I n, bf16* y) {  // y may be a or b
-    for (I e = blockIdx.x * (I)blockDim.x + threadIdx.x; e < n; e += (I)gridDim.x * blockDim.x) {
+__global__ void k_add(const bf16* a, const bf16* b, I n, int rest, bf16* y) {  // y may be a or b; as k_relu_mask
+    const I t = blockIdx.x * (I)blockDim.x + threadIdx.x;
+    for (I e = t; e < n; e += (I)gridDim.x * blockDim.x) {
         const Pack<V> p = load_pack<V>(a + (size_t)e * V), q = load_pack<V>(b + (size_t)e * V);
         Pack<V> o;
 #pragma unroll
         for (int k = 0; k < V; k++) o.v[k] = __float2bfloat16(__bfloat162float(p.v[k]) + __bfloat162float(q.v[k]));
         store_pack(y + (size_t)e * V, o);
     }
+    const size_t at = (size_t)n * V + t;
+    if (t < (I)rest) y[at] = __float2bfloat16(__bfloat162float(a[at]) + __bfloat162float(b[at]));
 }
 
 __global__ void k_mask_input(const uint8_t* __restrict__ mask, size_t vox, float value, bf16* __restrict__ x) {
@@ -537,7 +544,7 @@ extern "C" int lbm_nn_conv3d_wgrad(const void* x, const void* dy, int n, int d, 
     return rc ? rc : sum_few(part, nb, cout, dbias, S(stream));
 }
 
-// Runs go(V, I) with the widest pack that the channel counts (or total) `c` and
+// Runs go(V, I) with the widest pack that the channel counts `c` (0: any) and
 // the addresses `at` (ORed) allow, and indices wide enough for `total` values
 // plus a grid's stride.
 template <class F>
@@ -554,10 +561,10 @@ static uintptr_t adr(const void* p) { return reinterpret_cast<uintptr_t>(p); }
 
 extern "C" int lbm_nn_relu_mask(void* g, const void* act, size_t count, void* stream) {
     if (!g || !act) return fail(LBM_ERR_ARG, "lbm_nn_relu_mask: NULL");
-    by_width(count, adr(g) | adr(act), count, [&](auto V, auto I) {
+    by_width(0, adr(g) | adr(act), count, [&](auto V, auto I) {
         constexpr int v = decltype(V)::value;
         k_relu_mask<v, decltype(I)><<<grid_for(count / v), 256, 0, S(stream)>>>(
-            static_cast<bf16*>(g), static_cast<const bf16*>(act), (decltype(I))(count / v));
+            static_cast<bf16*>(g), static_cast<const bf16*>(act), (decltype(I))(count / v), (int)(count % v));
     });
     return check(cudaGetLastError(), "k_relu_mask launch");
 }
@@ -658,10 +665,11 @@ extern "C" int lbm_nn_adam(float* p, float* g, float* m, float* v, void* pb, siz
 
 extern "C" int lbm_nn_add(const void* a, const void* b, size_t count, void* y, void* stream) {
     if (!a || !b || !y) return fail(LBM_ERR_ARG, "lbm_nn_add: NULL");
-    by_width(count, adr(a) | adr(b) | adr(y), count, [&](auto V, auto I) {
+    by_width(0, adr(a) | adr(b) | adr(y), count, [&](auto V, auto I) {
         constexpr int v = decltype(V)::value;
         k_add<v, decltype(I)><<<grid_for(count / v), 256, 0, S(stream)>>>(
-            static_cast<const bf16*>(a), static_cast<const bf16*>(b), (decltype(I))(count / v), static_cast<bf16*>(y));
+            static_cast<const bf16*>(a), static_cast<const bf16*>(b), (decltype(I))(count / v), (int)(count % v),
+            static_cast<bf16*>(y));
     });
     return check(cudaGetLastError(), "k_add launch");
 }

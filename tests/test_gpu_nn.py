@@ -691,3 +691,22 @@ def test_conv_few_channels_column_depths(nn, case):
 ])
 def test_conv_routes(nn, case, offset):
     _check_conv(nn, case, offset)
+
+
+@pytest.mark.parametrize("count", [1, 7, 8, 4099, 70_001])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_sum_and_relu_mask_of_any_count(nn, count, offset):
+    """Packs of eight values and what is left behind them; nothing beyond is written."""
+    rng = np.random.default_rng(43 + count)
+    a, b = (R.bf16_round(rng.normal(size=count)) for _ in range(2))
+
+    def dev(v):
+        t = torch.full((offset + count + 9,), 3.0, dtype=torch.bfloat16, device="cuda")
+        t[offset:offset + count] = bf16_dev(v)
+        return t[offset:]
+
+    x, y = dev(a), dev(b)
+    nn.lbm_nn_add(x, y, count, y)
+    assert np.array_equal(f64(y[:count]), R.bf16_round(a + b)) and torch.all(y[count:] == 3.0)
+    nn.lbm_nn_relu_mask(x, y, count)
+    assert np.array_equal(f64(x[:count]), np.where(R.bf16_round(a + b) > 0, a, 0.0)) and torch.all(x[count:] == 3.0)
