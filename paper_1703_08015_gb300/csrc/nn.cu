@@ -151,18 +151,23 @@ __global__ void __launch_bounds__(128) k_conv(const bf16* __restrict__ x, int N,
 // of dy over the block's rows, in row order (one FP32 chain per channel: the
 // order is part of the result's rounding).  The block's threads bring the rows
 // to shared memory, tile after tile, 16 bytes at a time where VEC (C % 8 == 0,
-// aligned), the next tile in flight while one thread per channel walks the
-// last.  Bound by that chain, 4096 additions, about 10 us for any layer; walking
-// memory instead of shared memory the 15 layers of a training step on 8 x 64^3
-// voxels took 5.4 ms with their chunk sums.
+// aligned), else 4 (up to 256 channels: a tile is one run of values then), the next
+// tile in flight while one thread per channel walks the last.  Bound by that chain,
+// 4096 additions, about 10 us for 16 channels, and by the copies of one block per 4096
+// rows with many (128 channels on 16^3 voxels 53 us; off by one value 74, value by
+// value 310); walking memory instead of shared memory the 15 layers of a training step
+// on 8 x 64^3 voxels took 5.4 ms with their chunk sums.
 constexpr int kBiasThreads = 256;
 constexpr int kBiasRows = 4096;
-constexpr int kBiasTile = 8192;  // values of a tile, at most (a row wider than that takes several passes)
+constexpr int kBiasTile = 8192;  // values of a tile, at most (a row holds the block's 256 channels at most)
+
+// 1 where a value is the upper half of its 4-byte word.
+__device__ __forceinline__ int odd_start(const bf16* p) { return (int)(reinterpret_cast<uintptr_t>(p) >> 1) & 1; }
 
 template <bool VEC>
 __global__ void __launch_bounds__(kBiasThreads) k_bias_grad(const bf16* __restrict__ dy, long long M, int C,
                                                             float* __restrict__ part) {
-    __shared__ __align__(16) bf16 sm[2][kBiasTile];
+    __shared__ __align__(16) bf16 sm[2][kBiasTile + 8];
     const long long r0 = (long long)blockIdx.x * kBiasRows;
     const int rows = (int)(M - r0 < kBiasRows ? M - r0 : kBiasRows);
     // the channels from blockIdx.y * kBiasThreads, one per thread
@@ -172,7 +177,15 @@ __global__ void __launch_bounds__(kBiasThreads) k_bias_grad(const bf16* __restri
     auto load = [&](int t) {
         bf16* dst = sm[t & 1];
         const int n = rows - t * tr < tr ? rows - t * tr : tr;
-        if constexpr (VEC) {
+        if (!VEC && cn == C) {
+            // the tile is one run of values: whole words, and the values at its ends that share theirs
+            const bf16* from = src + (long long)t * tr * C;
+            const int odd = odd_start(from), total = n * C;
+            dst += odd;
+            for (int e = odd + 2 * threadIdx.x; e + 2 <= total; e += 2 * kBiasThreads) tc::cp_async4(dst + e, from + e);
+            if (threadIdx.x == 0 && odd) dst[0] = from[0];
+            if (threadIdx.x == 0 && (total - odd) % 2) dst[total - 1] = from[total - 1];
+        } else if constexpr (VEC) {
             const int g8 = cn / 8;
             for (int e = threadIdx.x; e < n * g8; e += kBiasThreads) {
                 const int r = e / g8, g = e - r * g8;
@@ -195,7 +208,7 @@ __global__ void __launch_bounds__(kBiasThreads) k_bias_grad(const bf16* __restri
         __syncthreads();
         const int n = rows - t * tr < tr ? rows - t * tr : tr;
         if ((int)threadIdx.x < cn) {
-            const bf16* p = sm[t & 1] + threadIdx.x;
+            const bf16* p = sm[t & 1] + threadIdx.x + (!VEC && cn == C ? odd_start(src + (long long)t * tr * C) : 0);
 #pragma unroll 16
             for (int r = 0; r < n; r++) s += __bfloat162float(p[r * cn]);
         }

@@ -150,6 +150,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int k = 0; k < 16; k++) v[k] = __uint_as_float(r[k]);
 }
 
+// The same for 4 bytes (both addresses 4-byte aligned), always read.
+__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+}
+
 // 16-byte global -> shared copy completing asynchronously (cp.async, cached
 // in L2 only: the blocks' shared memory leaves little L1); `full` false writes
 // 16 zero bytes without reading the source.

@@ -710,3 +710,26 @@ def test_sum_and_relu_mask_of_any_count(nn, count, offset):
     assert np.array_equal(f64(y[:count]), R.bf16_round(a + b)) and torch.all(y[count:] == 3.0)
     nn.lbm_nn_relu_mask(x, y, count)
     assert np.array_equal(f64(x[:count]), np.where(R.bf16_round(a + b) > 0, a, 0.0)) and torch.all(x[count:] == 3.0)
+
+
+@pytest.mark.parametrize("c", [1, 7, 16, 100, 128, 256, 300])
+def test_bias_gradient_of_unaligned_tensors(nn, c):
+    """Bias gradients from a dy on a 16-byte boundary, off by one and by two values: the same sums, bit for bit (one
+    chain per channel whatever the loads), within an FP32 chain's error of the FP64 ones."""
+    rng = np.random.default_rng(53 + c)
+    n, d, h, w = 1, 11, 20, 25  # 5500 rows: a whole block of 4096 and part of one
+    dy = rand_bf16(rng, (n, d, h, w, c))
+    x = torch.zeros(n * d * h * w, dtype=torch.bfloat16, device="cuda")
+    out = []
+    for offset in (0, 1, 2):
+        t = torch.empty(dy.size + offset, dtype=torch.bfloat16, device="cuda")[offset:]
+        t[:] = bf16_dev(dy).reshape(-1)
+        dw = torch.zeros(27 * c, dtype=torch.float32, device="cuda")
+        db = torch.full((c,), 0.5, dtype=torch.float32, device="cuda")
+        nn.lbm_nn_conv3d_wgrad(x, t, n, d, h, w, 1, c, 0, dw, db)
+        torch.cuda.synchronize()
+        out.append(db)
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+    # each of 4096 additions rounds by at most 2^-24 of the partial sum, itself at most sum |dy|
+    tol = 4096 * 2.0 ** -24 * np.abs(dy).reshape(-1, c).sum(axis=0)
+    assert np.all(np.abs(f64(out[0]) - 0.5 - dy.reshape(-1, c).sum(axis=0)) <= tol)
