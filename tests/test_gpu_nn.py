@@ -733,3 +733,32 @@ def test_bias_gradient_of_unaligned_tensors(nn, c):
     # each of 4096 additions rounds by at most 2^-24 of the partial sum, itself at most sum |dy|
     tol = 4096 * 2.0 ** -24 * np.abs(dy).reshape(-1, c).sum(axis=0)
     assert np.all(np.abs(f64(out[0]) - 0.5 - dy.reshape(-1, c).sum(axis=0)) <= tol)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("case", [
+    # n, d, h, w, cin, cout, wrap: several groups of input channels, dy of channel counts that are no multiple of
+    # eight; segments enough to use every stage of rings of four
+    # and of two again and again
+    (1, 6, 9, 10, 64, 64, 1), (2, 5, 8, 7, 100, 100, 0), (1, 4, 6, 9, 72, 51, 6), (1, 3, 5, 6, 40, 3, 0),
+    (2, 24, 33, 31, 2, 16, 0), (1, 20, 40, 40, 16, 16, 5), (1, 9, 90, 100, 96, 48, 0), (1, 3, 7, 2100, 64, 48, 1),
+])
+def test_conv_weight_gradient_rings(nn, case, offset):
+    n, d, h, w, cin, cout, wrap = case
+    rng = np.random.default_rng(47 + hash(case) % 2**31)
+    x = rand_bf16(rng, (n, d, h, w, cin))
+    dy = rand_bf16(rng, (n, d, h, w, cout))
+
+    def dev(a):
+        t = torch.empty(a.size + offset, dtype=torch.bfloat16, device="cuda")
+        t[offset:] = bf16_dev(a).reshape(-1)
+        return t[offset:]
+
+    dw = torch.full((27 * cin * cout,), 0.25, dtype=torch.float32, device="cuda")
+    nn.lbm_nn_conv3d_wgrad(dev(x), dev(dy), n, d, h, w, cin, cout, wrap, dw, None)
+    torch.cuda.synchronize()
+    assert nn.lbm_nn_tc_timeouts() == 0
+    ref = R.conv3d_bwd_weight(x, dy, wrap)[0]
+    tol = 2.0 ** -16 * R.conv3d_bwd_weight(np.abs(x), np.abs(dy), wrap)[0] + 1e-6
+    err = np.abs(f64(dw).reshape(27, cin, cout) - 0.25 - ref)
+    assert np.all(err <= tol), float(np.max(err / tol))
