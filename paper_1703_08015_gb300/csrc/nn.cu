@@ -498,7 +498,7 @@ static bool by_warps(const void* x, int n, int d, int h, int w, int cin, int cou
     if (cin % 16 || at % 16) return false;
     const double read = column * (d + 2 * ((d + 15) / 16));  // positions that the halo planes hold
     if (cin == 16 && cout <= 16) return read > 2.75 * voxels && read >= 1 << 17;
-    return read > (cin == 16 ? 9 : 16) * voxels && read >= 400e3;
+    return read > (cin == 16 ? 8.5 : 16) * voxels && read >= 400e3;
 }
 
 extern "C" int lbm_nn_conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt,
