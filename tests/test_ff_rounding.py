@@ -132,3 +132,35 @@ def test_lazy_sum_feeding_a_product_keeps_the_error_of_the_operands():
         scale = max(abs(float(a[0])), abs(float(b[0]))) * abs(float(c[0]))
         worst = max(worst, abs(float(got - exact)) / scale)
     assert worst < 3 * 2.0 ** -47, worst
+
+
+# ---- the wider rounding, for results that the one above does not take ----------------------------------------------
+# Each part is rounded to an integer by itself (round to nearest even): |x.h| < 2^47 as a 64-bit and |x.l| < 2^30 as a
+# 32-bit integer, their sum added to the bits of w, which every lattice weight allows within 2^48 ulps.
+
+
+def _round_wide(xh, xl):
+    return int(np.rint(np.float64(np.float32(xh)))) + int(np.rint(np.float64(np.float32(xl))))
+
+
+def test_wide_rounding_within_one_unit_and_in_the_binade():
+    rng = np.random.default_rng(11)
+    n = 4000
+    xh = np.float32(rng.choice([-1, 1], n) * 2.0 ** rng.uniform(-30, 47, n))
+    xl = np.float32(rng.choice([-1, 1], n) * 2.0 ** rng.uniform(-30, 30, n))
+    big, low = np.nextafter(np.float32(2.0 ** 47), np.float32(0)), np.nextafter(np.float32(2.0 ** 30), np.float32(0))
+    pairs = list(zip(xh, xl)) + [(h, l) for h in (big, -big, np.float32(2.0 ** 46), np.float32(0.5), np.float32(-1.5))
+                                 for l in (low, -low, np.float32(0.5), np.float32(-2.5), np.float32(0.0))]
+    for h, l in pairs:
+        if not (abs(h) < 2.0 ** 47 and abs(l) < 2.0 ** 30):
+            continue
+        r = _round_wide(h, l)
+        assert abs(r - _exact(h, l)) <= 1, (float(h), float(l))
+        assert abs(r) < 2 ** 47 + 2 ** 31
+
+
+def test_wide_and_narrow_rounding_agree_within_two_units():
+    rng = np.random.default_rng(13)
+    xh, xl = _random_pairs(rng, 2000, 1.5 * 2.0 ** 24)
+    for h, l in zip(xh, xl):
+        assert abs(_round_wide(h, l) - _round_units(h, l)) <= 2, (float(h), float(l))
