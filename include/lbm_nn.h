@@ -6,8 +6,8 @@
  * steady state in fewer steps; the LBM residual alone still decides
  * convergence.  These entry points are the network's GPU kernels: 3x3x3
  * convolutions on tensor cores (BF16 operands, FP32 accumulation; tcgen05, or
- * mma.sync for odd numbers of input channels) for the forward pass and both
- * backward passes, plus the pooling, upsampling, concatenation, loss and
+ * mma.sync for odd and some small numbers of input channels and for thin boxes)
+ * for the forward pass and both backward passes, plus the pooling, upsampling, concatenation, loss and
  * optimiser steps of training.
  *
  * Conventions
@@ -35,18 +35,18 @@ extern "C" {
  * which are periodic.  Output BF16 (y) and/or FP32 (y32); either may be NULL.
  * Any cout (output channels are tiled over the grid).  The backward-data pass
  * is this same call on dy with the weights from lbm_nn_weight_flip and the
- * same `wrap`.  For cin % 16 == 0 the weights are repacked into device memory
- * that the call takes and gives back in the order of its stream, so calls may
- * overlap on different streams, host threads and devices, and may be captured
- * into a graph (whose memory nodes then hold them). */
+ * same `wrap`.  For cin % 16 == 0 many weights (more than 64 KB) are repacked into
+ * device memory that the call takes and gives back in the order of its stream, so
+ * calls may overlap on different streams, host threads and devices, and may be
+ * captured into a graph (whose memory nodes then hold them). */
 int lbm_nn_conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt,
                   const float* bias, int cout, int relu, int wrap, void* y, float* y32, void* stream);
 
 /* lbm_nn_conv3d on the 5th-generation tensor cores (tcgen05), FP32
  * accumulator in tensor memory: for cin % 16 == 0 the tensor cores read the
  * activations straight from halo planes in shared memory, otherwise an implicit
- * GEMM gathers them.  The kernels of lbm_nn_conv3d, which takes every shape and
- * alignment; this entry needs cin % 8 == 0, cout % 16 == 0 and 16-byte aligned
+ * GEMM gathers them.  Kernels of lbm_nn_conv3d, which takes every shape and
+ * alignment and thin boxes by mma.sync; this entry needs cin % 8 == 0, cout % 16 == 0 and 16-byte aligned
  * x, wgt, y, y32 (else LBM_ERR_ARG). */
 int lbm_nn_conv3d_tc(const void* x, int n, int d, int h, int w, int cin, const void* wgt,
                      const float* bias, int cout, int relu, int wrap, void* y, float* y32, void* stream);
@@ -83,6 +83,8 @@ int lbm_nn_weight_flip(const void* wgt, int cin, int cout, void* wt, void* strea
  * channels-last tiles in shared memory (zero-padded to 8 input and 16 output
  * channels); the partial sums live in a library-owned device buffer (grown on
  * demand, kept for the process; calls must not overlap on different streams).
+ * The sums run over the zero padding as well: a value of x that is not finite at
+ * the box's edge makes every tap of its channel NaN.
  * Errors: LBM_ERR_ARG, LBM_ERR_OOM (no room for the partial sums),
  * LBM_ERR_CUDA. */
 int lbm_nn_conv3d_wgrad(const void* x, const void* dy, int n, int d, int h, int w, int cin, int cout,
