@@ -188,8 +188,8 @@ __device__ __forceinline__ int tc_nb(int c, int d, int n, bool wrap) {
 // A[p][(tap, ci)] = x[p + off(tap)][ci] (zero outside, or wrapped on the axes
 // of `wrap`) and B[co][(tap, ci)] = wgt[tap][ci][co].  One block computes 128
 // voxels x NT output channels from blockIdx.y * NT, NT % 16 == 0.  A is read G
-// channels at a time: 8 (Cin % 8 == 0, 16-byte aligned), 2 (even Cin, 4-byte
-// aligned) or 1.  Rows k >= 27 Cin of the last stage are zero; `n_stages` stages
+// channels at a time: 8 (Cin % 8 == 0, 16-byte aligned) or 2 (even Cin, 4-byte
+// aligned).  Rows k >= 27 Cin of the last stage are zero; `n_stages` stages
 // are reserved.
 //
 // Bound by the addresses and the latency of the gathers.
@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ x, int
                                                  const bf16* __restrict__ wgt, const float* __restrict__ bias,
                                                  int Cout, int NT, int relu, int wrap, bool vy, bool vy32,
                                                  bf16* __restrict__ y, float* __restrict__ y32) {
+    static_assert(G == 8 || G == 2, "16- or 4-byte loads");
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t mbar[TC_STAGES];
     __shared__ uint32_t tmem_slot;
@@ -255,15 +256,8 @@ __global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ x, int
                 uint32_t h[4];
 #pragma unroll
                 for (int q = 0; q < 4; q++) {
-                    if constexpr (G == 2) {
-                        const bf16* src = tap[q] >= 0 ? source(c, tap[q], ci[q]) : nullptr;
-                        h[q] = src ? __ldg(reinterpret_cast<const uint32_t*>(src)) : 0u;
-                    } else {
-                        const bf16* lo = tap[2 * q] >= 0 ? source(c, tap[2 * q], ci[2 * q]) : nullptr;
-                        const bf16* hi = tap[2 * q + 1] >= 0 ? source(c, tap[2 * q + 1], ci[2 * q + 1]) : nullptr;
-                        h[q] = (lo ? __ldg(reinterpret_cast<const unsigned short*>(lo)) : 0u) |
-                               (hi ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(hi)) << 16 : 0u);
-                    }
+                    const bf16* src = tap[q] >= 0 ? source(c, tap[q], ci[q]) : nullptr;
+                    h[q] = src ? __ldg(reinterpret_cast<const uint32_t*>(src)) : 0u;
                 }
                 *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
             }
@@ -406,13 +400,13 @@ __device__ __forceinline__ void fill_halo(unsigned char* dst, const HaloAxes& ax
 // and the tensor cores read an input plane 9 times instead of 27.  An output's
 // sum runs in the order (chunk, dz, dy, dx, 16 channels).
 //
-// What bounds it: the MMAs' reads of their 128 A rows from shared memory, up to
-// nt = 32 (an MMA of 128 x N x 16 takes max(N / 2, 32 + N / 4) cycles), beyond
-// that the MMAs.  Before and after (blocks of up to four planes that copied,
-// multiplied and stored in turn, 27 MMAs per plane): 48 -> 16 channels on 8 x
-// 64^3 voxels 639 and 216 us, 96 -> 32 on 8 x 32^3 292 and 87, 192 -> 64 on 8 x
-// 16^3 149 and 50, 192 -> 128 on 8 x 48^3 6411 and 1304; 16 -> 16 on 8 x 64^3,
-// bound by its outputs, 136 and 134.
+// What bounds it: the copies of the halo planes (about 16 bytes per cycle and SM) and,
+// beside them, the MMAs with their reads of 128 A rows from shared memory (an MMA of
+// 128 x N x 16 takes max(N / 2, 32 + N / 4) cycles); no unit is saturated.  Before and
+// after (blocks of up to four planes that copied, multiplied and stored in turn, 27
+// MMAs per plane): 48 -> 16 channels on 8 x 64^3 voxels 639 and 218 us, 96 -> 32 on 8
+// x 32^3 292 and 88, 192 -> 64 on 8 x 16^3 149 and 51, 192 -> 128 on 8 x 48^3 6411 and
+// 1300; 16 -> 16 on 8 x 64^3, bound by its outputs, 136 and 129.
 //
 // Blocks are persistent: each keeps one tile of output channels and walks over
 // bricks.  One warp issues the MMAs, eight copy the planes (the stages that
@@ -1341,7 +1335,7 @@ static int conv3d_few(const void* x, int n, int d, int h, int w, const void* wgt
     return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_conv_few launch");
 }
 
-// The convolution as an implicit GEMM, any channel counts and alignment.
+// The convolution as an implicit GEMM, an even number of input channels, x 4-byte aligned.
 static int conv3d_im2col(const void* x, int n, int d, int h, int w, int cin, const void* wgt, const float* bias, int cout,
                          int relu, int wrap, void* y, float* y32, bool vy, bool vy32, cudaStream_t s) {
     const int tiles = (cout + 127) / 128;
@@ -1361,7 +1355,7 @@ static int conv3d_im2col(const void* x, int n, int d, int h, int w, int cin, con
         return e == cudaSuccess ? LBM_OK : cuda_fail(e, "k_conv_tc launch");
     };
     if (cin % 8 == 0 && (uintptr_t)x % 16 == 0) return go(k_conv_tc<8>);
-    return cin % 2 == 0 && (uintptr_t)x % 4 == 0 ? go(k_conv_tc<2>) : go(k_conv_tc<1>);
+    return go(k_conv_tc<2>);
 }
 
 // Launch shape: the output-channel tile nt and brick depth mb of the least
@@ -1403,9 +1397,9 @@ static CvShape cv_pick(int n, int d, int h, int w, int cin, int cout, int* grid_
 constexpr size_t kGatherUnits = 4096;
 
 // The convolution: halo planes for cin % 16 == 0, rows put together from a halo
-// for two or four input channels, else the gathering implicit GEMM.  Any
-// channel counts and alignment (16-byte copies and stores where a tensor's
-// channels and address allow, else narrower ones).
+// for two or four input channels, else the gathering implicit GEMM (an even number
+// of input channels, x 4-byte aligned).  16-byte copies and stores where a tensor's
+// channels and address allow, else narrower ones.
 int conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt, const float* bias, int cout, int relu,
            int wrap, void* y, float* y32, cudaStream_t s) {
     const bool vy = cout % 8 == 0 && (uintptr_t)y % 16 == 0, vy32 = cout % 4 == 0 && (uintptr_t)y32 % 16 == 0;
@@ -1413,6 +1407,8 @@ int conv3d(const void* x, int n, int d, int h, int w, int cin, const void* wgt, 
         return conv3d_few<2>(x, n, d, h, w, wgt, bias, cout, relu, wrap, y, y32, vy, vy32, s);
     if (cin == 4 && (uintptr_t)x % 8 == 0)
         return conv3d_few<4>(x, n, d, h, w, wgt, bias, cout, relu, wrap, y, y32, vy, vy32, s);
+    if (cin % 16 && (cin % 2 || (uintptr_t)x % 4))
+        return fail(LBM_ERR_ARG, "convolution: %d input channels at an odd address on the tcgen05 kernels", cin);
     if (cin % 16) return conv3d_im2col(x, n, d, h, w, cin, wgt, bias, cout, relu, wrap, y, y32, vy, vy32, s);
     int gx = 1;
     const CvShape sh = cv_pick(n, d, h, w, cin, cout, &gx);

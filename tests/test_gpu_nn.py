@@ -762,3 +762,12 @@ def test_conv_weight_gradient_rings(nn, case, offset):
     tol = 2.0 ** -16 * R.conv3d_bwd_weight(np.abs(x), np.abs(dy), wrap)[0] + 1e-6
     err = np.abs(f64(dw).reshape(27, cin, cout) - 0.25 - ref)
     assert np.all(err <= tol), float(np.max(err / tol))
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2])
+@pytest.mark.parametrize("case", [
+    (1, 5, 9, 8, 2, 48, 1, 0), (2, 4, 7, 10, 8, 16, 0, 3), (1, 6, 5, 9, 24, 40, 0, 4), (1, 3, 8, 8, 34, 64, 1, 1),
+])
+def test_conv_even_channels_at_any_address(nn, case, offset):
+    """Even channel counts that are no multiple of 16 from a 16-byte boundary, an odd address and a 4-byte one."""
+    _check_conv(nn, case, offset)
