@@ -481,9 +481,9 @@ int wgrad_tc(const void* x, const void* dy, int n, int d, int h, int w, int cin,
 //   tensor off by one value: gathered value by value either way (1 -> 16 channels on
 //   4 x 32^3 voxels 21 and 47, 7 -> 9 84 and 171; from odd addresses 24 -> 32 285 and
 //   559, 104 -> 128 2051 and 3273);
-// - other voxels that allow no 8-channel loads, where both channels are few (6 -> 4 on
-//   16^3 23 and 27, 10 -> 32 36 and 41, 20 -> 4 61 and 66; but 26 -> 16 89 and 80, 10 ->
-//   64 52 and 46);
+// - other voxels that allow no 8-channel loads, where both channels are few or the
+//   outputs are up to 8 (6 -> 4 on 16^3 23 and 27, 10 -> 32 36 and 41, 20 -> 4 61 and 66;
+//   but 26 -> 16 89 and 80, 10 -> 64 52 and 46);
 // - boxes so thin along x or y that most of the 8 x 16 columns of the halo kernels is
 //   padding, once that is what they spend their time on (2 -> 16 on 512 x 1 x 512 49
 //   and 76, on 512 x 512 x 1, half as empty, 56 and 50; 16 -> 16 on 256 x 1 x 256 23
@@ -495,7 +495,7 @@ static bool by_warps(const void* x, int n, int d, int h, int w, int cin, int cou
     const double voxels = (double)n * d * h * w;
     const double column = (double)n * ((h + 15) / 16) * ((w + 7) / 8) * 128;  // positions of one plane
     if ((cin == 2 || cin == 4) && at % (2 * cin) == 0) return column * d > 8 * voxels && column * d >= 1 << 18;
-    if (cin % 16) return at % 4 || ((cin % 8 || at % 16) && cin <= 24 && cout <= 32);
+    if (cin % 16) return at % 4 || ((cin % 8 || at % 16) && (cout <= 8 || (cin <= 24 && cout <= 32)));
     if (at % 16) return false;
     const double read = column * (d + 2 * ((d + 15) / 16));  // positions that the halo planes hold
     if (cin == 16 && cout <= 16) return read > 2.75 * voxels && read >= 1 << 17;

@@ -771,3 +771,10 @@ def test_conv_weight_gradient_rings(nn, case, offset):
 def test_conv_even_channels_at_any_address(nn, case, offset):
     """Even channel counts that are no multiple of 16 from a 16-byte boundary, an odd address and a 4-byte one."""
     _check_conv(nn, case, offset)
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2, 4])
+@pytest.mark.parametrize("cin,cout", [(2, 12), (4, 6), (12, 50), (24, 36), (32, 20), (16, 34), (48, 24)])
+def test_conv_output_widths(nn, cin, cout, offset):
+    """Outputs of 8, 4, 2 and 1 values at a time, by the channels and the address."""
+    _check_conv(nn, (1, 5, 18, 11, cin, cout, 1, 3), offset)
