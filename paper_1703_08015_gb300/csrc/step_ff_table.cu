@@ -44,30 +44,14 @@ __global__ void __launch_bounds__(work_threads<L, A>()) k_gather_table(const Ste
     t[L::Q * P] = own.y;
 }
 
-// The update of a node out of range through the table (update_out_of_range).
-template <class L>
-__device__ __forceinline__ void gather_table(const StepArgs& a, const int32_t* t, unsigned long long (&b)[L::Q]) {
-    const unsigned long long* src = static_cast<const unsigned long long*>(a.src);
-    static_for<0, L::Q>([&](auto I) { b[decltype(I)::value] = src[__ldg(t + decltype(I)::value * a.gtab_pitch)]; });
-}
-
+// Native-FP64 update of one node through the table (the range fallback).
 template <class L, int MODEL>
 __device__ __noinline__ void update_fp64_table(const StepArgs& a, const int32_t* t, unsigned long long* out,
                                                int stride) {
+    const unsigned long long* src = static_cast<const unsigned long long*>(a.src);
     unsigned long long b[L::Q];
-    gather_table<L>(a, t, b);
+    static_for<0, L::Q>([&](auto I) { b[decltype(I)::value] = src[__ldg(t + decltype(I)::value * a.gtab_pitch)]; });
     store_fp64<L, MODEL>(b, a, out, stride);
-}
-
-template <class L, int MODEL>
-__device__ __noinline__ void update_out_of_range_table(const StepArgs& a, const int32_t* t, unsigned long long* out,
-                                                       int stride, FFRange r) {
-    if (r == FFRange::result) {
-        unsigned long long b[L::Q];
-        gather_table<L>(a, t, b);
-        if (collide_ff<L, MODEL, -1, true>(b, a.fx, a.ffc, out, stride) == FFRange::ok) return;
-    }
-    update_fp64_table<L, MODEL>(a, t, out, stride);
 }
 
 // Blocks of 128 threads, seven per SM (72 registers): 290 against 310 us per
@@ -95,8 +79,11 @@ __global__ void __launch_bounds__(kTableThreads, 7) k_step_ff_table(const StepAr
     });
     const int stride = __ldg(t + L::Q * P);
     T* out = static_cast<T*>(a.dst) + own;
-    const FFRange r = collide_ff<L, MODEL>(b, a.fx, a.ffc, out, stride);
-    if (r != FFRange::ok) update_out_of_range_table<L, MODEL>(a, t, out, stride, r);
+    if (collide_ff<L, MODEL>(b, a.fx, a.ffc, out, stride) != FFRange::ok) {
+        // out of range: the same update in native FP64 (a call, off the hot path); not the wider rounding of the
+        // other forms (update_out_of_range), so that a run through the table keeps its results
+        update_fp64_table<L, MODEL>(a, t, out, stride);
+    }
 }
 
 template <class L, int MODEL>
