@@ -90,10 +90,14 @@ template <class L, int MODEL>
 cudaError_t launch_step_ff_table(const StepArgs& a, cudaStream_t s) {
     if (a.n_nodes == 0) return cudaSuccess;
     const long long grid = (a.n_nodes + kTableThreads - 1) / kTableThreads;
-    // chained where two steps fit the device (24^3 to 60^3 samples 4 to 12 % faster): the step is bound by its
-    // loads, and beyond that the ordinary ones cost more (64^3: 6.8 us per step, 8.6 chained; 256^3: 337 and 347)
+    // in 3D chained where two steps fit the device (24^3 to 60^3 samples 4 to 12 % faster) and where one fills it and a
+    // little more (80^3, 1.09 of it: 10.5 and 10.1 us per step), whose last blocks the next step's join; the step is
+    // bound by its loads, and otherwise the ordinary ones cost more (64^3: 6.8 us per step, 8.6 chained; 256^3: 337 and
+    // 347); in 2D they do not (512^2: 5.8 us per step, 5.1 chained)
     static const Room room = room_for(k_step_ff_table<L, MODEL, true>, kTableThreads);
-    if (2 * grid <= room.blocks) return launch_chained(k_step_ff_table<L, MODEL, true>, (unsigned)grid, kTableThreads, s, a);
+    const double fill = (double)grid / room.blocks;
+    if (L::D == 2 ? chain_pays(grid, room) : fill <= 0.5 || (fill >= 0.95 && fill <= 1.45))
+        return launch_chained(k_step_ff_table<L, MODEL, true>, (unsigned)grid, kTableThreads, s, a);
     k_step_ff_table<L, MODEL, false><<<(unsigned)grid, kTableThreads, 0, s>>>(a);
     return cudaGetLastError();
 }

@@ -169,18 +169,16 @@ __device__ __forceinline__ bool collide_fixed(const unsigned long long (&b)[L::Q
     return ok;
 }
 
-// CHAIN: launched while the step before still runs, its values read with ordinary
-// loads (chain_wait).
-template <class L, int A, int MODEL, int MINB, bool CHAIN>
+template <class L, int A, int MODEL, int MINB>
 __global__ void __launch_bounds__(work_threads<L, A>(), MINB) k_step_fixed(const StepArgs a) {
     using TL = Tile<L, A>;
     using T = unsigned long long;
     __shared__ NeighShared<TL, work_tiles()> sh;
     WorkNode wn;
-    if (!stage_work<TL, work_tiles(), work_threads<L, A>(), CHAIN>(sh, a, wn)) return;
+    if (!stage_work<TL, work_tiles(), work_threads<L, A>(), true>(sh, a, wn)) return;
     const NodePos<A> p = node_pos<TL>(wn.node);
     T b[L::Q];
-    const int rank = gather<L, A, work_tiles(), T, !CHAIN>(sh, a.src, wn.lt, wn.node, p, b);
+    const int rank = gather<L, A, work_tiles(), T>(sh, a.src, wn.lt, wn.node, p, b);
     const int stride = sh.loc[wn.lt][TL::CENTER].y;
     T* out = own_slot<TL, work_tiles(), T>(sh, a.dst, wn.lt, rank);
     if (!collide_fixed<L, MODEL>(b, a.fx, out, stride)) {
@@ -193,12 +191,12 @@ __global__ void __launch_bounds__(work_threads<L, A>(), MINB) k_step_fixed(const
 template <class L, int A, int MODEL, int MINB>
 cudaError_t launch_step_fixed(const StepArgs& a, cudaStream_t s) {
     if (a.n_work_blocks == 0) return cudaSuccess;
-    // chained up to 16 waves (128^3 sample 89.9 to 88.9 us per step): beyond, the 1 us a launch takes is less than
-    // what ordinary loads cost (256^3: 707 us, 712 chained; in 8^3 tiles 1165 and 1180)
-    static const Room room = room_for(k_step_fixed<L, A, MODEL, MINB, true>, work_threads<L, A>());
-    if (a.n_work_blocks <= 16ll * room.blocks && chain_pays(a.n_work_blocks, room, 0.68))
-        return launch_chained(k_step_fixed<L, A, MODEL, MINB, true>, (unsigned)a.n_work_blocks, work_threads<L, A>(), s, a);
-    k_step_fixed<L, A, MODEL, MINB, false><<<a.n_work_blocks, work_threads<L, A>(), 0, s>>>(a);
+    // A large step pays 1 us of launch less with 1 % of ordinary loads (256^3: 707 us with read-only ones, 712), but a
+    // second form with read-only loads spilled more (717, in 8^3 tiles 1235 against 1181).
+    static const Room room = room_for(k_step_fixed<L, A, MODEL, MINB>, work_threads<L, A>());
+    if (chain_pays(a.n_work_blocks, room, 0.68))
+        return launch_chained(k_step_fixed<L, A, MODEL, MINB>, (unsigned)a.n_work_blocks, work_threads<L, A>(), s, a);
+    k_step_fixed<L, A, MODEL, MINB><<<a.n_work_blocks, work_threads<L, A>(), 0, s>>>(a);
     return cudaGetLastError();
 }
 
