@@ -488,7 +488,9 @@ int wgrad_tc(const void* x, const void* dy, int n, int d, int h, int w, int cin,
 //   padding, once that is what they spend their time on (2 -> 16 on 512 x 1 x 512 49
 //   and 76, on 512 x 512 x 1, half as empty, 56 and 50; 16 -> 16 on 256 x 1 x 256 23
 //   and 77, 64 -> 64 154 and 256), and boxes of one plane of 16 channels, each plane
-//   with its two neighbours in z (16 -> 4 on 1 x 256 x 256 19 and 25).
+//   with its two neighbours in z (16 -> 4 on 1 x 256 x 256 19 and 25).  Of multiples of
+//   16 channels only boxes of up to 4 voxels along x or y, or one plane: any other
+//   keeps the halo kernel's sums.
 static bool by_warps(const void* x, int n, int d, int h, int w, int cin, int cout) {
     const uintptr_t at = reinterpret_cast<uintptr_t>(x);
     if (cin % 2) return true;
@@ -496,7 +498,7 @@ static bool by_warps(const void* x, int n, int d, int h, int w, int cin, int cou
     const double column = (double)n * ((h + 15) / 16) * ((w + 7) / 8) * 128;  // positions of one plane
     if ((cin == 2 || cin == 4) && at % (2 * cin) == 0) return column * d > 8 * voxels && column * d >= 1 << 18;
     if (cin % 16) return at % 4 || ((cin % 8 || at % 16) && (cout <= 8 || (cin <= 24 && cout <= 32)));
-    if (at % 16) return false;
+    if (at % 16 || (w > 4 && h > 4 && d > 1)) return false;
     const double read = column * (d + 2 * ((d + 15) / 16));  // positions that the halo planes hold
     if (cin == 16 && cout <= 16) return read > 2.75 * voxels && read >= 1 << 17;
     return read > (cin == 16 ? 8.5 : 16) * voxels && read >= 400e3;
